@@ -135,9 +135,9 @@ def work(case):
             "flops": case["layers"] * 4 * sh.num_q_heads * sh.head_dim * keys}
 
 
-def prepare(case, seed):
-    """A serving program's state before the call: the layers' KV pools with their cached rows, the new rows and queries
-    (N(0,1) in bf16, as normalised activations are), the page tables with randomly scattered pages, the context."""
+def _inputs(case, seed):
+    """The iteration's batch (page tables, lengths) and, per layer, the pool with its cached rows, the new rows and the
+    queries: N(0,1) in bf16, as normalised activations are, with randomly scattered pages."""
     rng = np.random.Generator(np.random.PCG64(seed))
     sh, chunks, lens = _shape(case), _chunks(case), rng.permutation(_contexts(case))
     need = sum(-(-int(x) // PAGE) for x in lens) + sum(-(-(p + c) // PAGE) for p, c in chunks)
@@ -155,17 +155,24 @@ def prepare(case, seed):
     def normal(*size):
         return torch.empty(*size, dtype=torch.bfloat16, device=dev).normal_(generator=gen)
 
-    state = {
-        "call": case["call"],
-        "ctx": B.Context(sh, num_pages, max(batch.chunk_len, 1), max(batch.num_decode, 1), need + 16, device=dev.index),
+    return need, batch, {
         "pools": [normal(num_pages * sh.page_elems) for _ in range(layers)],
         "q": [normal(rows, sh.num_q_heads, sh.head_dim) for _ in range(layers)],
         "k_new": [normal(rows, sh.num_kv_heads, sh.head_dim) for _ in range(layers)],
         "v_new": [normal(rows, sh.num_kv_heads, sh.head_dim) for _ in range(layers)],
-        "out": [torch.zeros(rows, sh.num_q_heads, sh.head_dim, dtype=torch.bfloat16, device=dev) for _ in range(layers)],
-        "lse": [torch.zeros(rows, sh.num_q_heads, dtype=torch.float32, device=dev) if case["lse"] else None
-                for _ in range(layers)],
     }
+
+
+def prepare(case, seed):
+    """A serving program's state before the call: the inputs, the output buffers, the batch on the device, the context."""
+    need, batch, state = _inputs(case, seed)
+    sh, dev = _shape(case), state["q"][0].device
+    rows, layers = batch.num_rows, case["layers"]
+    state["call"] = case["call"]
+    state["ctx"] = B.Context(sh, need + 64, max(batch.chunk_len, 1), max(batch.num_decode, 1), need + 16, device=dev.index)
+    state["out"] = [torch.zeros(rows, sh.num_q_heads, sh.head_dim, dtype=torch.bfloat16, device=dev) for _ in range(layers)]
+    state["lse"] = [torch.zeros(rows, sh.num_q_heads, dtype=torch.float32, device=dev) if case["lse"] else None
+                    for _ in range(layers)]
     if case["call"] == "host":
         for name in ("q", "k_new", "v_new", "out", "lse"):
             state[name] = [None if t is None else t.cpu().pin_memory() for t in state[name]]
@@ -194,3 +201,59 @@ def tolerance(case):
     fp64, on rows sampled from every listed case and six drawn ones, the outputs are off by 2.4e-3 at most in the 2-norm
     and by 0.013 in the largest element: about four times that is stated.  (The pools hold copies: exact.)"""
     return {"rel": 1e-2, "max": 0.06}
+
+
+def _attend(q, k, v, scale, causal_from):
+    """64-bit attention of q [rows, heads, d] over k / v [keys, kv heads, d]; row i sees keys [0, causal_from + i].
+    Returns (out [rows, heads, d], lse [rows, heads])."""
+    rows, hq, d = q.shape
+    keys, hkv, _ = k.shape
+    g = hq // hkv
+    out, lse = torch.empty(rows, hq, d, dtype=torch.float64, device=q.device), torch.empty(rows, hq, dtype=torch.float64, device=q.device)
+    step = max(1, int(2.5e8) // (keys * g))                                # rows at a time: about 2 GB of scores
+    at = torch.arange(keys, device=q.device)
+    for h in range(hkv):
+        kh, vh = k[:, h].double().t().contiguous(), v[:, h].double().contiguous()
+        for r0 in range(0, rows, step):
+            n = min(step, rows - r0)
+            s = (q[r0:r0 + n, h * g:(h + 1) * g].double().reshape(n * g, d) @ kh).mul_(scale).view(n, g, keys)
+            first = causal_from + r0 + 1                                   # earlier keys are seen by every one of these rows
+            seen = at[first:] <= causal_from + r0 + torch.arange(n, device=q.device)[:, None]
+            s[:, :, first:].masked_fill_(~seen[:, None, :], -math.inf)
+            m = s.amax(-1, keepdim=True)
+            s.sub_(m).exp_()
+            total = s.sum(-1, keepdim=True)
+            out[r0:r0 + n, h * g:(h + 1) * g] = (s.view(n * g, keys) @ vh).view(n, g, d) / total
+            lse[r0:r0 + n, h * g:(h + 1) * g] = (m + total.log()).squeeze(-1)
+    return out, lse
+
+
+def exact(case, seed):
+    """The same iteration as plain torch gives it in 64 bits: every request's rows are put into its pages, its keys and
+    values gathered, and ordinary softmax attention done.  (The pools hold copies and stay bf16.)"""
+    _, batch, given = _inputs(case, seed)
+    sh, chunks = _shape(case), _chunks(case)
+    spans, row, page = [], 0, 0                                            # (first row, rows, first position, pages)
+    for p, c in chunks:
+        n = -(-(p + c) // PAGE)
+        spans.append((row, c, p, batch.prefill_pages[page:page + n]))
+        row, page = row + c, page + n
+    for i, x in enumerate(batch.decode_kv_len):
+        pages = batch.decode_pages[batch.decode_page_indptr[i]:batch.decode_page_indptr[i + 1]]
+        spans.append((row + i, 1, int(x) - 1, pages))
+    result = {"out": [], "pools": given["pools"], "lse": []}
+    for pool, q, k_new, v_new in zip(given["pools"], given["q"], given["k_new"], given["v_new"]):
+        pages_of = pool.view(-1, 2, sh.num_kv_heads, PAGE, sh.head_dim)
+        out = torch.empty(q.shape, dtype=torch.float64, device=q.device)
+        lse = torch.empty(q.shape[:2], dtype=torch.float64, device=q.device)
+        for r, n, first, pages in spans:
+            ids = torch.from_numpy(np.ascontiguousarray(pages).astype(np.int64)).to(q.device)
+            pos = torch.arange(first, first + n, device=q.device)
+            pages_of[ids[pos // PAGE], 0, :, pos % PAGE] = k_new[r:r + n]
+            pages_of[ids[pos // PAGE], 1, :, pos % PAGE] = v_new[r:r + n]
+            kv = pages_of[ids].permute(1, 0, 3, 2, 4).reshape(2, -1, sh.num_kv_heads, sh.head_dim)[:, :first + n]
+            out[r:r + n], lse[r:r + n] = _attend(q[r:r + n], kv[0], kv[1], sh.head_dim ** -0.5, first)
+        result["out"].append(out)
+        if case["lse"]:
+            result["lse"].append(lse)
+    return result
