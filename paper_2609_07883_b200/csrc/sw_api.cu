@@ -368,6 +368,8 @@ sw_status run_mixed(sw_ctx* ctx, void* kv_pool, const sw_batch* batch, const voi
         p.k_new = static_cast<const __nv_bfloat16*>(k_new);
         p.v_new = static_cast<const __nv_bfloat16*>(v_new);
         p.pool = static_cast<__nv_bfloat16*>(kv_pool);
+        p.append_first = p.C > 0;
+        p.append_last = p.C == 0;
     }
     p.ctrl = reinterpret_cast<int32_t*>(ctx->ws + ctx->w.ctrl);
     p.tickets = reinterpret_cast<int32_t*>(ctx->ws + ctx->w.tickets);

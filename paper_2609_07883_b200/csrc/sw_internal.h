@@ -22,8 +22,11 @@ constexpr int kMaxChunks = 8;           // prefill chunks (of different prompts)
 constexpr int kMaxChunk = 65536;        // chunk tokens per iteration (256-row groups are planned in shared memory)
 
 // Control words at the start of the workspace.
-// kCtrAppend counts the CTAs of a fused launch that have finished writing their share of the new K/V rows.
-enum CtrlWord { kCtrWork = 0, kCtrDone = 1, kCtrStatus = 2, kCtrDetail = 3, kCtrPrefill = 4, kCtrAppend = 5, kCtrWords = 64 };
+// kCtrArrived counts the CTAs that have ended, modulo two grids; launches use the two counter sets at kCtrSets in turn.
+enum CtrlWord { kCtrArrived = 0, kCtrStatus = 2, kCtrDetail = 3, kCtrSets = 16, kCtrWords = 64 };
+// Words of a counter set: decode units handed out by the counter, chunk-prefill entries likewise, and (fused launches with
+// chunks) CTAs that have written their share of the new K/V rows.
+enum SetWord { kSetWork = 0, kSetPrefill = 1, kSetAppend = 2, kSetWords = 16 };
 
 // Device-detected problem locators written to kCtrDetail (high byte = site, low 24 bits = index).
 enum DetailSite { kSiteAppendPage = 1, kSiteAppendLen = 2, kSiteAttnLen = 3, kSiteAttnPage = 4, kSiteWait = 5,
@@ -58,6 +61,8 @@ struct MixedParams {
     const __nv_bfloat16* k_new;
     const __nv_bfloat16* v_new;
     __nv_bfloat16* pool;
+    bool append_first;   // launches with chunks: every CTA writes its share of the rows before anything else
+    bool append_last;    // decode-only launches: a request's new row is written by the units that reach its last page
     // scratch
     int32_t* ctrl;
     int32_t* tickets;   // [max_decode * Hkv]: order in which the units of a (request, kv head) near their end

@@ -117,17 +117,18 @@ cudaError_t launch_kv_append(const AppendParams& p, int num_sms, cudaStream_t st
     return cudaLaunchKernelEx(&cfg, sw_kv_append_kernel, p);
 }
 
-// Fused launches (append and attention in one kernel): every CTA writes its share of the new K/V rows at the start of
-// the kernel and then adds one to a counter.  A page that can hold one of those rows (the last page of a decode
-// request; the chunk's own keys) is not fetched before the counter shows every CTA's share.  The grid is one CTA per
-// SM, so all CTAs are resident and the wait is short; it is bounded all the same.  Whole-warp call; false when the
-// wait ran out.
-__device__ __forceinline__ bool wait_append(const MixedParams& p) {
-    if (p.pool == nullptr) return true;
+// Fused launches with chunks (append and attention in one kernel): every CTA writes its share of the new K/V rows at the
+// start of the kernel and then adds one to a counter.  A page that can hold one of those rows (the last page of a decode
+// request; the chunk's own keys) is not fetched before the counter shows every CTA's share.  The grid is one CTA per SM,
+// so all CTAs are resident and the wait is short; it is bounded all the same.  Whole-warp call; false when the wait ran
+// out.  (Fused decode-only launches need no counter, see load_new_row.)
+__device__ __forceinline__ bool wait_append(const MixedParams& p, uint32_t set_addr) {
+    if (!p.append_first) return true;
     int ok = 1;
     if ((threadIdx.x & 31) == 0) {
+        const int32_t* counters = p.ctrl + lds_s32(set_addr);
         const long long t0 = clock64();
-        while (ld_acquire_gpu(&p.ctrl[kCtrAppend]) < (int)gridDim.x) {
+        while (ld_acquire_gpu(&counters[kSetAppend]) < (int)gridDim.x) {
             if (clock64() - t0 > kWaitBudgetCycles) {
                 ok = 0;
                 break;
@@ -143,20 +144,22 @@ __device__ __forceinline__ bool wait_append(const MixedParams& p) {
 // ---------------------------------------------------------------------------------------------------------------
 // mixed attention: shared-memory plan
 // ---------------------------------------------------------------------------------------------------------------
-constexpr int kStages = 2;  // K/V page buffers in flight per warp
-
 template <int D>
 struct Geo {
     static constexpr int kHalves = D / 64;                    // 128-byte swizzled column blocks per row
     static constexpr int kBlockBytes = kPageSize * 128;       // one [16 tokens][64 elems] swizzled block
     static constexpr int kStageBytes = 2 * kHalves * kBlockBytes;  // K then V of one (page, kv head)
+    static constexpr int kStages = 256 / D;                   // page buffers in flight per warp: 16 KB whatever the head size
     static constexpr int kRingBytes = kWarps * kStages * kStageBytes;
     static constexpr int kBarOffset = kRingBytes;                              // kWarps*kStages mbarriers
     static constexpr int kPfBarOffset = kBarOffset + kWarps * kStages * 8;     // barriers of the prefill tiles
+    static constexpr int kLastBarOffset = kPfBarOffset + 31 * 8;               // barrier: the list of last pages is there
     static constexpr int kPlanOffset = kPfBarOffset + 32 * 8;                  // int32 unit_prefix[kMaxDecode+1]
     static constexpr int kLenOffset = kPlanOffset + (kMaxDecode + 1) * 4 + 12;  // int32 kv_len[kMaxDecode]
     static constexpr int kIndptrOffset = kLenOffset + kMaxDecode * 4;           // int32 page_indptr[kMaxDecode+1]
-    static constexpr int kMiscOffset = kIndptrOffset + (kMaxDecode + 1) * 4 + 12; // scan scratch, TMEM base, abort flag
+    static constexpr int kLastOffset = kIndptrOffset + (kMaxDecode + 1) * 4 + 12; // int32 id of request i's last page
+    static constexpr int kMiscOffset = kLastOffset + kMaxDecode * 4;              // scan scratch, TMEM base, abort flag
+    static constexpr int kSetOffset = kMiscOffset + (32 + 7) * 4;                 // where this launch's counters start (words into ctrl)
     static constexpr int kSmemBytes = kMiscOffset + 768;   // 64 ints scan scratch and flags, the plan's counters, the chunk table
 };
 
@@ -357,7 +360,7 @@ template <int D>
 struct WarpRing {
     uint32_t buf;   // shared address of this warp's first stage
     uint32_t bar;   // shared address of this warp's first mbarrier
-    uint32_t it;    // pages consumed so far (stage = it % kStages, parity = (it / kStages) & 1)
+    uint32_t it;    // pages consumed so far (stage = it % stages, parity = (it / stages) & 1)
 };
 
 // Lane 0 arms the stage's barrier and fetches the page with one copy: the head's K blocks, then its V blocks.
@@ -365,7 +368,7 @@ template <int D>
 __device__ __forceinline__ void issue_page(const CUtensorMap* kvp_map, const WarpRing<D>& ring, uint32_t issue_it, int page,
                                            int kvh) {
     if ((threadIdx.x & 31) == 0) {
-        const uint32_t stage = issue_it % kStages;
+        const uint32_t stage = issue_it % Geo<D>::kStages;
         const uint32_t bar = ring.bar + stage * 8;
         mbar_arrive_expect_tx(bar, Geo<D>::kStageBytes);
         // a decode page is read once: evict-first keeps it from pushing the chunk's K/V tiles out of L2
@@ -373,11 +376,11 @@ __device__ __forceinline__ void issue_page(const CUtensorMap* kvp_map, const War
     }
 }
 
-// Merge of the splits of one (request, kv head) by the last unit to arrive, all rows together so that the loads of
-// one pass are in flight at once.  G >= group size is a compile-time bound: rows beyond the group read row 0 with
+// Merge of the splits of one (request, kv head), rows [row0, row0 + nrows) of the group (all of them, or one row when several
+// units share the merge).  J splits at a time: lane j fetches (m, l) of split j while all lanes fetch their four (two) columns
+// of the J partial outputs, so a merge of up to J splits costs one round trip to L2; it is the round trips (about a
+// microsecond each) that a merge consists of.  G >= nrows is a compile-time bound: rows beyond the group read row 0 with
 // weight zero, which keeps the loops free of branches.  Slots of the splits are Hkv apart.
-// The warp merges rows [row0, row0 + nrows) of the group (all of them, or one row when several units share the merge);
-// J = splits whose partial outputs are loaded together.
 template <int D, int G, int J = (G >= 8 ? 2 : (G == 4 ? 4 : 8))>
 __device__ __forceinline__ void merge_splits(const MixedParams& p, const Unit& u, int row0, int nrows) {
     constexpr int V = D / 32;                 // output columns per lane
@@ -385,96 +388,66 @@ __device__ __forceinline__ void merge_splits(const MixedParams& p, const Unit& u
     const int g = p.group;
     const int slot0 = u.slot - u.split * p.Hkv;
     const int ns = u.nsplit;
-    const float* ml0 = p.part_ml + (int64_t)slot0 * (2 * kMaxGroup);  // split s: + s * ml_stride
+    const float* ml0 = p.part_ml + (int64_t)slot0 * (2 * kMaxGroup) + row0;  // split s: + s * ml_stride
     const int64_t ml_stride = (int64_t)p.Hkv * (2 * kMaxGroup);
-    // pass 1: lanes take splits; per row the running maximum and the row sum rescaled to it, then one warp reduction
-    float m_all[G], l_all[G], m_first[G];
+    const float* po0 = p.part_o + ((int64_t)slot0 * g + row0) * D + lane * V;  // split s, row r: + s * po_stride + r * D
+    const int64_t po_stride = (int64_t)p.Hkv * g * D;
+    float m_all[G], l_all[G], acc[G][V];
 #pragma unroll
     for (int r = 0; r < G; ++r) {
         m_all[r] = -INFINITY;
         l_all[r] = 0.f;
-        m_first[r] = -INFINITY;
-    }
-    for (int s0 = 0; s0 < ns; s0 += 32) {
-        const int sidx = min(s0 + lane, ns - 1);
-        const bool live = s0 + lane < ns;
-        float ms[G], ls[G];
-#pragma unroll
-        for (int r = 0; r < G; ++r) {
-            const int rr = row0 + (r < nrows ? r : 0);
-            ms[r] = __ldcg(ml0 + sidx * ml_stride + rr);
-            ls[r] = __ldcg(ml0 + sidx * ml_stride + kMaxGroup + rr);
-        }
-#pragma unroll
-        for (int r = 0; r < G; ++r) {
-            if (!live) ms[r] = -INFINITY;
-            if (s0 == 0) m_first[r] = ms[r];
-            const float m_new = fmaxf(m_all[r], ms[r]);
-            const float a = m_all[r] == -INFINITY ? 0.f : fast_exp2((m_all[r] - m_new) * p.sm_scale_log2);
-            const float b = ms[r] == -INFINITY ? 0.f : fast_exp2((ms[r] - m_new) * p.sm_scale_log2);
-            l_all[r] = l_all[r] * a + ls[r] * b;
-            m_all[r] = m_new;
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < G; ++r) {
-        float mw = m_all[r];
-#pragma unroll
-        for (int o2 = 16; o2 > 0; o2 >>= 1) mw = fmaxf(mw, __shfl_xor_sync(0xffffffffu, mw, o2));
-        float lw = m_all[r] == -INFINITY ? 0.f : l_all[r] * fast_exp2((m_all[r] - mw) * p.sm_scale_log2);
-#pragma unroll
-        for (int o2 = 16; o2 > 0; o2 >>= 1) lw += __shfl_xor_sync(0xffffffffu, lw, o2);
-        m_all[r] = mw;
-        l_all[r] = lw;
-    }
-    // pass 2: weighted sum of the partial outputs; lanes take V adjacent columns of every row, J splits per batch
-    float acc[G][V];
-#pragma unroll
-    for (int r = 0; r < G; ++r)
 #pragma unroll
         for (int v = 0; v < V; ++v) acc[r][v] = 0.f;
-    const float* po0 = p.part_o + (int64_t)slot0 * g * D + lane * V;  // split s, row r: + s * po_stride + r * D
-    const int64_t po_stride = (int64_t)p.Hkv * g * D;
-    for (int s0 = 0; s0 < ns; s0 += 32) {
+    }
+#pragma unroll 1
+    for (int s0 = 0; s0 < ns; s0 += J) {
+        float x[J][G][V];
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const float* src = po0 + min(s0 + j, ns - 1) * po_stride;
+#pragma unroll
+            for (int r = 0; r < G; ++r) {
+                const float* row = src + (r < nrows ? r : 0) * D;
+                if constexpr (V == 4) {
+                    const float4 t = __ldcg(reinterpret_cast<const float4*>(row));
+                    x[j][r][0] = t.x, x[j][r][1] = t.y, x[j][r][2] = t.z, x[j][r][3] = t.w;
+                } else {
+                    const float2 t = __ldcg(reinterpret_cast<const float2*>(row));
+                    x[j][r][0] = t.x, x[j][r][1] = t.y;
+                }
+            }
+        }
+        const bool live = lane < J && s0 + lane < ns;
+        const float* ml = ml0 + min(s0 + (lane < J ? lane : 0), ns - 1) * ml_stride;
         float w[G];
 #pragma unroll
         for (int r = 0; r < G; ++r) {
-            float ms = m_first[r];
-            if (s0 > 0) {
-                ms = __ldcg(ml0 + min(s0 + lane, ns - 1) * ml_stride + row0 + (r < nrows ? r : 0));
-                if (s0 + lane >= ns) ms = -INFINITY;
-            }
-            w[r] = (ms == -INFINITY || r >= nrows) ? 0.f : fast_exp2((ms - m_all[r]) * p.sm_scale_log2);
+            float ms = __ldcg(ml + (r < nrows ? r : 0));
+            const float ls = __ldcg(ml + kMaxGroup + (r < nrows ? r : 0));
+            if (!live) ms = -INFINITY;
+            float mw = fmaxf(ms, m_all[r]);
+#pragma unroll
+            for (int o2 = 16; o2 > 0; o2 >>= 1) mw = fmaxf(mw, __shfl_xor_sync(0xffffffffu, mw, o2));
+            w[r] = ms == -INFINITY ? 0.f : fast_exp2((ms - mw) * p.sm_scale_log2);
+            float lw = w[r] * ls;
+            if (!live) lw = 0.f;
+#pragma unroll
+            for (int o2 = 16; o2 > 0; o2 >>= 1) lw += __shfl_xor_sync(0xffffffffu, lw, o2);
+            const float a = m_all[r] == -INFINITY ? 0.f : fast_exp2((m_all[r] - mw) * p.sm_scale_log2);
+            l_all[r] = l_all[r] * a + lw;
+            m_all[r] = mw;
+#pragma unroll
+            for (int v = 0; v < V; ++v) acc[r][v] *= a;
         }
-        const int cnt = min(32, ns - s0);
-        for (int j0 = 0; j0 < cnt; j0 += J) {
-            float x[J][G][V];
 #pragma unroll
-            for (int j = 0; j < J; ++j) {
-                const float* src = po0 + (s0 + min(j0 + j, cnt - 1)) * po_stride;
+        for (int j = 0; j < J; ++j)
 #pragma unroll
-                for (int r = 0; r < G; ++r) {
-                    const float* row = src + (row0 + (r < nrows ? r : 0)) * D;
-                    if constexpr (V == 4) {
-                        const float4 t = __ldcg(reinterpret_cast<const float4*>(row));
-                        x[j][r][0] = t.x, x[j][r][1] = t.y, x[j][r][2] = t.z, x[j][r][3] = t.w;
-                    } else {
-                        const float2 t = __ldcg(reinterpret_cast<const float2*>(row));
-                        x[j][r][0] = t.x, x[j][r][1] = t.y;
-                    }
-                }
+            for (int r = 0; r < G; ++r) {
+                const float wj = __shfl_sync(0xffffffffu, w[r], j);   // zero past the last split
+#pragma unroll
+                for (int v = 0; v < V; ++v) acc[r][v] = fmaf(wj, x[j][r][v], acc[r][v]);
             }
-#pragma unroll
-            for (int j = 0; j < J; ++j) {
-#pragma unroll
-                for (int r = 0; r < G; ++r) {
-                    float wj = __shfl_sync(0xffffffffu, w[r], (j0 + j) & 31);
-                    if (j0 + j >= cnt) wj = 0.f;
-#pragma unroll
-                    for (int v = 0; v < V; ++v) acc[r][v] = fmaf(wj, x[j][r][v], acc[r][v]);
-                }
-            }
-        }
     }
 #pragma unroll
     for (int r = 0; r < G; ++r) {
@@ -493,58 +466,95 @@ __device__ __forceinline__ void merge_splits(const MixedParams& p, const Unit& u
     }
 }
 
-// Which row of the group a unit of a request with many units merges (-1: none).  Not inlined: the rare case should
-// not cost the common one registers or instructions.
-__device__ __noinline__ int wide_merge_row(int nsplit, int split, int kvh, int g, int Hkv) {
-    const int d = nsplit - 1 - split;
-    if (nsplit >= 2 * g * Hkv) {
-        const int q = d >> 1;
-        return (!(d & 1) && q % Hkv == kvh && q / Hkv < g) ? q / Hkv : -1;
+// The new row of a (request, KV head) pair as 16-byte pieces: lanes 0 .. D/8-1 hold K, the next D/8 hold V.
+//
+// Fused decode-only launches: the new row of a request is written into its last page by the units that reach that page (one
+// per KV head), and, since the page's copy may have been made before, into the copy as well.  Requests that share their last
+// page (drafts of one sequence, say) find each other's new rows through the list of last pages.  Nobody waits for anybody.
+// (Appending first and counting the shares, as launches with chunks do, puts 3.5 us before the first page copy and makes the
+// units that reach a last page wait up to 6 us for the counter.  Measured with the units spread over the SMs and the shared
+// merge of small batches: one 8192-token context 23.5 -> 18.4 us per launch, 16 contexts of 256-2048 tokens 25.3 -> 22.4 us.)
+template <int D>
+__device__ __forceinline__ uint4 load_new_row(const MixedParams& p, int i, int kvh) {
+    const int lane = threadIdx.x & 31;
+    if (lane >= D / 4) return make_uint4(0u, 0u, 0u, 0u);
+    const __nv_bfloat16* src = lane < D / 8 ? p.k_new : p.v_new;
+    return *reinterpret_cast<const uint4*>(src + ((int64_t)i * p.Hkv + kvh) * D + (lane % (D / 8)) * 8);
+}
+template <int D>
+__device__ __forceinline__ void patch_row(uint32_t buf, int slot, uint4 v) {
+    const int lane = threadIdx.x & 31, chunk = lane % (D / 8);
+    if (lane < D / 4)
+        sts_v4(buf + (lane / (D / 8)) * (Geo<D>::kHalves * Geo<D>::kBlockBytes) + (chunk >> 3) * Geo<D>::kBlockBytes + slot * 128 +
+                   (((chunk & 7) ^ (slot & 7)) << 4), v.x, v.y, v.z, v.w);
+}
+// All new rows of the page in buffer `buf`, the last one of request i.  `lists`: shared address of the plan region.
+template <int D>
+__device__ __forceinline__ void patch_page(const MixedParams& p, uint32_t smem, uint32_t buf, int i, int kvh, int valid, uint4 own) {
+    const int lane = threadIdx.x & 31;
+    const int page = lds_s32(smem + Geo<D>::kLastOffset + i * 4);
+#pragma unroll 1
+    for (int j0 = 0; j0 < p.n; j0 += 32) {
+        const int j = j0 + lane;
+        bool hit = false;
+        if (j < p.n && j != i && lds_s32(smem + Geo<D>::kLastOffset + j * 4) == page)
+            hit = (lds_s32(smem + Geo<D>::kLenOffset + j * 4) - 1) % kPageSize + 1 < valid;
+        unsigned found = __ballot_sync(0xffffffffu, hit);
+        while (found) {
+            const int other = j0 + __ffs(found) - 1;
+            found &= found - 1;
+            patch_row<D>(buf, (lds_s32(smem + Geo<D>::kLenOffset + other * 4) - 1) % kPageSize, load_new_row<D>(p, other, kvh));
+        }
     }
-    return d < g ? d : -1;
+    patch_row<D>(buf, valid - 1, own);
+    if (page >= 0 && lane < D / 4) {
+        const int64_t block = ((int64_t)page * 2 + lane / (D / 8)) * p.Hkv + kvh;
+        *reinterpret_cast<uint4*>(p.pool + (block * kPageSize + valid - 1) * D + (lane % (D / 8)) * 8) = own;
+    }
+    __syncwarp();
 }
 
 // Runs one unit; returns false if a bounded wait expired.
+//
+// The products are transposed: the 16 rows of an mma.m16n8k16 are keys (of S = K Q^T) or output columns (of O^T = V^T P^T) and
+// its 8 columns are the query heads of the group (columns past the group are zero queries), half the instructions of the form
+// with the heads as rows, which would be padded to 16.
 template <int D>
-__device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const Unit& u, WarpRing<D>& ring, int fixed_items, bool pulls,
-                         int& next_item) {
-    constexpr int KS = D / 16;  // k-slices of QK^T; also pairs of 8-wide output column tiles of PV
+__device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const Unit& u, WarpRing<D>& ring, uint32_t smem,
+                         int32_t* work, int fixed_items, bool pulls, bool resident, int& next_item) {
+    constexpr int KS = D / 16;  // k-slices of K Q^T; also 16-column tiles of O
+    constexpr int kStages = Geo<D>::kStages;
     const int lane = threadIdx.x & 31;
-    const int qrow_in_group = lane >> 2;  // accumulator row held in c0/c1
     const int g = p.group;
+    const bool patch = p.append_last;   // the new rows are written here; with chunks they were written before
 
-    // A fragments of Q: rows 0..g-1 are the query heads sharing this KV head, rows >= g are zero
-    uint32_t qa[KS][2];
+    // B fragments of Q^T: the lane holds head lane / 4, elements 2 (lane % 4) + {0, 1} (+ 8) of every 16
+    uint32_t qb[KS][2];
     {
-        const __nv_bfloat16* qbase = p.q + ((int64_t)u.q_row * p.Hq + (int64_t)u.kvh * g) * D;
+        const uint32_t* src = reinterpret_cast<const uint32_t*>(p.q + ((int64_t)u.q_row * p.Hq + u.kvh * g + (lane >> 2)) * D + (lane & 3) * 2);
+        const bool live = (lane >> 2) < g;
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks) {
-            uint32_t v0 = 0, v1 = 0;
-            if (qrow_in_group < g) {
-                const uint32_t* src = reinterpret_cast<const uint32_t*>(qbase + qrow_in_group * D + ks * 16 + (lane & 3) * 2);
-                v0 = src[0];
-                v1 = src[4];  // +8 elements
-            }
-            qa[ks][0] = v0;
-            qa[ks][1] = v1;
+            qb[ks][0] = live ? src[ks * 8] : 0u;
+            qb[ks][1] = live ? src[ks * 8 + 4] : 0u;
         }
     }
 
-    float o[2 * KS][2];
+    float o[KS][4];   // O^T: columns 16 t + lane / 4 (+ 8) of heads 2 (lane % 4) + {0, 1}
 #pragma unroll
-    for (int i = 0; i < 2 * KS; ++i) o[i][0] = o[i][1] = 0.f;
-    float m_run = -INFINITY, l_run = 0.f;
+    for (int i = 0; i < KS; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
+    float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;   // of those two heads; l over the lane's own keys
 
     const int pg0 = u.t_begin / kPageSize;
     const int pg1 = (u.t_end + kPageSize - 1) / kPageSize;
     const int npg = pg1 - pg0;
 
-    // per-lane shared-memory offsets of the ldmatrix rows (128-byte swizzle: 16-byte chunk ^= row % 8)
-    const int k_tok = ((lane >> 4) << 3) + (lane & 7);
-    const int k_sel = (lane >> 3) & 1;
-    const int v_tok = (((lane >> 3) & 1) << 3) + (lane & 7);
-    const int v_sel = lane >> 4;
-    const int swz = lane & 7;
+    // Per-lane offsets of the ldmatrix rows: the four 8x8 matrices are keys 0-7 / 8-15 of one 8-element block, then of the next
+    // (K), or the two blocks of keys 0-7, then of keys 8-15 (V, transposed).  In the 128-byte swizzle 16-byte chunk c of row r
+    // lies at c ^ (r % 8), so a step of two chunks flips address bits 5 and 6.
+    const uint32_t k_lane = (lane & 15) * 128 + (((lane >> 4) ^ (lane & 7)) << 4);
+    const uint32_t v_lane = Geo<D>::kHalves * Geo<D>::kBlockBytes + ((lane & 7) + ((lane >> 4) << 3)) * 128 +
+                            ((((lane >> 3) & 1) ^ (lane & 7)) << 4);
 
     int ids = 0;
     int issued = 0;
@@ -563,7 +573,7 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
             page = 0;
         }
         // the request's last page holds the row this iteration appends
-        if (p.pool != nullptr && (pg0 + issued + 1) * kPageSize >= u.len && !wait_append(p)) {
+        if (p.append_first && (pg0 + issued + 1) * kPageSize >= u.len && !wait_append(p, smem + Geo<D>::kSetOffset)) {
             if (lane == 0) report(p.ctrl, SW_ERR_DEVICE_TIMEOUT, kSiteWait, u.q_row);
             append_timeout = true;
         }
@@ -575,139 +585,163 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
     // round trip hides behind the last pages, and no warp hoards a unit while others are still idle.
     // With the claim the unit draws its ticket among the units of its (request, kv head): the last ticket makes it
     // the one that merges.  Both answers are read at the end of the unit, when they have long arrived.
-    // A request cut into many units (kWideMergeSplits or more) has g mergers per kv head, fixed in advance among its
-    // last units, one query-head row each.  Such a unit will wait for the request's other units, so it must not hold
-    // a claimed unit meanwhile (another merger could be waiting for that one): it claims its next unit after the merge.
-    // With enough units the mergers of the different heads and rows are every other unit from the end (row j of head
-    // h: unit nsplit - 1 - 2 (j Hkv + h)), which puts them on different SMs; otherwise the last g units of each head.
-    const bool wide = g > 1 && u.nsplit >= kWideMergeSplits;
-    const int merge_row = wide ? wide_merge_row(u.nsplit, u.split, u.kvh, g, p.Hkv) : -1;
+    // A request cut into many units (kWideMergeSplits or more) has g mergers per kv head, fixed in advance: its last g
+    // units, one query-head row each (units of one request and head are Hkv apart in the order in which SMs take them, so
+    // the mergers sit on different SMs).  Such a unit will wait for the request's other units, so it must not hold a
+    // claimed unit meanwhile (another merger could be waiting for that one): it claims its next unit after the merge.
+    // Where every unit of the launch has a warp of its own (`resident`) nobody can wait for a unit that nobody runs, and the merge
+    // is shared as soon as there are g units.
+    const bool wide = g > 1 && u.nsplit >= (resident ? g : kWideMergeSplits);
+    const int merge_row = wide && u.nsplit - 1 - u.split < g ? u.nsplit - 1 - u.split : -1;
     bool claimed = merge_row >= 0;
     int ticket = 0;  // lane 0
     auto claim_next = [&]() {
         if (!claimed && issued >= npg) {
             claimed = true;
             if (lane == 0) {
-                next_item = pulls ? fixed_items + atomicAdd(&p.ctrl[kCtrWork], 1) : 0x7fffffff;
+                next_item = pulls ? fixed_items + atomicAdd(work, 1) : 0x7fffffff;
                 if (u.nsplit > 1 && !wide) ticket = atomicAdd(&p.tickets[u.ticket], 1);
             }
         }
     };
     claim_next();
 
+    uint32_t sK = 0;
     for (int k = 0; k < npg; ++k) {
         if (append_timeout) return false;
         const uint32_t stage = ring.it % kStages;
         const uint32_t parity = (ring.it / kStages) & 1;
-        const uint32_t sK = ring.buf + stage * Geo<D>::kStageBytes;
-        const uint32_t sV = sK + Geo<D>::kHalves * Geo<D>::kBlockBytes;
+        sK = ring.buf + stage * Geo<D>::kStageBytes;
+        const int valid = u.len - (pg0 + k) * kPageSize;   // keys of this page that are attended (16 or more: all)
+        const bool patched = patch && valid <= kPageSize;
+        uint4 row;
+        if (patched) row = load_new_row<D>(p, u.q_row, u.kvh);   // (no chunk rows: q_row is the request)
         if (!mbar_wait(ring.bar + stage * 8, parity)) {
             report(p.ctrl, SW_ERR_DEVICE_TIMEOUT, kSiteWait, u.q_row);
             return false;
         }
-        const int t0 = (pg0 + k) * kPageSize;
+        if (patched) {
+            if (!mbar_wait(smem + Geo<D>::kLastBarOffset, 0)) {
+                report(p.ctrl, SW_ERR_DEVICE_TIMEOUT, kSiteWait, u.q_row);
+                return false;
+            }
+            __syncwarp();
+            patch_page<D>(p, smem, sK, u.q_row, u.kvh, valid, row);
+        }
 
-        // S = Q K^T for 16 keys
-        float s[2][4];
-#pragma unroll
-        for (int i = 0; i < 2; ++i) s[i][0] = s[i][1] = s[i][2] = s[i][3] = 0.f;
+        // S^T = K Q^T for 16 keys, in two chains
+        float s[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f};
+        const uint32_t k_addr = sK + k_lane, v_addr = sK + v_lane;
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks) {
-            const int chunk = 2 * ks + k_sel;
-            const uint32_t addr = sK + (chunk >> 3) * Geo<D>::kBlockBytes + k_tok * 128 + (((chunk & 7) ^ swz) << 4);
-            uint32_t b0, b1, b2, b3;
-            ldmatrix_x4(addr, b0, b1, b2, b3);
-            mma_bf16_16816(s[0], qa[ks][0], 0u, qa[ks][1], 0u, b0, b1);
-            mma_bf16_16816(s[1], qa[ks][0], 0u, qa[ks][1], 0u, b2, b3);
+            uint32_t a0, a1, a2, a3;
+            ldmatrix_x4((k_addr ^ ((ks & 3) * 32)) + (ks >> 2) * Geo<D>::kBlockBytes, a0, a1, a2, a3);
+            mma_bf16_16816(ks & 1 ? s2 : s, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
         }
-        // mask keys outside [t_begin, t_end)
-        const int valid_hi = u.t_end - t0;   // keys with index >= valid_hi are masked
-        const int valid_lo = u.t_begin - t0; // keys with index <  valid_lo are masked (always <= 0 here)
-        float mx = -INFINITY;
+        // the lane's keys are lane / 4 and lane / 4 + 8; keys past the context are masked
+        const bool ok0 = (lane >> 2) < valid, ok1 = (lane >> 2) + 8 < valid;
+        s[0] = ok0 ? s[0] + s2[0] : -INFINITY;
+        s[1] = ok0 ? s[1] + s2[1] : -INFINITY;
+        s[2] = ok1 ? s[2] + s2[2] : -INFINITY;
+        s[3] = ok1 ? s[3] + s2[3] : -INFINITY;
+        float mx0 = fmaxf(s[0], s[2]), mx1 = fmaxf(s[1], s[3]);
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const int key = nt * 8 + (lane & 3) * 2 + j;
-                const float v = (key < valid_hi && key >= valid_lo) ? s[nt][j] : -INFINITY;
-                s[nt][j] = v;
-                mx = fmaxf(mx, v);
-            }
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-        const float m_new = fmaxf(m_run, mx);
-        const float corr = fast_exp2((m_run - m_new) * p.sm_scale_log2);
-        const float mb = m_new * p.sm_scale_log2;
-        float pr[2][2];
-        float psum = 0.f;
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                pr[nt][j] = fast_exp2(fmaf(s[nt][j], p.sm_scale_log2, -mb));
-                psum += pr[nt][j];
-            }
-        l_run = l_run * corr + psum;
-        m_run = m_new;
-#pragma unroll
-        for (int i = 0; i < 2 * KS; ++i) {
-            o[i][0] *= corr;
-            o[i][1] *= corr;
+        for (int w = 4; w < 32; w <<= 1) {
+            mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, w));
+            mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, w));
         }
-        const uint32_t pa0 = pack_bf16x2(pr[0][0], pr[0][1]);
-        const uint32_t pa2 = pack_bf16x2(pr[1][0], pr[1][1]);
+        mx0 = fmaxf(m0, mx0);
+        mx1 = fmaxf(m1, mx1);
+        const float c0 = fast_exp2((m0 - mx0) * p.sm_scale_log2), c1 = fast_exp2((m1 - mx1) * p.sm_scale_log2);
+        m0 = mx0;
+        m1 = mx1;
+        const float b0 = mx0 * p.sm_scale_log2, b1 = mx1 * p.sm_scale_log2;
+        s[0] = fast_exp2(fmaf(s[0], p.sm_scale_log2, -b0));
+        s[1] = fast_exp2(fmaf(s[1], p.sm_scale_log2, -b1));
+        s[2] = fast_exp2(fmaf(s[2], p.sm_scale_log2, -b0));
+        s[3] = fast_exp2(fmaf(s[3], p.sm_scale_log2, -b1));
+        l0 = l0 * c0 + (s[0] + s[2]);
+        l1 = l1 * c1 + (s[1] + s[3]);
+#pragma unroll
+        for (int i = 0; i < KS; ++i) {
+            o[i][0] *= c0;
+            o[i][1] *= c1;
+            o[i][2] *= c0;
+            o[i][3] *= c1;
+        }
+        // P^T [keys][heads] as the B operand: keys along the fragment's registers, so the 8x8 blocks are transposed
+        const uint32_t p0 = movmatrix_trans(pack_bf16x2(s[0], s[1])), p1 = movmatrix_trans(pack_bf16x2(s[2], s[3]));
 
         // the unwritten slots of a partly filled last page hold whatever the pool held: zero those V rows so that
         // 0 * garbage cannot produce NaN
-        if (valid_hi < kPageSize) {
+        if (valid < kPageSize) {
             __syncwarp();
-            const int dead_rows = kPageSize - valid_hi;
+            const int dead_rows = kPageSize - valid;
             for (int c = lane; c < dead_rows * (D / 8); c += 32) {
-                const int row = valid_hi + c / (D / 8);
+                const int row_i = valid + c / (D / 8);
                 const int chunk = c % (D / 8);
-                const uint32_t addr = sV + (chunk >> 3) * Geo<D>::kBlockBytes + row * 128 + (((chunk & 7) ^ (row & 7)) << 4);
-                asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(addr), "r"(0u) : "memory");
+                sts_v4(sK + (Geo<D>::kHalves + (chunk >> 3)) * Geo<D>::kBlockBytes + row_i * 128 + (((chunk & 7) ^ (row_i & 7)) << 4),
+                       0u, 0u, 0u, 0u);
             }
             __syncwarp();
         }
 
-        // O += P V
+        // O^T += V^T P^T
 #pragma unroll
         for (int dn = 0; dn < KS; ++dn) {
-            const int chunk = 2 * dn + v_sel;
-            const uint32_t addr = sV + (chunk >> 3) * Geo<D>::kBlockBytes + v_tok * 128 + (((chunk & 7) ^ swz) << 4);
-            uint32_t b0, b1, b2, b3;
-            ldmatrix_x4_trans(addr, b0, b1, b2, b3);
-            float acc0[4] = {o[2 * dn][0], o[2 * dn][1], 0.f, 0.f};
-            float acc1[4] = {o[2 * dn + 1][0], o[2 * dn + 1][1], 0.f, 0.f};
-            mma_bf16_16816(acc0, pa0, 0u, pa2, 0u, b0, b1);
-            mma_bf16_16816(acc1, pa0, 0u, pa2, 0u, b2, b3);
-            o[2 * dn][0] = acc0[0];
-            o[2 * dn][1] = acc0[1];
-            o[2 * dn + 1][0] = acc1[0];
-            o[2 * dn + 1][1] = acc1[1];
+            uint32_t a0, a1, a2, a3;
+            ldmatrix_x4_trans((v_addr ^ ((dn & 3) * 32)) + (dn >> 2) * Geo<D>::kBlockBytes, a0, a1, a2, a3);
+            mma_bf16_16816(o[dn], a0, a1, a2, a3, p0, p1);
         }
         ring.it += 1;
         __syncwarp();  // every lane is done reading this stage before it is refilled
-        if (valid_hi < kPageSize) fence_proxy_async_smem();
         if (issued < npg) issue_next();
         claim_next();
     }
 
-    // finish: row sums across the quad
-    l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
-    l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
-    const bool row_ok = qrow_in_group < g;
-    const int head = u.kvh * g + qrow_in_group;
-    if (u.nsplit == 1) {
-        if (row_ok) {
-            const float inv = 1.f / l_run;
-            __nv_bfloat16* dst = p.out + ((int64_t)u.q_row * p.Hq + head) * D + (lane & 3) * 2;
+    // Finish: the row sums over the keys of all lanes, then (m, l, O) through the unit's last page buffer, so that rows leave in
+    // whole lines: O[head][D] with the 32-byte groups of a row rotated by half the head (the lanes' four head pairs then fall
+    // on different banks).
 #pragma unroll
-            for (int i = 0; i < 2 * KS; ++i)
-                *reinterpret_cast<uint32_t*>(dst + i * 8) = pack_bf16x2(o[i][0] * inv, o[i][1] * inv);
-            if (p.lse && (lane & 3) == 0) p.lse[(int64_t)u.q_row * p.Hq + head] = m_run * p.sm_scale + __logf(l_run);
+    for (int w = 4; w < 32; w <<= 1) {
+        l0 += __shfl_xor_sync(0xffffffffu, l0, w);
+        l1 += __shfl_xor_sync(0xffffffffu, l1, w);
+    }
+    {
+        const int h = (lane & 3) * 2;
+        const uint32_t addr = sK + (h * D + (lane >> 2)) * 4;
+#pragma unroll
+        for (int t = 0; t < KS; ++t) {
+            const uint32_t a0 = addr + ((16 * t) ^ (h * 4)) * 4, a1 = addr + ((16 * t + 8) ^ (h * 4)) * 4;
+            if (h < g) {
+                sts_f32(a0, o[t][0]);
+                sts_f32(a1, o[t][2]);
+            }
+            if (h + 1 < g) {
+                sts_f32(a0 + D * 4, o[t][1]);
+                sts_f32(a1 + D * 4, o[t][3]);
+            }
         }
+    }
+    __syncwarp();
+    constexpr int kRowLanes = D / 4;   // lanes that hold a row, four columns each
+    const int col = (lane % kRowLanes) * 4;
+    if (u.nsplit == 1) {
+        for (int r0 = 0; r0 < g; r0 += 32 / kRowLanes) {
+            const int r = r0 + lane / kRowLanes;
+            const float ma = __shfl_sync(0xffffffffu, m0, r >> 1), mb = __shfl_sync(0xffffffffu, m1, r >> 1);
+            const float la = __shfl_sync(0xffffffffu, l0, r >> 1), lb = __shfl_sync(0xffffffffu, l1, r >> 1);
+            if (r < g) {
+                const float4 x = lds_f4(sK + (r * D + (col ^ ((r >> 1) * 8))) * 4);
+                const float inv = 1.f / (r & 1 ? lb : la);
+                const int head = u.kvh * g + r;
+                *reinterpret_cast<uint2*>(p.out + ((int64_t)u.q_row * p.Hq + head) * D + col) =
+                    make_uint2(pack_bf16x2(x.x * inv, x.y * inv), pack_bf16x2(x.z * inv, x.w * inv));
+                if (p.lse && col == 0) p.lse[(int64_t)u.q_row * p.Hq + head] = (r & 1 ? mb : ma) * p.sm_scale + __logf(r & 1 ? lb : la);
+            }
+        }
+        fence_proxy_async_smem();  // the buffer was written with plain stores and is refilled by the copy engine
+        __syncwarp();
         return true;
     }
 
@@ -715,15 +749,15 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
     // `ready` counter, without waiting for anything); the one that did waits until the others have and merges.  It is
     // usually the last to finish, so its wait is short, and no fence or ticket round trip sits between its last page
     // and the merge.
-    if (row_ok) {
-        float* po = p.part_o + ((int64_t)u.slot * g + qrow_in_group) * D + (lane & 3) * 2;
-#pragma unroll
-        for (int i = 0; i < 2 * KS; ++i) *reinterpret_cast<float2*>(po + i * 8) = make_float2(o[i][0], o[i][1]);
-        if ((lane & 3) == 0) {
-            p.part_ml[(int64_t)u.slot * (2 * kMaxGroup) + qrow_in_group] = m_run;
-            p.part_ml[(int64_t)u.slot * (2 * kMaxGroup) + kMaxGroup + qrow_in_group] = l_run;
-        }
+    for (int r = lane / kRowLanes; r < g; r += 32 / kRowLanes)
+        *reinterpret_cast<float4*>(p.part_o + ((int64_t)u.slot * g + r) * D + col) = lds_f4(sK + (r * D + (col ^ ((r >> 1) * 8))) * 4);
+    if (lane < 4) {
+        float* ml = p.part_ml + (int64_t)u.slot * (2 * kMaxGroup) + lane * 2;
+        if (lane * 2 < g) ml[0] = m0, ml[kMaxGroup] = l0;
+        if (lane * 2 + 1 < g) ml[1] = m1, ml[kMaxGroup + 1] = l1;
     }
+    fence_proxy_async_smem();  // the buffer was written with plain stores and is refilled by the copy engine
+    __syncwarp();
     if (wide) {
         // Many splits (one long context cut for all the warps): a single warp would load their partial outputs a few
         // at a time.  Every unit publishes its partial result; g of the request's last units then merge one row of
@@ -754,7 +788,7 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
         merge_splits<D, 1, 16>(p, u, merge_row, 1);
         if (lane == 0) {
             if (atomicAdd(&p.ready[u.ticket], 1) == u.nsplit + g - 1) p.ready[u.ticket] = 0;  // ready for the next launch
-            next_item = pulls ? fixed_items + atomicAdd(&p.ctrl[kCtrWork], 1) : 0x7fffffff;
+            next_item = pulls ? fixed_items + atomicAdd(work, 1) : 0x7fffffff;
         }
         return true;
     }
@@ -824,11 +858,15 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
     // the chunks' descriptors go to shared memory: the roles of the chunk-prefill phase look them up by the item's chunk
     // number instead of carrying them in registers
     if (kMulti && warp == 2) pf_fill_chunk_table(p, scratch + kChunkTable);
-    if (threadIdx.x == 0) {
-        tma_prefetch_desc(&kv_map);
+    if (threadIdx.x < kWarps * Geo<D>::kStages) {
+        mbar_init(base + Geo<D>::kBarOffset + threadIdx.x * 8, 1);
+        fence_mbar_init();
+    }
+    if (threadIdx.x == 96) {
         tma_prefetch_desc(&kvp_map);
-        for (int i = 0; i < kWarps * kStages; ++i) mbar_init(base + Geo<D>::kBarOffset + i * 8, 1);
+        mbar_init(base + Geo<D>::kLastBarOffset, kWarps);
         if (tensor_prefill) {
+            tma_prefetch_desc(&kv_map);
             tma_prefetch_desc(&q_map);
             tma_prefetch_desc(&out_map);
             pf_init_barriers(base + Geo<D>::kPfBarOffset);
@@ -841,13 +879,20 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
     // kernels of the stream wrote (the pool after the KV append, q, the page tables): wait for them to finish.
     grid_dependency_wait();
     grid_launch_dependents();
-    if (p.pool != nullptr) {
-        // fused launch: this CTA's share of the new K/V rows, then its mark on the counter the readers wait for
+    // Counters come in two sets that launches use in turn, so that no CTA has to wait at its end to find out whether it is
+    // the last one: every CTA counts itself once when it ends (modulo two grids), hence a launch that reads between 0 and
+    // grid - 1 uses set 0, one that reads more uses set 1, and it clears the other one for the launch after it.
+    const int set = ld_relaxed_gpu(&p.ctrl[kCtrArrived]) >= (int)gridDim.x ? 1 : 0;
+    int32_t* counters = p.ctrl + kCtrSets + set * kSetWords;
+    if (threadIdx.x == 0) misc[7] = kCtrSets + set * kSetWords;
+    if (blockIdx.x == 0 && threadIdx.x < kSetWords) p.ctrl[kCtrSets + (set ^ 1) * kSetWords + threadIdx.x] = 0;
+    if (p.append_first) {
+        // fused launch with chunks: this CTA's share of the new K/V rows, then its mark on the counter the readers wait for
         append_rows<kMulti>(p, D, (int64_t)blockIdx.x * kThreads + threadIdx.x, (int64_t)gridDim.x * kThreads);
         fence_proxy_async_global();
         __threadfence();
         __syncthreads();
-        if (threadIdx.x == 0) atomicAdd(&p.ctrl[kCtrAppend], 1);
+        if (threadIdx.x == 0) atomicAdd(&counters[kSetAppend], 1);
     }
     __syncthreads();
 
@@ -893,19 +938,41 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
     const Plan plan = make_plan(p, unit_prefix, reinterpret_cast<int*>(smem + Geo<D>::kLenOffset),
                                 reinterpret_cast<int*>(smem + Geo<D>::kIndptrOffset), scratch, late,
                                 p.stages_per_us);
+    if (p.append_last) {
+        // The requests' last pages, which fused decode-only launches write.  Only warps with a request wait for the load.
+        for (int i = threadIdx.x; i < p.n; i += kThreads) {
+            const int len = plan.len[i], pi = (len - 1) / kPageSize;
+            int id = -1;
+            if (len < 1 || pi >= p.decode_page_indptr[i + 1] - plan.indptr[i]) {
+                if (blockIdx.x == 0) report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAppendLen, i);
+            } else {
+                id = p.decode_pages[plan.indptr[i] + pi];
+                if (id < 0 || (int64_t)id >= p.num_pages) {
+                    if (blockIdx.x == 0) report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAppendPage, i);
+                    id = -1;
+                }
+            }
+            sts_s32(base + Geo<D>::kLastOffset + i * 4, id);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(base + Geo<D>::kLastBarOffset);
+    }
     if (plan.total_items > p.max_items) {
         if (threadIdx.x == 0) report(p.ctrl, SW_ERR_WORKSPACE, kSiteScratch, plan.total_items);
     } else {
+        int32_t* work = p.ctrl + lds_s32(base + Geo<D>::kSetOffset) + kSetWork;
         WarpRing<D> ring;
-        ring.buf = base + warp * kStages * Geo<D>::kStageBytes;
-        ring.bar = base + Geo<D>::kBarOffset + warp * kStages * 8;
+        ring.buf = base + warp * Geo<D>::kStages * Geo<D>::kStageBytes;
+        ring.bar = base + Geo<D>::kBarOffset + warp * Geo<D>::kStages * 8;
         ring.it = 0;
         const int fixed_items = ((int)gridDim.x - prefill_ctas) * kWarps;  // units handed out without the counter
         // with two unit sizes the early CTAs run their one large unit each and leave the counter to the late CTAs
         const bool pulls = !plan.two_sizes || (int)blockIdx.x < prefill_ctas;
-        int item = ((int)blockIdx.x - prefill_ctas) * kWarps + warp;
+        const bool resident = prefill_ctas == 0 && plan.total_items <= fixed_items;
+        // neighbouring units go to different SMs: a batch with fewer units than warps is spread over all of them
+        int item = warp * ((int)gridDim.x - prefill_ctas) + (int)blockIdx.x - prefill_ctas;
         if ((int)blockIdx.x < prefill_ctas) {
-            if (lane == 0) item = fixed_items + atomicAdd(&p.ctrl[kCtrWork], 1);
+            if (lane == 0) item = fixed_items + atomicAdd(work, 1);
             item = __shfl_sync(0xffffffffu, item, 0);
         }
         while (item < plan.total_items) {
@@ -940,28 +1007,17 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
             if (!ok) {
                 if (lane == 0) {
                     report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAttnLen, u.q_row);
-                    next_item = pulls ? fixed_items + atomicAdd(&p.ctrl[kCtrWork], 1) : 0x7fffffff;
+                    next_item = pulls ? fixed_items + atomicAdd(work, 1) : 0x7fffffff;
                 }
-            } else if (!run_unit<D>(&kvp_map, p, u, ring, fixed_items, pulls, next_item)) {
+            } else if (!run_unit<D>(&kvp_map, p, u, ring, base, work, fixed_items, pulls, resident, next_item)) {
                 break;
             }
             item = __shfl_sync(0xffffffffu, next_item, 0);
         }
     }
 
-    // the last CTA to finish re-arms the work counter for the next launch
     __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const int done = atomicAdd(&p.ctrl[kCtrDone], 1);
-        if (done == (int)gridDim.x - 1) {
-            p.ctrl[kCtrWork] = 0;
-            p.ctrl[kCtrPrefill] = 0;
-            p.ctrl[kCtrAppend] = 0;
-            p.ctrl[kCtrDone] = 0;
-            __threadfence();
-        }
-    }
+    if (threadIdx.x == 0) atomicInc(reinterpret_cast<unsigned*>(&p.ctrl[kCtrArrived]), 2 * gridDim.x - 1);
 }
 
 // Self-test of the bounded wait: one warp waits on a barrier that nothing will ever complete; the wait must give up

@@ -417,7 +417,7 @@ __device__ __forceinline__ bool pf_produce(const CUtensorMap* kv_map, const CUte
                                 h * 64, it.kvh * p.group, pf_chunk<D, kMulti>(p, sh, 2, it.chunk) + it.tok0[t]);
     }
     // fused launch: tiles that reach into the chunk's own keys wait until every CTA has written its share of them
-    if (p.pool != nullptr && it.j1 * 128 > pf_chunk<D, kMulti>(p, sh, 0, it.chunk) && !wait_append(p)) {
+    if (p.append_first && it.j1 * 128 > pf_chunk<D, kMulti>(p, sh, 0, it.chunk) && !wait_append(p, sh.smem + Geo<D>::kSetOffset)) {
         if (lane == 0) {
             *sh.abort_flag = 1;
             report(p.ctrl, SW_ERR_DEVICE_TIMEOUT, kSiteWait, it.item);
@@ -923,7 +923,7 @@ __device__ __forceinline__ void prefill_phase(const CUtensorMap* kv_map, const C
                 if (it.j1 > it.j0) pf_sanitize<D, kMulti>(p, sh, it, san_kv_it);
             } else {
                 // entries 0 .. plan.ctas-1 are the CTAs' first ones; the counter hands out the rest
-                if (lane == 0) next[iter & 1] = plan.ctas + atomicAdd(&p.ctrl[kCtrPrefill], 1);
+                if (lane == 0) next[iter & 1] = plan.ctas + atomicAdd(p.ctrl + lds_s32(sh.smem + Geo<D>::kSetOffset) + kSetPrefill, 1);
             }
             if (!piece_sync()) break;
             entry = next[iter & 1];
