@@ -855,9 +855,6 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
     const bool tensor_prefill = p.C > 0;
     volatile int* misc = reinterpret_cast<volatile int*>(scratch + 32);  // [0] TMEM base, [1] abort flag, [2..3] ticket flags
     if (threadIdx.x >= 32 && threadIdx.x < 32 + kPlanCounters) scratch[64 + threadIdx.x - 32] = 0;  // block-sum counters
-    // the chunks' descriptors go to shared memory: the roles of the chunk-prefill phase look them up by the item's chunk
-    // number instead of carrying them in registers
-    if (kMulti && warp == 2) pf_fill_chunk_table(p, scratch + kChunkTable);
     if (threadIdx.x < kWarps * Geo<D>::kStages) {
         mbar_init(base + Geo<D>::kBarOffset + threadIdx.x * 8, 1);
         fence_mbar_init();
@@ -886,6 +883,10 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
     int32_t* counters = p.ctrl + kCtrSets + set * kSetWords;
     if (threadIdx.x == 0) misc[7] = kCtrSets + set * kSetWords;
     if (blockIdx.x == 0 && threadIdx.x < kSetWords) p.ctrl[kCtrSets + (set ^ 1) * kSetWords + threadIdx.x] = 0;
+    // the chunks' descriptors go to shared memory: the roles of the chunk-prefill phase look them up by the item's chunk
+    // number instead of carrying them in registers (the table depends on the decode page count, which an earlier kernel may
+    // have written)
+    if (kMulti && warp == 2) pf_fill_chunk_table(p, scratch + kChunkTable);
     if (p.append_first) {
         // fused launch with chunks: this CTA's share of the new K/V rows, then its mark on the counter the readers wait for
         append_rows<kMulti>(p, D, (int64_t)blockIdx.x * kThreads + threadIdx.x, (int64_t)gridDim.x * kThreads);

@@ -189,7 +189,7 @@ __device__ __forceinline__ float pf_decode_steps(const MixedParams& p) {  // the
 // Several chunks in one iteration: the tail items (the last n_items mod G ones, G the CTAs that take entries) belong to chunks of very
 // different lengths, e.g. the end of a long prompt next to the start of a new one.  Each chunk gets its own piece
 // count, sized by its shortest item; while the tail entries outnumber the CTAs, the chunk with the shortest pieces
-// gives one up.  Run by one whole warp in the kernel prologue, lane j owning chunk j; fills the chunk table:
+// gives one up.  Run by one whole warp once earlier kernels have finished, lane j owning chunk j; fills the chunk table:
 // fields 0-3 the descriptors, 4 pieces per tail item, 5 items before the chunk, 6 tail entries before the chunk's
 // tail items (fields 5 and 6 hold INT_MAX where nothing may match), then the plan's totals.
 __device__ __forceinline__ void pf_fill_chunk_table(const MixedParams& p, int* tbl) {
