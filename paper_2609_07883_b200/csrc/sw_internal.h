@@ -47,6 +47,7 @@ struct MixedParams {
     // prefill_pages[cPage0[j]] (cPage0[nchunks] = num_prefill_pages).
     int C, n;
     int nchunks;
+    int chunk_items;      // work items of all chunks: 256-row groups times KV heads
     int cP[kMaxChunks], cC[kMaxChunks], cRow0[kMaxChunks], cPage0[kMaxChunks + 1];
     const int32_t* prefill_pages;
     int num_prefill_pages;

@@ -144,12 +144,14 @@ __device__ __forceinline__ bool wait_append(const MixedParams& p, uint32_t set_a
 // ---------------------------------------------------------------------------------------------------------------
 // mixed attention: shared-memory plan
 // ---------------------------------------------------------------------------------------------------------------
+constexpr int kPageHashBits = 2048;   // buckets of the hash that tells pages with one writer from pages that may have several
+
 template <int D>
 struct Geo {
     static constexpr int kHalves = D / 64;                    // 128-byte swizzled column blocks per row
     static constexpr int kBlockBytes = kPageSize * 128;       // one [16 tokens][64 elems] swizzled block
     static constexpr int kStageBytes = 2 * kHalves * kBlockBytes;  // K then V of one (page, kv head)
-    static constexpr int kStages = 256 / D;                   // page buffers in flight per warp: 16 KB whatever the head size
+    static constexpr int kStages = 2;                          // page buffers in flight per warp (four at head size 64 gain nothing)
     static constexpr int kRingBytes = kWarps * kStages * kStageBytes;
     static constexpr int kBarOffset = kRingBytes;                              // kWarps*kStages mbarriers
     static constexpr int kPfBarOffset = kBarOffset + kWarps * kStages * 8;     // barriers of the prefill tiles
@@ -160,7 +162,8 @@ struct Geo {
     static constexpr int kLastOffset = kIndptrOffset + (kMaxDecode + 1) * 4 + 12; // int32 id of request i's last page
     static constexpr int kMiscOffset = kLastOffset + kMaxDecode * 4;              // scan scratch, TMEM base, abort flag
     static constexpr int kSetOffset = kMiscOffset + (32 + 7) * 4;                 // where this launch's counters start (words into ctrl)
-    static constexpr int kSmemBytes = kMiscOffset + 768;   // 64 ints scan scratch and flags, the plan's counters, the chunk table
+    static constexpr int kSharedOffset = kMiscOffset + 768;   // after 64 ints scan scratch and flags, the plan's counters, the chunk table:
+    static constexpr int kSmemBytes = kSharedOffset + 2 * kPageHashBits / 8;      // two bit sets over hashed last pages
 };
 
 constexpr int kWideMergeSplits = 24;  // from this many units of a request on, its last g units share the merge
@@ -426,14 +429,16 @@ __device__ __forceinline__ void merge_splits(const MixedParams& p, const Unit& u
             float ms = __ldcg(ml + (r < nrows ? r : 0));
             const float ls = __ldcg(ml + kMaxGroup + (r < nrows ? r : 0));
             if (!live) ms = -INFINITY;
-            float mw = fmaxf(ms, m_all[r]);
+            float mw = fmaxf(ms, m_all[r]);   // over lanes 0 .. J-1
 #pragma unroll
-            for (int o2 = 16; o2 > 0; o2 >>= 1) mw = fmaxf(mw, __shfl_xor_sync(0xffffffffu, mw, o2));
+            for (int o2 = J / 2; o2 > 0; o2 >>= 1) mw = fmaxf(mw, __shfl_xor_sync(0xffffffffu, mw, o2));
+            mw = __shfl_sync(0xffffffffu, mw, 0);
             w[r] = ms == -INFINITY ? 0.f : fast_exp2((ms - mw) * p.sm_scale_log2);
             float lw = w[r] * ls;
             if (!live) lw = 0.f;
 #pragma unroll
-            for (int o2 = 16; o2 > 0; o2 >>= 1) lw += __shfl_xor_sync(0xffffffffu, lw, o2);
+            for (int o2 = J / 2; o2 > 0; o2 >>= 1) lw += __shfl_xor_sync(0xffffffffu, lw, o2);
+            lw = __shfl_sync(0xffffffffu, lw, 0);
             const float a = m_all[r] == -INFINITY ? 0.f : fast_exp2((m_all[r] - mw) * p.sm_scale_log2);
             l_all[r] = l_all[r] * a + lw;
             m_all[r] = mw;
@@ -488,13 +493,17 @@ __device__ __forceinline__ void patch_row(uint32_t buf, int slot, uint4 v) {
         sts_v4(buf + (lane / (D / 8)) * (Geo<D>::kHalves * Geo<D>::kBlockBytes) + (chunk >> 3) * Geo<D>::kBlockBytes + slot * 128 +
                    (((chunk & 7) ^ (slot & 7)) << 4), v.x, v.y, v.z, v.w);
 }
+__device__ __forceinline__ unsigned page_hash(int page) { return ((unsigned)page * 2654435761u) >> 21; }
+static_assert(kPageHashBits == 1 << (32 - 21), "the hash has as many values as there are buckets");
 // All new rows of the page in buffer `buf`, the last one of request i.  `lists`: shared address of the plan region.
 template <int D>
 __device__ __forceinline__ void patch_page(const MixedParams& p, uint32_t smem, uint32_t buf, int i, int kvh, int valid, uint4 own) {
     const int lane = threadIdx.x & 31;
     const int page = lds_s32(smem + Geo<D>::kLastOffset + i * 4);
+    const unsigned h = page_hash(page);
+    const bool several = lds_s32(smem + Geo<D>::kSharedOffset + (kPageHashBits + h) / 32 * 4) >> (h & 31) & 1;
 #pragma unroll 1
-    for (int j0 = 0; j0 < p.n; j0 += 32) {
+    for (int j0 = 0; several && j0 < p.n; j0 += 32) {
         const int j = j0 + lane;
         bool hit = false;
         if (j < p.n && j != i && lds_s32(smem + Geo<D>::kLastOffset + j * 4) == page)
@@ -859,6 +868,8 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
         mbar_init(base + Geo<D>::kBarOffset + threadIdx.x * 8, 1);
         fence_mbar_init();
     }
+    if (threadIdx.x >= 128 && threadIdx.x < 128 + 2 * kPageHashBits / 32)
+        reinterpret_cast<unsigned*>(smem + Geo<D>::kSharedOffset)[threadIdx.x - 128] = 0;
     if (threadIdx.x == 96) {
         tma_prefetch_desc(&kvp_map);
         mbar_init(base + Geo<D>::kLastBarOffset, kWarps);
@@ -872,6 +883,14 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
         misc[1] = 0;
         fence_mbar_init();
     }
+    // The plan of the chunk-prefill phase and, with several chunks, their descriptors go to shared memory: the roles look them
+    // up instead of carrying them in registers.  It may depend on the decode page count, which an earlier kernel may have
+    // written, and is made after the wait below; several chunks whose plan does not depend on it are planned here (the table
+    // takes a microsecond).
+    const bool plan_now = kMulti && !(p.n > 0 && p.chunk_items >= (int)gridDim.x);
+    if constexpr (kMulti) {
+        if (warp == 2 && plan_now) pf_fill_chunk_table(p, scratch + kChunkTable);
+    }
     // Everything above touched only shared memory and kernel parameters.  From here on the kernel reads what earlier
     // kernels of the stream wrote (the pool after the KV append, q, the page tables): wait for them to finish.
     grid_dependency_wait();
@@ -883,10 +902,10 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
     int32_t* counters = p.ctrl + kCtrSets + set * kSetWords;
     if (threadIdx.x == 0) misc[7] = kCtrSets + set * kSetWords;
     if (blockIdx.x == 0 && threadIdx.x < kSetWords) p.ctrl[kCtrSets + (set ^ 1) * kSetWords + threadIdx.x] = 0;
-    // the chunks' descriptors go to shared memory: the roles of the chunk-prefill phase look them up by the item's chunk
-    // number instead of carrying them in registers (the table depends on the decode page count, which an earlier kernel may
-    // have written)
-    if (kMulti && warp == 2) pf_fill_chunk_table(p, scratch + kChunkTable);
+    if (tensor_prefill && warp == 2 && !plan_now) {
+        if constexpr (kMulti) pf_fill_chunk_table(p, scratch + kChunkTable); else pf_fill_plan(p, scratch + kChunkTable);
+        __syncwarp();
+    }
     if (p.append_first) {
         // fused launch with chunks: this CTA's share of the new K/V rows, then its mark on the counter the readers wait for
         append_rows<kMulti>(p, D, (int64_t)blockIdx.x * kThreads + threadIdx.x, (int64_t)gridDim.x * kThreads);
@@ -903,7 +922,7 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
     int prefill_ctas = 0;
     LateJoin late{0, 0.f};
     if (tensor_prefill) {
-        const PfPlan pplan = pf_make_plan<kMulti>(p, base + Geo<D>::kMiscOffset + kChunkTable * 4);
+        const PfPlan pplan = pf_make_plan(base + Geo<D>::kMiscOffset + kChunkTable * 4);
         prefill_ctas = min(pplan.n_entries, pplan.ctas);
         late.ctas = prefill_ctas;
         late.us = kLateBaseUs + p.step_us * ((pplan.longest + pplan.pieces - 1) / pplan.pieces);
@@ -954,6 +973,10 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
                 }
             }
             sts_s32(base + Geo<D>::kLastOffset + i * 4, id);
+            // first request in its bucket: marked in the first set; any other: the bucket is marked in the second
+            unsigned* sets = reinterpret_cast<unsigned*>(smem + Geo<D>::kSharedOffset);
+            const unsigned h = page_hash(id), bit = 1u << (h & 31);
+            if (atomicOr(&sets[h / 32], bit) & bit) atomicOr(&sets[(kPageHashBits + h) / 32], bit);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(base + Geo<D>::kLastBarOffset);

@@ -260,21 +260,10 @@ __device__ __forceinline__ void pf_fill_chunk_table(const MixedParams& p, int* t
     }
 }
 
-template <bool kMulti>
-__device__ __forceinline__ PfPlan pf_make_plan(const MixedParams& p, uint32_t table) {
+// The same for a single chunk, whose descriptors are kernel parameters: the plan's totals only.  Run by one whole warp likewise, so
+// that the planning costs the roles of the chunk-prefill phase no register.
+__device__ __forceinline__ void pf_fill_plan(const MixedParams& p, int* tbl) {
     PfPlan plan;
-    plan.table = table;
-    if constexpr (kMulti) {  // worked out once per CTA by pf_fill_chunk_table
-        const uint32_t tot = table + kChunkTotals * 4;
-        plan.n_items = lds_s32(tot);
-        plan.n_whole = lds_s32(tot + 4);
-        plan.n_entries = lds_s32(tot + 8);
-        plan.longest = lds_s32(tot + 12);
-        plan.shortest = lds_s32(tot + 16);
-        plan.pieces = lds_s32(tot + 20);
-        plan.ctas = lds_s32(tot + 24);
-        return plan;
-    }
     int G = (int)gridDim.x;
     const int n_tp = pf_num_groups(p.group, p.cC[0]);
     plan.n_items = n_tp * p.Hkv;
@@ -285,9 +274,26 @@ __device__ __forceinline__ PfPlan pf_make_plan(const MixedParams& p, uint32_t ta
         plan.shortest = pf_steps_of_rank(p.group, p.cP[0], p.cC[0], n_tp, n_tp - 1);
     }
     const float decode_steps = pf_decode_steps(p);
-    const int entry_ctas = pf_entry_ctas(p, G, plan.n_items, 0.5f * (float)(plan.longest + plan.shortest) * (float)plan.n_items,
+    int entry_ctas = pf_entry_ctas(p, G, plan.n_items, 0.5f * (float)(plan.longest + plan.shortest) * (float)plan.n_items,
                                          decode_steps);
-    const bool rounds = entry_ctas < G;  // whole rounds of items (their lengths fall linearly with the rank) beside decode CTAs
+    if (p.n > 0 && plan.n_items < G && decode_steps >= kDecodeCtasMinSteps) {
+        // Fewer items than CTAs beside a decode phase bound by the streaming rate: on c CTAs, in rounds of whole items, they may
+        // end the launch sooner than side by side, since G - c CTAs stream from the start.  Lane l tries its own c (the last one
+        // the plain order, every item on its own CTA) and estimates the end in steps; a sixteenth has to be gained.  128 decodes
+        // of 128-16384 tokens beside 1024 tokens at prefix 4096: 128 items on 64 CTAs instead of 128, 331 -> 301 us; 16 of
+        // 16384-65536 beside 512 at 8192: 455 -> 431 us; where the plain order is kept (512 at 4096 or 16384, 256 at 28672
+        // beside the 128) nothing changes.
+        const float wp = 0.5f * (float)(plan.longest + plan.shortest) * (float)plan.n_items + kEntryCostSteps * (float)plan.n_items;
+        const int lane = threadIdx.x & 31;
+        const int c = lane < 31 ? (lane + 1) * 4 : plan.n_items;
+        const float t = c < plan.n_items ? kEntrySafety * wp / (float)c : (float)plan.longest + kEntryCostSteps;
+        const float rate = fminf(1.f, (float)(G - c) / (float)kDecodeCtasAtFullRate);
+        const int end = c <= plan.n_items ? (int)(16.f * (t + fmaxf(0.f, decode_steps - t * rate))) : 0x3ffffff;
+        const int plain = min(__shfl_sync(0xffffffffu, end, 31), 0x3ffffff);
+        const int best = __reduce_min_sync(0xffffffffu, (min(end, 0x3ffffff) << 5) | lane);
+        if ((best >> 5) < plain - plain / 16) entry_ctas = ((best & 31) + 1) * 4;
+    }
+    const bool rounds = entry_ctas < G;  // rounds of whole items (their lengths fall linearly with the rank) beside decode CTAs
     G = entry_ctas;
     plan.ctas = G;
     const int r = plan.n_items % G;
@@ -333,6 +339,29 @@ __device__ __forceinline__ PfPlan pf_make_plan(const MixedParams& p, uint32_t ta
     }
     if (plan.pieces == 1) plan.n_whole = plan.n_items;
     plan.n_entries = plan.n_whole + (plan.n_items - plan.n_whole) * plan.pieces;
+    if ((threadIdx.x & 31) == 0) {
+        int* tot = tbl + kChunkTotals;
+        tot[0] = plan.n_items;
+        tot[1] = plan.n_whole;
+        tot[2] = plan.n_entries;
+        tot[3] = plan.longest;
+        tot[4] = plan.shortest;
+        tot[5] = plan.pieces;
+        tot[6] = plan.ctas;
+    }
+}
+
+__device__ __forceinline__ PfPlan pf_make_plan(uint32_t table) {  // worked out once per CTA by one of the two
+    PfPlan plan;
+    plan.table = table;
+    const uint32_t tot = table + kChunkTotals * 4;
+    plan.n_items = lds_s32(tot);
+    plan.n_whole = lds_s32(tot + 4);
+    plan.n_entries = lds_s32(tot + 8);
+    plan.longest = lds_s32(tot + 12);
+    plan.shortest = lds_s32(tot + 16);
+    plan.pieces = lds_s32(tot + 20);
+    plan.ctas = lds_s32(tot + 24);
     return plan;
 }
 
