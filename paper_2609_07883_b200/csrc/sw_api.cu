@@ -352,7 +352,6 @@ sw_status run_mixed(sw_ctx* ctx, void* kv_pool, const sw_batch* batch, const voi
     p.C = ch.rows;
     p.n = batch->num_decode;
     p.nchunks = ch.n;
-    for (int j = 0; j < ch.n; ++j) p.chunk_items += (ch.C[j] + 256 / p.group - 1) / (256 / p.group) * p.Hkv;
     std::memcpy(p.cP, ch.P, sizeof p.cP);
     std::memcpy(p.cC, ch.C, sizeof p.cC);
     std::memcpy(p.cRow0, ch.row0, sizeof p.cRow0);

@@ -25,8 +25,8 @@ constexpr int kMaxChunk = 65536;        // chunk tokens per iteration (256-row g
 // kCtrArrived counts the CTAs that have ended, modulo two grids; launches use the two counter sets at kCtrSets in turn.
 enum CtrlWord { kCtrArrived = 0, kCtrStatus = 2, kCtrDetail = 3, kCtrSets = 16, kCtrWords = 64 };
 // Words of a counter set: decode units handed out by the counter, chunk-prefill entries likewise, and (fused launches with
-// chunks) CTAs that have written their share of the new K/V rows.
-enum SetWord { kSetWork = 0, kSetPrefill = 1, kSetAppend = 2, kSetWords = 16 };
+// chunks) CTAs that have written their share of the new K/V rows; decode units of the launch + 1 once they are known.
+enum SetWord { kSetWork = 0, kSetPrefill = 1, kSetAppend = 2, kSetItems = 3, kSetWords = 16 };
 
 // Device-detected problem locators written to kCtrDetail (high byte = site, low 24 bits = index).
 enum DetailSite { kSiteAppendPage = 1, kSiteAppendLen = 2, kSiteAttnLen = 3, kSiteAttnPage = 4, kSiteWait = 5,
@@ -47,7 +47,6 @@ struct MixedParams {
     // prefill_pages[cPage0[j]] (cPage0[nchunks] = num_prefill_pages).
     int C, n;
     int nchunks;
-    int chunk_items;      // work items of all chunks: 256-row groups times KV heads
     int cP[kMaxChunks], cC[kMaxChunks], cRow0[kMaxChunks], cPage0[kMaxChunks + 1];
     const int32_t* prefill_pages;
     int num_prefill_pages;

@@ -28,65 +28,80 @@ __device__ __forceinline__ void report(int32_t* ctrl, int code, int site, int in
 // ---------------------------------------------------------------------------------------------------------------
 // KV append
 // ---------------------------------------------------------------------------------------------------------------
-// One thread per (row, 16-byte piece of the row's Hkv*D elements); it copies that piece of K and of V.  `first` and
-// `stride` spread the pieces over the calling threads.
+// A warp takes 32 of the 16-byte pieces of a row's Hkv*D elements, of K and of V, kAppendBatch times at once: what the append
+// costs is its chain of latencies (position, page id, row, store), not its bytes.  `first` and `stride` spread the pieces over
+// the calling warps.  (One piece per thread and pass, with 64-bit divisions, took 7.6-11 us of a launch with 2048 chunk rows.)
 // (P is AppendParams or MixedParams: the fields have the same names; every index into the chunk arrays is a
 // compile-time constant so that the kernel parameters stay in constant memory.)
+constexpr int kAppendBatch = 4;
 template <bool kMulti, class P>
-__device__ __forceinline__ void append_rows(const P& p, int head_dim, int64_t first, int64_t stride) {
+__device__ __forceinline__ void append_rows(const P& p, int head_dim, int first, int stride) {
+    const int lane = threadIdx.x & 31;
     const int pieces_per_row = p.Hkv * head_dim / 8;
-    const int64_t total = (int64_t)(p.C + p.n) * pieces_per_row;
-    for (int64_t idx = first; idx < total; idx += stride) {
-        const int row = (int)(idx / pieces_per_row);
-        const int piece = (int)(idx % pieces_per_row);
-        int64_t pos;
-        const int32_t* pages;
-        int npages;
-        if (row < p.C) {
-            // the chunk this row belongs to: the last one that starts at or before it
-            int cP = p.cP[0], cRow0 = 0, page0 = 0, page1 = p.num_prefill_pages;
+    const int per_row = (pieces_per_row + 31) / 32;   // warp-wide parts of a row
+    const int total = (p.C + p.n) * per_row;
+#pragma unroll 1
+    for (int c0 = first; c0 < total; c0 += kAppendBatch * stride) {
+        uint4 k[kAppendBatch], v[kAppendBatch];
+        int page[kAppendBatch], slot[kAppendBatch];   // slot: -1 = no such position in the list (reported)
 #pragma unroll
-            for (int j = 0; j < kMaxChunks; ++j)
-                if (kMulti && j < p.nchunks && row >= p.cRow0[j]) {
-                    cP = p.cP[j];
-                    cRow0 = p.cRow0[j];
-                    page0 = p.cPage0[j];
-                    page1 = p.cPage0[j + 1];
-                }
-            pos = (int64_t)cP + (row - cRow0);
-            pages = p.prefill_pages + page0;
-            npages = page1 - page0;
-        } else {
-            const int i = row - p.C;
-            const int len = p.decode_kv_len[i];
-            if (len < 1) {
-                report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAppendLen, i);
+        for (int b = 0; b < kAppendBatch; ++b) {
+            const int c = c0 + b * stride;
+            slot[b] = -1;
+            if (c >= total) break;
+            const int row = c / per_row, piece = (c - row * per_row) * 32 + lane;
+            if (piece < pieces_per_row) {
+                const int64_t src = ((int64_t)row * pieces_per_row + piece) * 8;
+                k[b] = *reinterpret_cast<const uint4*>(p.k_new + src);
+                v[b] = *reinterpret_cast<const uint4*>(p.v_new + src);
+            }
+            unsigned pos;
+            const int32_t* pages;
+            int npages;
+            if (row < p.C) {
+                // the chunk this row belongs to: the last one that starts at or before it
+                int cP = p.cP[0], cRow0 = 0, page0 = 0, page1 = p.num_prefill_pages;
+#pragma unroll
+                for (int j = 0; j < kMaxChunks; ++j)
+                    if (kMulti && j < p.nchunks && row >= p.cRow0[j]) {
+                        cP = p.cP[j];
+                        cRow0 = p.cRow0[j];
+                        page0 = p.cPage0[j];
+                        page1 = p.cPage0[j + 1];
+                    }
+                pos = (unsigned)cP + (unsigned)(row - cRow0);
+                pages = p.prefill_pages + page0;
+                npages = page1 - page0;
+            } else {
+                const int i = row - p.C;
+                const int len = p.decode_kv_len[i];
+                pos = len < 1 ? 0xffffffffu : (unsigned)len - 1;
+                const int beg = p.decode_page_indptr[i];
+                pages = p.decode_pages + beg;
+                npages = p.decode_page_indptr[i + 1] - beg;
+            }
+            const int pi = (int)(pos / kPageSize);
+            if (pi < npages) {
+                slot[b] = (int)(pos % kPageSize);
+                page[b] = pages[pi];
+            } else {
+                report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAppendLen, row);
+            }
+        }
+#pragma unroll
+        for (int b = 0; b < kAppendBatch; ++b) {
+            const int c = c0 + b * stride;
+            if (c >= total) break;
+            const int row = c / per_row, e0 = ((c - row * per_row) * 32 + lane) * 8;   // element offset inside the row's [Hkv][D]
+            if (slot[b] < 0 || e0 >= pieces_per_row * 8) continue;
+            if (page[b] < 0 || page[b] >= p.num_pages) {
+                report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAppendPage, row);
                 continue;
             }
-            pos = (int64_t)len - 1;
-            const int beg = p.decode_page_indptr[i];
-            pages = p.decode_pages + beg;
-            npages = p.decode_page_indptr[i + 1] - beg;
+            const int64_t block = ((int64_t)page[b] * 2 * p.Hkv + e0 / head_dim) * kPageSize + slot[b];   // K; V is Hkv blocks further
+            *reinterpret_cast<uint4*>(p.pool + block * head_dim + e0 % head_dim) = k[b];
+            *reinterpret_cast<uint4*>(p.pool + (block + (int64_t)p.Hkv * kPageSize) * head_dim + e0 % head_dim) = v[b];
         }
-        const int64_t pi = pos / kPageSize;
-        const int slot = (int)(pos % kPageSize);
-        if (pi >= npages) {
-            report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAppendLen, row);
-            continue;
-        }
-        const int64_t page = pages[pi];
-        if (page < 0 || page >= p.num_pages) {
-            report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAppendPage, row);
-            continue;
-        }
-        const int e0 = piece * 8;          // element offset inside the row's [Hkv][D]
-        const int kvh = e0 / head_dim;
-        const int e = e0 % head_dim;
-        const int64_t src = (int64_t)row * p.Hkv * head_dim + e0;
-        const int64_t dst_k = ((((int64_t)page * 2 + 0) * p.Hkv + kvh) * kPageSize + slot) * head_dim + e;
-        const int64_t dst_v = ((((int64_t)page * 2 + 1) * p.Hkv + kvh) * kPageSize + slot) * head_dim + e;
-        *reinterpret_cast<uint4*>(p.pool + dst_k) = *reinterpret_cast<const uint4*>(p.k_new + src);
-        *reinterpret_cast<uint4*>(p.pool + dst_v) = *reinterpret_cast<const uint4*>(p.v_new + src);
     }
 }
 
@@ -95,14 +110,14 @@ __global__ void sw_kv_append_kernel(const AppendParams p) {
     // the previous iteration, possibly still reading this pool) drains; nothing is touched before this wait
     grid_launch_dependents();
     grid_dependency_wait();
-    append_rows<true>(p, p.D, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+    append_rows<true>(p, p.D, (int)(blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32), (int)(gridDim.x * (blockDim.x / 32)));
 }
 
 cudaError_t launch_kv_append(const AppendParams& p, int num_sms, cudaStream_t stream) {
-    const int64_t total = (int64_t)(p.C + p.n) * (p.Hkv * p.D / 8);
+    const int64_t total = (int64_t)(p.C + p.n) * ((p.Hkv * p.D / 8 + 31) / 32);   // warp-wide parts of rows
     if (total == 0) return cudaSuccess;
     const int threads = 256;
-    int64_t blocks = (total + threads - 1) / threads;
+    int64_t blocks = (total + threads / 32 - 1) / (threads / 32);
     if (blocks > (int64_t)num_sms * 8) blocks = (int64_t)num_sms * 8;   // eight 256-thread blocks fill an SM
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks);
@@ -862,7 +877,7 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
     int* scratch = reinterpret_cast<int*>(smem + Geo<D>::kMiscOffset);
 
     const bool tensor_prefill = p.C > 0;
-    volatile int* misc = reinterpret_cast<volatile int*>(scratch + 32);  // [0] TMEM base, [1] abort flag, [2..3] ticket flags
+    volatile int* misc = reinterpret_cast<volatile int*>(scratch + 32);  // [0] TMEM base, [1] abort flag, [2..3] ticket flags, [5..6] next entry, [7] where this launch's counters start, [8] no units left
     if (threadIdx.x >= 32 && threadIdx.x < 32 + kPlanCounters) scratch[64 + threadIdx.x - 32] = 0;  // block-sum counters
     if (threadIdx.x < kWarps * Geo<D>::kStages) {
         mbar_init(base + Geo<D>::kBarOffset + threadIdx.x * 8, 1);
@@ -881,15 +896,15 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
         }
         misc[0] = 0;
         misc[1] = 0;
+        misc[8] = 0;
         fence_mbar_init();
     }
     // The plan of the chunk-prefill phase and, with several chunks, their descriptors go to shared memory: the roles look them
-    // up instead of carrying them in registers.  It may depend on the decode page count, which an earlier kernel may have
-    // written, and is made after the wait below; several chunks whose plan does not depend on it are planned here (the table
-    // takes a microsecond).
-    const bool plan_now = kMulti && !(p.n > 0 && p.chunk_items >= (int)gridDim.x);
+    // up instead of carrying them in registers.  It depends on the decode page count, which an earlier kernel may have written,
+    // so it is made after the wait below; the table of several chunks (a microsecond) is filled here for the usual case, that
+    // every CTA takes entries, and filled again after the wait where that turns out otherwise.
     if constexpr (kMulti) {
-        if (warp == 2 && plan_now) pf_fill_chunk_table(p, scratch + kChunkTable);
+        if (warp == 2) pf_fill_chunk_table(p, scratch + kChunkTable, (int)gridDim.x);
     }
     // Everything above touched only shared memory and kernel parameters.  From here on the kernel reads what earlier
     // kernels of the stream wrote (the pool after the KV append, q, the page tables): wait for them to finish.
@@ -902,13 +917,21 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
     int32_t* counters = p.ctrl + kCtrSets + set * kSetWords;
     if (threadIdx.x == 0) misc[7] = kCtrSets + set * kSetWords;
     if (blockIdx.x == 0 && threadIdx.x < kSetWords) p.ctrl[kCtrSets + (set ^ 1) * kSetWords + threadIdx.x] = 0;
-    if (tensor_prefill && warp == 2 && !plan_now) {
-        if constexpr (kMulti) pf_fill_chunk_table(p, scratch + kChunkTable); else pf_fill_plan(p, scratch + kChunkTable);
+    if (tensor_prefill && warp == 2) {
+        if constexpr (kMulti) {
+            __syncwarp();
+            const int ctas = pf_table_ctas(p, scratch + kChunkTable);
+            __syncwarp();
+            if (ctas != (int)gridDim.x) pf_fill_chunk_table(p, scratch + kChunkTable, ctas);
+        } else {
+            pf_fill_plan(p, scratch + kChunkTable);
+        }
         __syncwarp();
     }
     if (p.append_first) {
-        // fused launch with chunks: this CTA's share of the new K/V rows, then its mark on the counter the readers wait for
-        append_rows<kMulti>(p, D, (int64_t)blockIdx.x * kThreads + threadIdx.x, (int64_t)gridDim.x * kThreads);
+        // fused launch with chunks: this CTA's share of the new K/V rows (the planning warp has none), then its mark on the
+        // counter the readers wait for
+        if (warp != 2) append_rows<kMulti>(p, D, (int)blockIdx.x * (kWarps - 1) + warp - (warp > 2), (int)gridDim.x * (kWarps - 1));
         fence_proxy_async_global();
         __threadfence();
         __syncthreads();
@@ -954,6 +977,10 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
         }
         __syncthreads();
     }
+    if (p.n == 0 || misc[8]) {   // no decode units, or none left for this CTA
+        if (threadIdx.x == 0) atomicInc(reinterpret_cast<unsigned*>(&p.ctrl[kCtrArrived]), 2 * gridDim.x - 1);
+        return;
+    }
 
     const Plan plan = make_plan(p, unit_prefix, reinterpret_cast<int*>(smem + Geo<D>::kLenOffset),
                                 reinterpret_cast<int*>(smem + Geo<D>::kIndptrOffset), scratch, late,
@@ -981,6 +1008,7 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
         __syncwarp();
         if (lane == 0) mbar_arrive(base + Geo<D>::kLastBarOffset);
     }
+    if ((int)blockIdx.x == prefill_ctas && threadIdx.x == 0) atomicExch(p.ctrl + misc[7] + kSetItems, plan.total_items + 1);
     if (plan.total_items > p.max_items) {
         if (threadIdx.x == 0) report(p.ctrl, SW_ERR_WORKSPACE, kSiteScratch, plan.total_items);
     } else {

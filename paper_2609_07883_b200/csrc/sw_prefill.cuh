@@ -189,10 +189,10 @@ __device__ __forceinline__ float pf_decode_steps(const MixedParams& p) {  // the
 // Several chunks in one iteration: the tail items (the last n_items mod G ones, G the CTAs that take entries) belong to chunks of very
 // different lengths, e.g. the end of a long prompt next to the start of a new one.  Each chunk gets its own piece
 // count, sized by its shortest item; while the tail entries outnumber the CTAs, the chunk with the shortest pieces
-// gives one up.  Run by one whole warp once earlier kernels have finished, lane j owning chunk j; fills the chunk table:
+// gives one up.  G: CTAs that take entries.  Run by one whole warp, lane j owning chunk j; fills the chunk table:
 // fields 0-3 the descriptors, 4 pieces per tail item, 5 items before the chunk, 6 tail entries before the chunk's
 // tail items (fields 5 and 6 hold INT_MAX where nothing may match), then the plan's totals.
-__device__ __forceinline__ void pf_fill_chunk_table(const MixedParams& p, int* tbl) {
+__device__ __forceinline__ void pf_fill_chunk_table(const MixedParams& p, int* tbl, int G) {
     const int lane = threadIdx.x & 31;
     int P = 0, C = 0, row0 = 0, page0 = 0;
 #pragma unroll
@@ -221,9 +221,7 @@ __device__ __forceinline__ void pf_fill_chunk_table(const MixedParams& p, int* t
         longest = pf_steps_of_rank(p.group, P, C, n_tp, 0);
         shortest = pf_steps_of_rank(p.group, P, C, n_tp, n_tp - 1);
     }
-    // beside enough decode pages a few CTAs take no entry (the rule of the single-chunk plan; pieces in one round here)
     const int steps2 = __reduce_add_sync(0xffffffffu, n_tp > 0 ? (longest + shortest) * cnt : 0);
-    const int G = pf_entry_ctas(p, (int)gridDim.x, n_items, 0.5f * (float)steps2, pf_decode_steps(p));
     const int n_whole = n_items - n_items % G;
     const int tail = max(0, before + cnt - max(before, n_whole));
     int k = tail > 0 ? pf_pieces_for(shortest) : 1;
@@ -257,7 +255,14 @@ __device__ __forceinline__ void pf_fill_chunk_table(const MixedParams& p, int* t
         tot[4] = shortest;
         tot[5] = n_whole == 0 ? k0 : 1;
         tot[6] = G;
+        tot[7] = steps2;
     }
+}
+// Beside enough decode pages a few CTAs take no entry (the rule of the single-chunk plan; pieces in one round here): how many do, for
+// a table filled with the whole grid.
+__device__ __forceinline__ int pf_table_ctas(const MixedParams& p, const int* tbl) {
+    const int* tot = tbl + kChunkTotals;
+    return pf_entry_ctas(p, (int)gridDim.x, tot[0], 0.5f * (float)tot[7], pf_decode_steps(p));
 }
 
 // The same for a single chunk, whose descriptors are kernel parameters: the plan's totals only.  Run by one whole warp likewise, so
@@ -918,7 +923,7 @@ __device__ __forceinline__ bool pf_softmax(const CUtensorMap* out_map, const Mix
 }
 
 // ---- the prefill phase of one CTA ----------------------------------------------------------------------------------
-// `next` points at two shared-memory ints: the idle warp fetches the following entry from the global counter while
+// `next` points at two shared-memory ints (after them: where the launch's counters start, and whether no decode unit is left): the idle warp fetches the following entry from the global counter while
 // the current one is processed and leaves it in next[iteration parity]; everyone reads it after the piece barrier.
 template <int D, bool kMulti>
 __device__ __forceinline__ void prefill_phase(const CUtensorMap* kv_map, const CUtensorMap* q_map, const CUtensorMap* out_map,
@@ -950,6 +955,14 @@ __device__ __forceinline__ void prefill_phase(const CUtensorMap* kv_map, const C
                 if (it.j1 > it.j0) pf_mma<D>(p, sh, it, mma_state);
             } else if (warp == 2) {
                 if (it.j1 > it.j0) pf_sanitize<D, kMulti>(p, sh, it, san_kv_it);
+                // Near the end of what may be the CTA's last entry: whether the decode units have all been handed out (the CTAs
+                // that started with them have published their number).  Then the CTA need not work the decode plan out afterwards,
+                // which takes 2-3 us.
+                if (lane == 0 && p.n > 0) {
+                    const int32_t* counters = p.ctrl + next[2];
+                    const int items = ld_relaxed_gpu(&counters[kSetItems]) - 1, drawn = ld_relaxed_gpu(&counters[kSetWork]);
+                    next[3] = items >= 0 && ((int)gridDim.x - min(plan.n_entries, plan.ctas)) * kWarps + drawn >= items;
+                }
             } else {
                 // entries 0 .. plan.ctas-1 are the CTAs' first ones; the counter hands out the rest
                 if (lane == 0) next[iter & 1] = plan.ctas + atomicAdd(p.ctrl + lds_s32(sh.smem + Geo<D>::kSetOffset) + kSetPrefill, 1);
