@@ -71,6 +71,12 @@ WsLayout ws_layout(const sw_layout& l, int max_chunk, int max_decode, int64_t ma
 
 }  // namespace
 
+// Host-buffer iterations of kHostPartBytes of inputs or more are run in parts, so that one part's launch runs beside the next one's
+// copies.  Two parts: more of them cost more calls and launches than they hide (576 rows of 12 KB: 320 us whole, 297 in two parts,
+// 312 in three or four).
+constexpr int kHostParts = 2;
+constexpr size_t kHostPartBytes = 4u << 20;
+
 struct sw_ctx {
     sw_layout layout;
     int device = 0;
@@ -88,6 +94,9 @@ struct sw_ctx {
     };
     std::vector<MapEntry> kv_maps;  // small cache: one entry per pool of a layer stack
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+    // host-buffer iterations in parts: the copies' stream and events, made by the first call that uses them
+    cudaStream_t copies = nullptr;
+    cudaEvent_t ev_start = nullptr, ev_up = nullptr, ev_done[kHostParts + 1] = {};   // the last one: the decode rows
 };
 
 namespace {
@@ -282,6 +291,11 @@ void sw_destroy(sw_ctx* ctx) {
     if (!ctx) return;
     if (ctx->ev0) cudaEventDestroy(ctx->ev0);
     if (ctx->ev1) cudaEventDestroy(ctx->ev1);
+    if (ctx->copies) cudaStreamDestroy(ctx->copies);
+    if (ctx->ev_start) cudaEventDestroy(ctx->ev_start);
+    if (ctx->ev_up) cudaEventDestroy(ctx->ev_up);
+    for (cudaEvent_t e : ctx->ev_done)
+        if (e) cudaEventDestroy(e);
     delete ctx;
 }
 
@@ -427,6 +441,158 @@ sw_status sw_mixed_iteration_run(sw_ctx* ctx, void* kv_pool, const sw_batch* bat
     return run_iteration(ctx, kv_pool, batch, k_new, v_new, q, out, lse, stream, "sw_mixed_iteration_run");
 }
 
+namespace {
+// The device copies of a host batch's page tables, inside the workspace.
+struct HostTables {
+    int32_t *len, *indptr, *dec_pages, *pf_pages;
+};
+
+sw_status copy_tables(const sw_batch* hb, const HostTables& t, int64_t n_dec_pages, cudaStream_t s) {
+    const int n = hb->num_decode;
+    if (n > 0) {
+        SW_CUDA(cudaMemcpyAsync(t.len, hb->decode_kv_len, (size_t)n * 4, cudaMemcpyHostToDevice, s));
+        SW_CUDA(cudaMemcpyAsync(t.indptr, hb->decode_page_indptr, (size_t)(n + 1) * 4, cudaMemcpyHostToDevice, s));
+        if (n_dec_pages > 0)
+            SW_CUDA(cudaMemcpyAsync(t.dec_pages, hb->decode_pages, (size_t)n_dec_pages * 4, cudaMemcpyHostToDevice, s));
+    }
+    if (hb->num_prefill_pages > 0)
+        SW_CUDA(cudaMemcpyAsync(t.pf_pages, hb->prefill_pages, (size_t)hb->num_prefill_pages * 4, cudaMemcpyHostToDevice, s));
+    return SW_OK;
+}
+
+// Whether a page that chunk rows are written to is also the last page of a decode request (then a decode row and chunk rows may
+// attend each other, and the iteration is not taken apart).
+bool chunks_meet_decodes(const sw_batch* hb, const Chunks& ch) {
+    std::vector<int32_t> written;
+    for (int j = 0; j < ch.n; ++j)
+        for (int64_t pi = ch.P[j] / sw::kPageSize; pi <= ((int64_t)ch.P[j] + ch.C[j] - 1) / sw::kPageSize; ++pi)
+            written.push_back(hb->prefill_pages[ch.page0[j] + pi]);
+    std::sort(written.begin(), written.end());
+    for (int i = 0; i < hb->num_decode; ++i) {
+        const int pages = (int)(((int64_t)hb->decode_kv_len[i] + sw::kPageSize - 1) / sw::kPageSize);
+        const int beg = hb->decode_page_indptr[i], end = hb->decode_page_indptr[i + 1];
+        if (pages < 1 || beg < 0 || end > hb->decode_page_indptr[hb->num_decode] || pages > end - beg) continue;
+        if (std::binary_search(written.begin(), written.end(), hb->decode_pages[beg + pages - 1])) return true;
+    }
+    return false;
+}
+
+// Chunk rows of a part of a host-buffer iteration (0: it is run whole).  Parts are whole 256-row groups.  Where the chunks'
+// arithmetic (at 1.2 PFLOP/s) takes longer than the way up (at 46 GB/s), parts of fewer work items than there are SMs would cost
+// more than they hide.
+int host_part_rows(const sw_ctx* ctx, const sw_batch* hb, const Chunks& ch, size_t up_bytes) {
+    const sw_layout& l = ctx->layout;
+    if (ch.rows == 0 || up_bytes < kHostPartBytes) return 0;
+    const int group_rows = 256 / (l.num_q_heads / l.num_kv_heads);
+    int groups = ((ch.rows + kHostParts - 1) / kHostParts + group_rows - 1) / group_rows;
+    double pairs = 0.;   // attended (query, key) pairs
+    for (int j = 0; j < ch.n; ++j) pairs += (double)ch.C[j] * ((double)ch.P[j] + 0.5 * (double)ch.C[j]);
+    if (pairs * 4. * l.num_q_heads * l.head_dim / 1.2e15 > (double)up_bytes / 46e9)
+        groups = std::max(groups, ctx->num_sms / l.num_kv_heads);
+    if (groups * group_rows >= ch.rows) return 0;
+    try {
+        return chunks_meet_decodes(hb, ch) ? 0 : groups * group_rows;
+    } catch (...) {
+        return 0;   // no host memory for the comparison
+    }
+}
+
+sw_status make_host_streams(sw_ctx* ctx) {
+    if (!ctx->copies) SW_CUDA(cudaStreamCreateWithFlags(&ctx->copies, cudaStreamNonBlocking));
+    if (!ctx->ev_start) SW_CUDA(cudaEventCreateWithFlags(&ctx->ev_start, cudaEventDisableTiming));
+    if (!ctx->ev_up) SW_CUDA(cudaEventCreateWithFlags(&ctx->ev_up, cudaEventDisableTiming));
+    for (cudaEvent_t& e : ctx->ev_done)
+        if (!e) SW_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    return SW_OK;
+}
+
+// The host-buffer iteration in parts: the decode rows, then the chunk rows in runs of `per` consecutive rows (a chunk cut at a row
+// is the same attention: the rows behind the cut have a longer prefix).  While a part computes, the next one's inputs are on their way.
+sw_status iterate_parts(sw_ctx* ctx, void* kv_pool, const sw_batch* hb, const Chunks& ch, int per, const HostTables& t,
+                        int64_t n_dec_pages, const void* h_q, const void* h_k, const void* h_v, void* h_out, float* h_lse,
+                        cudaStream_t s) {
+    const sw_layout& l = ctx->layout;
+    const size_t q_row = (size_t)l.num_q_heads * l.head_dim * 2, kv_row = (size_t)l.num_kv_heads * l.head_dim * 2;
+    uint8_t *d_q = ctx->ws + ctx->w.st_q, *d_k = ctx->ws + ctx->w.st_k, *d_v = ctx->ws + ctx->w.st_v, *d_out = ctx->ws + ctx->w.st_out;
+    float* d_lse = h_lse ? reinterpret_cast<float*>(ctx->ws + ctx->w.st_lse) : nullptr;
+    const int n = hb->num_decode;
+    auto up_rows = [&](int r0, int rows) -> sw_status {
+        SW_CUDA(cudaMemcpyAsync(d_k + r0 * kv_row, (const uint8_t*)h_k + r0 * kv_row, rows * kv_row, cudaMemcpyHostToDevice, ctx->copies));
+        SW_CUDA(cudaMemcpyAsync(d_v + r0 * kv_row, (const uint8_t*)h_v + r0 * kv_row, rows * kv_row, cudaMemcpyHostToDevice, ctx->copies));
+        SW_CUDA(cudaMemcpyAsync(d_q + r0 * q_row, (const uint8_t*)h_q + r0 * q_row, rows * q_row, cudaMemcpyHostToDevice, ctx->copies));
+        return SW_OK;
+    };
+    auto down_rows = [&](int r0, int rows) -> sw_status {
+        SW_CUDA(cudaMemcpyAsync((uint8_t*)h_out + r0 * q_row, d_out + r0 * q_row, rows * q_row, cudaMemcpyDeviceToHost, ctx->copies));
+        if (h_lse)
+            SW_CUDA(cudaMemcpyAsync(h_lse + (size_t)r0 * l.num_q_heads, d_lse + (size_t)r0 * l.num_q_heads,
+                                    (size_t)rows * l.num_q_heads * 4, cudaMemcpyDeviceToHost, ctx->copies));
+        return SW_OK;
+    };
+    // the copies come after whatever the caller's stream was doing (it may produce the host buffers)
+    SW_CUDA(cudaEventRecord(ctx->ev_start, s));
+    SW_CUDA(cudaStreamWaitEvent(ctx->copies, ctx->ev_start, 0));
+    sw_status st = copy_tables(hb, t, n_dec_pages, ctx->copies);
+    if (st != SW_OK) return st;
+    sw_batch part = *hb;
+    part.decode_kv_len = t.len;
+    part.decode_page_indptr = t.indptr;
+    part.decode_pages = t.dec_pages;
+    if (n > 0) {
+        if ((st = up_rows(ch.rows, n)) != SW_OK) return st;
+        SW_CUDA(cudaEventRecord(ctx->ev_up, ctx->copies));
+        SW_CUDA(cudaStreamWaitEvent(s, ctx->ev_up, 0));
+        part.num_chunks = part.prefix_len = part.chunk_len = part.num_prefill_pages = 0;
+        st = sw_mixed_iteration_run(ctx, kv_pool, &part, d_k + ch.rows * kv_row, d_v + ch.rows * kv_row, d_q + ch.rows * q_row,
+                                    d_out + ch.rows * q_row, d_lse ? d_lse + (size_t)ch.rows * l.num_q_heads : nullptr, s);
+        if (st != SW_OK) return st;
+        SW_CUDA(cudaEventRecord(ctx->ev_done[kHostParts], s));
+    }
+    int done = 0;
+    for (int r0 = 0; r0 < ch.rows; r0 += per, ++done) {
+        const int rows = std::min(per, ch.rows - r0);
+        if ((st = up_rows(r0, rows)) != SW_OK) return st;
+        SW_CUDA(cudaEventRecord(ctx->ev_up, ctx->copies));
+        SW_CUDA(cudaStreamWaitEvent(s, ctx->ev_up, 0));
+        part.num_decode = 0;
+        int32_t prefix[sw::kMaxChunks], len[sw::kMaxChunks], pages[sw::kMaxChunks + 1];
+        int m = 0, page0 = 0;
+        for (int j = 0; j < ch.n; ++j) {
+            const int a = std::max(r0, ch.row0[j]), b = std::min(r0 + rows, ch.row0[j] + ch.C[j]);
+            if (a >= b) continue;
+            if (m == 0) page0 = ch.page0[j];
+            prefix[m] = ch.P[j] + (a - ch.row0[j]);
+            len[m] = b - a;
+            pages[m] = ch.page0[j] - page0;
+            pages[++m] = ch.page0[j + 1] - page0;
+        }
+        part.prefill_pages = t.pf_pages + page0;
+        part.num_prefill_pages = pages[m];
+        part.num_chunks = m > 1 ? m : 0;
+        part.prefix_len = prefix[0];
+        part.chunk_len = m > 1 ? rows : len[0];
+        part.chunk_prefix_lens = prefix;
+        part.chunk_lens = len;
+        part.chunk_page_indptr = pages;
+        st = sw_mixed_iteration_run(ctx, kv_pool, &part, d_k + r0 * kv_row, d_v + r0 * kv_row, d_q + r0 * q_row, d_out + r0 * q_row,
+                                    d_lse ? d_lse + (size_t)r0 * l.num_q_heads : nullptr, s);
+        if (st != SW_OK) return st;
+        SW_CUDA(cudaEventRecord(ctx->ev_done[done], s));
+    }
+    // The results follow the last inputs on the same stream: copies of a few megabytes in both directions at once are slower on
+    // this platform than one after the other (4 MB each way: 80 us alone, 370 us together).
+    if (n > 0) {
+        SW_CUDA(cudaStreamWaitEvent(ctx->copies, ctx->ev_done[kHostParts], 0));
+        if ((st = down_rows(ch.rows, n)) != SW_OK) return st;
+    }
+    for (int i = 0; i < done; ++i) {
+        SW_CUDA(cudaStreamWaitEvent(ctx->copies, ctx->ev_done[i], 0));
+        if ((st = down_rows(i * per, std::min(per, ch.rows - i * per))) != SW_OK) return st;
+    }
+    return SW_OK;
+}
+}  // namespace
+
 sw_status sw_mixed_iteration_host(sw_ctx* ctx, void* kv_pool, const sw_batch* hb, const void* h_q, const void* h_k_new,
                                   const void* h_v_new, void* h_out, float* h_lse, void* stream) {
     sw_status st = SW_OK;
@@ -454,26 +620,35 @@ sw_status sw_mixed_iteration_host(sw_ctx* ctx, void* kv_pool, const sw_batch* hb
     const size_t kv_bytes = (size_t)rows * l.num_kv_heads * l.head_dim * 2;
     uint8_t* ws = ctx->ws;
     int32_t* d_pages = reinterpret_cast<int32_t*>(ws + ctx->w.st_pages);
-    int32_t* d_len = d_pages;                         // [n]
-    int32_t* d_indptr = d_len + ctx->max_decode;      // [n+1]
-    int32_t* d_dec_pages = d_indptr + ctx->max_decode + 2;
-    int32_t* d_pf_pages = d_dec_pages + n_dec_pages;
+    HostTables t;                                     // [n], [n+1], then the page lists
+    t.len = d_pages;
+    t.indptr = t.len + ctx->max_decode;
+    t.dec_pages = t.indptr + ctx->max_decode + 2;
+    t.pf_pages = t.dec_pages + n_dec_pages;
+    sw_batch db = *hb;
+    db.prefill_pages = t.pf_pages;
+    db.decode_kv_len = t.len;
+    db.decode_page_indptr = t.indptr;
+    db.decode_pages = t.dec_pages;
+    Chunks checked;
+    if (check_batch(ctx, &db, "sw_mixed_iteration_run", &checked) == SW_OK && check_current_device(ctx, "sw_mixed_iteration_run") == SW_OK) {
+        const int per = host_part_rows(ctx, hb, hch, q_bytes + 2 * kv_bytes);
+        if (per > 0) {
+            st = make_host_streams(ctx);
+            if (st != SW_OK) return st;
+            st = iterate_parts(ctx, kv_pool, hb, hch, per, t, n_dec_pages, h_q, h_k_new, h_v_new, h_out, h_lse, s);
+            // (after an error too: nothing may still be reading or writing the caller's buffers)
+            const cudaError_t e[2] = {cudaStreamSynchronize(s), cudaStreamSynchronize(ctx->copies)};
+            if (st != SW_OK) return st;
+            for (cudaError_t x : e) SW_CUDA(x);
+            return SW_OK;
+        }
+    }
     SW_CUDA(cudaMemcpyAsync(ws + ctx->w.st_q, h_q, q_bytes, cudaMemcpyHostToDevice, s));
     SW_CUDA(cudaMemcpyAsync(ws + ctx->w.st_k, h_k_new, kv_bytes, cudaMemcpyHostToDevice, s));
     SW_CUDA(cudaMemcpyAsync(ws + ctx->w.st_v, h_v_new, kv_bytes, cudaMemcpyHostToDevice, s));
-    if (n > 0) {
-        SW_CUDA(cudaMemcpyAsync(d_len, hb->decode_kv_len, (size_t)n * 4, cudaMemcpyHostToDevice, s));
-        SW_CUDA(cudaMemcpyAsync(d_indptr, hb->decode_page_indptr, (size_t)(n + 1) * 4, cudaMemcpyHostToDevice, s));
-        if (n_dec_pages > 0)
-            SW_CUDA(cudaMemcpyAsync(d_dec_pages, hb->decode_pages, (size_t)n_dec_pages * 4, cudaMemcpyHostToDevice, s));
-    }
-    if (hb->num_prefill_pages > 0)
-        SW_CUDA(cudaMemcpyAsync(d_pf_pages, hb->prefill_pages, (size_t)hb->num_prefill_pages * 4, cudaMemcpyHostToDevice, s));
-    sw_batch db = *hb;
-    db.prefill_pages = d_pf_pages;
-    db.decode_kv_len = d_len;
-    db.decode_page_indptr = d_indptr;
-    db.decode_pages = d_dec_pages;
+    st = copy_tables(hb, t, n_dec_pages, s);
+    if (st != SW_OK) return st;
     float* d_lse = h_lse ? reinterpret_cast<float*>(ws + ctx->w.st_lse) : nullptr;
     st = sw_mixed_iteration_run(ctx, kv_pool, &db, ws + ctx->w.st_k, ws + ctx->w.st_v, ws + ctx->w.st_q, ws + ctx->w.st_out,
                                 d_lse, stream);
