@@ -951,6 +951,7 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
         late.us = kLateBaseUs + p.step_us * ((pplan.longest + pplan.pieces - 1) / pplan.pieces);
         if (pplan.n_items >= pplan.ctas)  // whole rounds: the prefill CTAs share all items' steps
             late.us = kLateBaseUs + p.step_us * (0.5f * (float)(pplan.longest + pplan.shortest) * (float)pplan.n_items / (float)pplan.ctas);
+        if (kMulti && pplan.end_steps > 0) late.us = kLateBaseUs + p.step_us * (float)pplan.end_steps;
         const int first_entry = blockIdx.x;
         if (first_entry < prefill_ctas) {  // CTA-uniform: this CTA has prefill work
             if (warp == 1) {

@@ -45,7 +45,7 @@ enum PfBar {
 constexpr int kPfRegsLaunch = 168, kPfRegsLight = 72, kPfRegsHeavy = 216;
 
 constexpr int kChunkTable = 88;  // ints into the CTA's scratch: P[8], C[8], first row[8], page-list offset[8], pieces[8] of the chunks
-constexpr int kChunkTotals = 7 * 8;  // ints into the table: the plan's totals, after seven fields of eight chunks
+constexpr int kChunkTotals = 8 * 8;  // ints into the table: the plan's totals, after eight fields of eight chunks
 
 struct PfShared {
     uint32_t smem;    // 1024-aligned shared address of the tile region
@@ -111,6 +111,7 @@ constexpr float kEntryCostSteps = 3.f;        // fill and drain of an entry, in 
 constexpr float kEntrySafety = 1.25f;
 constexpr int kPfMinRoundPieceSteps = 24;  // pieces that run in several rounds: at least this many KV steps each
 constexpr int kPfMaxRoundPieces = 12;
+constexpr int kSearchMinSteps = 64;        // several chunks: shortest plan (steps of its longest entry) for which piece lengths are tried
 
 struct PfPlan {
     int longest, shortest;             // steps of the longest and of the shortest item (items are numbered chunk by chunk)
@@ -119,6 +120,7 @@ struct PfPlan {
     int pieces;         // k: pieces per tail item (1 = tail items are whole too); several chunks: of the first chunk's
     int n_entries;      // n_whole + (n_items - n_whole) * k; several chunks: every chunk's tail items times its own k
     int ctas;           // CTAs that take entries (the first ones by index); the others start with decode units
+    int end_steps;      // several chunks: estimated end of the entries in steps where their lengths were searched (else 0)
     uint32_t table;     // several chunks: shared address of the chunk table (k of chunk j is field 4)
 };
 
@@ -162,6 +164,15 @@ __device__ __forceinline__ int pf_pieces_for(int steps) {
     return max(1, min(k, steps / kPfMinPieceSteps));
 }
 
+// pieces of an item of `steps` steps when pieces are to have about `per` steps
+__device__ __forceinline__ int pf_pieces_of_length(int steps, int per) {
+    return max(1, min((steps + per - 1) / per, steps / kPfMinPieceSteps));
+}
+// steps that a piece costs when an item is cut into k: its own, fill and drain, and its share of the merge
+__device__ __forceinline__ int pf_piece_steps(int steps, int k) {
+    return (steps + k - 1) / k + (int)kEntryCostSteps + (k > 1 ? 2 + k / 2 : 0);
+}
+
 // CTAs that take chunk-prefill entries when n_items items of wp steps in all run beside the decode requests (the
 // others start with decode units); G when the plain order is kept.
 __device__ __forceinline__ int pf_entry_ctas(const MixedParams& p, int G, int n_items, float wp, float decode_steps) {
@@ -191,7 +202,7 @@ __device__ __forceinline__ float pf_decode_steps(const MixedParams& p) {  // the
 // count, sized by its shortest item; while the tail entries outnumber the CTAs, the chunk with the shortest pieces
 // gives one up.  G: CTAs that take entries.  Run by one whole warp, lane j owning chunk j; fills the chunk table:
 // fields 0-3 the descriptors, 4 pieces per tail item, 5 items before the chunk, 6 tail entries before the chunk's
-// tail items (fields 5 and 6 hold INT_MAX where nothing may match), then the plan's totals.
+// tail items (fields 5 and 6 hold INT_MAX where nothing may match), 7 scratch slots before them, then the plan's totals.
 __device__ __forceinline__ void pf_fill_chunk_table(const MixedParams& p, int* tbl, int G) {
     const int lane = threadIdx.x & 31;
     int P = 0, C = 0, row0 = 0, page0 = 0;
@@ -222,8 +233,8 @@ __device__ __forceinline__ void pf_fill_chunk_table(const MixedParams& p, int* t
         shortest = pf_steps_of_rank(p.group, P, C, n_tp, n_tp - 1);
     }
     const int steps2 = __reduce_add_sync(0xffffffffu, n_tp > 0 ? (longest + shortest) * cnt : 0);
-    const int n_whole = n_items - n_items % G;
-    const int tail = max(0, before + cnt - max(before, n_whole));
+    int n_whole = n_items - n_items % G;
+    int tail = max(0, before + cnt - max(before, n_whole));
     int k = tail > 0 ? pf_pieces_for(shortest) : 1;
     int total = __reduce_add_sync(0xffffffffu, tail * k);
     while (total > G) {  // warp-uniform
@@ -233,7 +244,48 @@ __device__ __forceinline__ void pf_fill_chunk_table(const MixedParams& p, int* t
         if (key == best) k -= 1;
         total -= __shfl_sync(0xffffffffu, tail, best & 31);
     }
+    // When the longest entry ends, in steps.  Where that is far off, because one chunk's items are much longer than the others' and
+    // are whole entries or cut too little, every chunk's items are cut instead: lane l tries pieces of its own length (4, 5, 6, ...
+    // growing by a sixth; the last lane leaves every item whole) for all chunks and estimates when the last one ends.  There may
+    // be more pieces than CTAs, as long as the partial results of those that are cut fit the scratch.
+    // 300 tokens at prefix 60000 with 1064 at prefix 0 beside 64 chats: 718 -> 400 us (40 items of 475 steps were whole entries); 21 at
+    // 78262 with 689 at 0 beside 4 decodes 152 -> 105 us; 256 at 28672 with 512 at 0 beside 64 chats 206 -> 195 us.  Below 64 steps the
+    // search (2 us) costs more than it finds.
+    int end = 0;
+    {
+        const int own = cnt == 0 ? 0 : max(cnt > tail ? longest + (int)kEntryCostSteps : 0, tail > 0 ? pf_piece_steps(longest, k) : 0);
+        const int plain = __reduce_max_sync(0xffffffffu, own);
+        if (plain >= kSearchMinSteps) {
+            int per = 1 << 20;
+            if (lane < 31) per = max(4 + lane, (int)(4.f * exp2f(0.23f * (float)lane)));
+            int entries = 0, slots = 0, longest_piece = 0;
+            float work = 0.f;
+#pragma unroll 1
+            for (int j = 0; j < p.nchunks; ++j) {
+                const int cj = __shfl_sync(0xffffffffu, cnt, j), lj = __shfl_sync(0xffffffffu, longest, j),
+                          sj = __shfl_sync(0xffffffffu, shortest, j);
+                const int kj = pf_pieces_of_length(sj, per);
+                entries += cj * kj;
+                slots += kj > 1 ? cj * kj : 0;
+                work += (float)cj * (0.5f * (float)(lj + sj) + (float)(kj * (pf_piece_steps(0, kj))));
+                longest_piece = max(longest_piece, pf_piece_steps(lj, kj));
+            }
+            int tried = entries <= G ? longest_piece : max(longest_piece, (int)(work / (float)G + 0.5f * (float)min(per, longest_piece)) + 1);
+            if (slots > p.pf_slots) tried = 0x3ffffff;
+            const int best = __reduce_min_sync(0xffffffffu, (min(tried, 0x3ffffff) << 5) | lane);
+            const int per_best = __shfl_sync(0xffffffffu, per, best & 31);
+            if ((best >> 5) < plain - plain / 8) {
+                end = best >> 5;
+                n_whole = 0;
+                tail = cnt;
+                k = cnt > 0 ? pf_pieces_of_length(shortest, per_best) : 1;
+                total = __reduce_add_sync(0xffffffffu, tail * k);
+            }
+        }
+    }
     const int acc = scan(tail * k) - tail * k;
+    const int cut = k > 1 ? tail * k : 0;
+    const int slot_acc = scan(cut) - cut;
     longest = __reduce_max_sync(0xffffffffu, longest);
     shortest = __reduce_min_sync(0xffffffffu, shortest);
     const int k0 = __shfl_sync(0xffffffffu, k, 0);
@@ -245,6 +297,7 @@ __device__ __forceinline__ void pf_fill_chunk_table(const MixedParams& p, int* t
         tbl[4 * kMaxChunks + lane] = k;
         tbl[5 * kMaxChunks + lane] = live ? before : 0x7fffffff;
         tbl[6 * kMaxChunks + lane] = tail > 0 ? acc : 0x7fffffff;
+        tbl[7 * kMaxChunks + lane] = slot_acc;
     }
     if (lane == 0) {
         int* tot = tbl + kChunkTotals;
@@ -256,6 +309,7 @@ __device__ __forceinline__ void pf_fill_chunk_table(const MixedParams& p, int* t
         tot[5] = n_whole == 0 ? k0 : 1;
         tot[6] = G;
         tot[7] = steps2;
+        tot[8] = end;
     }
 }
 // Beside enough decode pages a few CTAs take no entry (the rule of the single-chunk plan; pieces in one round here): how many do, for
@@ -353,6 +407,7 @@ __device__ __forceinline__ void pf_fill_plan(const MixedParams& p, int* tbl) {
         tot[4] = plan.shortest;
         tot[5] = plan.pieces;
         tot[6] = plan.ctas;
+        tot[8] = 0;
     }
 }
 
@@ -367,6 +422,7 @@ __device__ __forceinline__ PfPlan pf_make_plan(uint32_t table) {  // worked out 
     plan.shortest = lds_s32(tot + 16);
     plan.pieces = lds_s32(tot + 20);
     plan.ctas = lds_s32(tot + 24);
+    plan.end_steps = lds_s32(tot + 32);
     return plan;
 }
 
@@ -409,7 +465,7 @@ __device__ __forceinline__ PfItem pf_entry(const MixedParams& p, const PfPlan& p
             const int idx = rel / it.pieces;
             it.item = max(before, plan.n_whole) + idx;
             it.piece = rel - idx * it.pieces;
-            it.slot0 = key - it.piece;
+            it.slot0 = lds_s32(col + 7 * kMaxChunks * 4) + idx * it.pieces;
         }
     }
     const int local = it.item - before;
