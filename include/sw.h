@@ -122,9 +122,10 @@ sw_status sw_mixed_attn_run(sw_ctx* ctx, const void* kv_pool, const sw_batch* ba
                             float* lse, void* stream);
 
 /* KV manager step and executor step of one iteration in ONE kernel launch: what sw_kv_append followed by
- * sw_mixed_attn_run computes, without the second launch and the gap between the two.  Every CTA of the persistent
- * grid first writes its share of the k_new / v_new rows into the pool; the chunk-prefill tiles that reach into the
- * chunk's own keys and the decode units that reach a request's last page wait (bounded) until every CTA has done so.
+ * sw_mixed_attn_run computes, without the second launch and the gap between the two.  In iterations with chunks every CTA of
+ * the persistent grid first writes its share of the k_new / v_new rows into the pool; the chunk-prefill tiles that reach into
+ * the chunk's own keys and the decode units that reach a request's last page wait (bounded) until every CTA has done so.  In
+ * decode-only iterations the units that reach a request's last page write its row.
  * Arguments as for the two calls.  Contract beyond theirs: no page of a decode request other than its last, and no
  * page below the chunk's first row, is written by this call (true of any page table in which requests own their
  * pages, shared prompt prefixes included).  Asynchronous.
@@ -135,7 +136,9 @@ sw_status sw_mixed_iteration_run(sw_ctx* ctx, void* kv_pool, const sw_batch* bat
                                  const void* q, void* out, float* lse, void* stream);
 
 /* The same iteration from HOST buffers: copies q / k_new / v_new and the page tables to the device (into the
- * workspace), runs sw_mixed_iteration_run, copies `out` (and lse if non-NULL) back and waits.
+ * workspace), runs sw_mixed_iteration_run, copies `out` (and lse if non-NULL) back and waits.  Iterations with 4 MB of inputs
+ * or more may be run in parts (decode rows, runs of chunk rows), copies on a stream of the context beside the launches on
+ * `stream`; the copies start after the work that is already on `stream`.
  * All pointers inside `h_batch` and h_q / h_k_new / h_v_new / h_out / h_lse are HOST pointers (pinned memory
  * makes the copies asynchronous); kv_pool stays a device pointer. */
 sw_status sw_mixed_iteration_host(sw_ctx* ctx, void* kv_pool, const sw_batch* h_batch, const void* h_q,

@@ -94,7 +94,7 @@ struct sw_ctx {
     };
     std::vector<MapEntry> kv_maps;  // small cache: one entry per pool of a layer stack
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-    // host-buffer iterations in parts: the copies' stream and events, made by the first call that uses them
+    // host-buffer iterations in parts: the copies' stream and events
     cudaStream_t copies = nullptr;
     cudaEvent_t ev_start = nullptr, ev_up = nullptr, ev_done[kHostParts + 1] = {};   // the last one: the decode rows
 };
@@ -210,6 +210,17 @@ sw_status check_batch(const sw_ctx* ctx, const sw_batch* b, const char* who, Chu
 
 }  // namespace
 
+namespace {
+sw_status make_copy_stream(sw_ctx* ctx) {
+    SW_CUDA(cudaStreamCreateWithFlags(&ctx->copies, cudaStreamNonBlocking));
+    SW_CUDA(cudaEventCreateWithFlags(&ctx->ev_start, cudaEventDisableTiming));
+    SW_CUDA(cudaEventCreateWithFlags(&ctx->ev_up, cudaEventDisableTiming));
+    for (cudaEvent_t& e : ctx->ev_done)
+        SW_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    return SW_OK;
+}
+}  // namespace
+
 extern "C" {
 
 size_t sw_workspace_bytes(const sw_layout* layout, int32_t max_chunk, int32_t max_decode, int64_t max_pages) {
@@ -282,6 +293,13 @@ sw_status sw_create(const sw_layout* layout, int device, void* workspace, size_t
     if (e != cudaSuccess) {
         delete ctx;
         return sw_fail(SW_ERR_CUDA, "sw_create: device set-up failed: %s", cudaGetErrorString(e));
+    }
+    if (max_pages > 0) {   // the context may take host-buffer iterations (0.1 ms here rather than in the first of them)
+        const sw_status st = make_copy_stream(ctx);
+        if (st != SW_OK) {
+            sw_destroy(ctx);
+            return st;
+        }
     }
     *out = ctx;
     return SW_OK;
@@ -497,15 +515,6 @@ int host_part_rows(const sw_ctx* ctx, const sw_batch* hb, const Chunks& ch, size
     }
 }
 
-sw_status make_host_streams(sw_ctx* ctx) {
-    if (!ctx->copies) SW_CUDA(cudaStreamCreateWithFlags(&ctx->copies, cudaStreamNonBlocking));
-    if (!ctx->ev_start) SW_CUDA(cudaEventCreateWithFlags(&ctx->ev_start, cudaEventDisableTiming));
-    if (!ctx->ev_up) SW_CUDA(cudaEventCreateWithFlags(&ctx->ev_up, cudaEventDisableTiming));
-    for (cudaEvent_t& e : ctx->ev_done)
-        if (!e) SW_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    return SW_OK;
-}
-
 // The host-buffer iteration in parts: the decode rows, then the chunk rows in runs of `per` consecutive rows (a chunk cut at a row
 // is the same attention: the rows behind the cut have a longer prefix).  While a part computes, the next one's inputs are on their way.
 sw_status iterate_parts(sw_ctx* ctx, void* kv_pool, const sw_batch* hb, const Chunks& ch, int per, const HostTables& t,
@@ -633,9 +642,7 @@ sw_status sw_mixed_iteration_host(sw_ctx* ctx, void* kv_pool, const sw_batch* hb
     Chunks checked;
     if (check_batch(ctx, &db, "sw_mixed_iteration_run", &checked) == SW_OK && check_current_device(ctx, "sw_mixed_iteration_run") == SW_OK) {
         const int per = host_part_rows(ctx, hb, hch, q_bytes + 2 * kv_bytes);
-        if (per > 0) {
-            st = make_host_streams(ctx);
-            if (st != SW_OK) return st;
+        if (per > 0 && ctx->copies) {
             st = iterate_parts(ctx, kv_pool, hb, hch, per, t, n_dec_pages, h_q, h_k_new, h_v_new, h_out, h_lse, s);
             // (after an error too: nothing may still be reading or writing the caller's buffers)
             const cudaError_t e[2] = {cudaStreamSynchronize(s), cudaStreamSynchronize(ctx->copies)};
