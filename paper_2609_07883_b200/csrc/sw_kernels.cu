@@ -1021,7 +1021,7 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
         const int fixed_items = ((int)gridDim.x - prefill_ctas) * kWarps;  // units handed out without the counter
         // with two unit sizes the early CTAs run their one large unit each and leave the counter to the late CTAs
         const bool pulls = !plan.two_sizes || (int)blockIdx.x < prefill_ctas;
-        const bool resident = prefill_ctas == 0 && plan.total_items <= fixed_items;
+        const bool resident = plan.total_items <= fixed_items;   // every unit has a warp of its own in a CTA that started with units
         // neighbouring units go to different SMs: a batch with fewer units than warps is spread over all of them
         int item = warp * ((int)gridDim.x - prefill_ctas) + (int)blockIdx.x - prefill_ctas;
         if ((int)blockIdx.x < prefill_ctas) {

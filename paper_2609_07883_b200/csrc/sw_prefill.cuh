@@ -250,7 +250,7 @@ __device__ __forceinline__ void pf_fill_chunk_table(const MixedParams& p, int* t
     // be more pieces than CTAs, as long as the partial results of those that are cut fit the scratch.
     // 300 tokens at prefix 60000 with 1064 at prefix 0 beside 64 chats: 718 -> 400 us (40 items of 475 steps were whole entries); 21 at
     // 78262 with 689 at 0 beside 4 decodes 152 -> 105 us; 256 at 28672 with 512 at 0 beside 64 chats 206 -> 195 us.  Below 64 steps the
-    // search (2 us) costs more than it finds.
+    // search (2 us) costs more than it finds, and the estimate has to promise a quarter: it does not see the decode phase.
     int end = 0;
     {
         const int own = cnt == 0 ? 0 : max(cnt > tail ? longest + (int)kEntryCostSteps : 0, tail > 0 ? pf_piece_steps(longest, k) : 0);
@@ -274,7 +274,7 @@ __device__ __forceinline__ void pf_fill_chunk_table(const MixedParams& p, int* t
             if (slots > p.pf_slots) tried = 0x3ffffff;
             const int best = __reduce_min_sync(0xffffffffu, (min(tried, 0x3ffffff) << 5) | lane);
             const int per_best = __shfl_sync(0xffffffffu, per, best & 31);
-            if ((best >> 5) < plain - plain / 8) {
+            if ((best >> 5) < plain - plain / 4) {
                 end = best >> 5;
                 n_whole = 0;
                 tail = cnt;
