@@ -240,7 +240,12 @@ __device__ __forceinline__ int plan_split_pages(const MixedParams& p, int total_
     const int rounds = one_round <= kOneRoundMaxPages ? 1 : (one_round <= 160 ? 2 : 4);
     int units_target = max(1, rounds * warps_per_head - p.n);
     units_target = min(units_target, max(1, p.target_items / p.Hkv));
-    return max((total_pages + units_target - 1) / units_target, kMinSplitTokens / kPageSize);
+    // Where the batch is at most 16 stages per SM its time is the chain of a unit's pages, and units of half the smallest size
+    // are faster although more of them are merged: one 1024-token context 14.8 -> 12.5 us, one of 4096 16.0 -> 14.9, four of 256-2048
+    // 15.6 -> 13.9 (8192 tokens, 28 stages per SM: 18.3 -> 20.1); not for contexts of a few pages, which would be split for
+    // nothing (200 of 16-100 tokens 11.3 -> 12.3).
+    const bool small = (int64_t)total_pages * p.Hkv <= 16 * (int64_t)gridDim.x && total_pages >= 5 * p.n;
+    return max((total_pages + units_target - 1) / units_target, kMinSplitTokens / kPageSize / (small ? 2 : 1));
 }
 
 // CTAs that start with chunk-prefill work turn to decode units later than the others.
