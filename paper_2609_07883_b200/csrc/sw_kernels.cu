@@ -515,13 +515,15 @@ __device__ __forceinline__ void patch_row(uint32_t buf, int slot, uint4 v) {
 }
 __device__ __forceinline__ unsigned page_hash(int page) { return ((unsigned)page * 2654435761u) >> 21; }
 static_assert(kPageHashBits == 1 << (32 - 21), "the hash has as many values as there are buckets");
-// All new rows of the page in buffer `buf`, the last one of request i.  `lists`: shared address of the plan region.
+// All new rows of the page in buffer `buf`, the last one of request i.  A request whose last page lies outside the pool has id -1 in
+// the list and reads page 0: it shares that page with nobody.  (Requests of length 0 and less have id -1 too, and no row at all: a
+// search for -1 would find them and write in front of the buffer.)
 template <int D>
 __device__ __forceinline__ void patch_page(const MixedParams& p, uint32_t smem, uint32_t buf, int i, int kvh, int valid, uint4 own) {
     const int lane = threadIdx.x & 31;
     const int page = lds_s32(smem + Geo<D>::kLastOffset + i * 4);
     const unsigned h = page_hash(page);
-    const bool several = lds_s32(smem + Geo<D>::kSharedOffset + (kPageHashBits + h) / 32 * 4) >> (h & 31) & 1;
+    const bool several = page >= 0 && (lds_s32(smem + Geo<D>::kSharedOffset + (kPageHashBits + h) / 32 * 4) >> (h & 31) & 1);
 #pragma unroll 1
     for (int j0 = 0; several && j0 < p.n; j0 += 32) {
         const int j = j0 + lane;

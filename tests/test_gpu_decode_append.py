@@ -60,3 +60,38 @@ def test_a_bad_last_page_is_reported_and_nothing_is_written(oracle):
         r.dbatch = r.B.DeviceBatch(batch, r.dev)               # the context is usable afterwards
         r.iterate()
         assert r.status() == (0, 0)
+
+
+@pytest.mark.parametrize("heads", [(32, 8, 128), (16, 4, 64), (4, 4, 64)])
+@pytest.mark.parametrize("empty_len", [0, -1, -14, -(1 << 31)])
+def test_bad_last_pages_beside_requests_without_a_row(oracle, heads, empty_len):
+    """Requests whose last page lies outside the pool and requests of length 0 or less in one batch, in either order: both are
+    reported, and every other request's output and row are what they are without them."""
+    shape = W.AttnShape(*heads)
+    rng = np.random.default_rng(23)
+    lens = [40, 33, 7, 300, 16, 95, 1, 20, 50]
+    base = W.make_batch(shape, sum(-(-x // 16) for x in lens) + 3, lens, 0, 0, rng)
+    t = W.host_tensors(base, rng)
+    broken_page, broken_len = (0, 4, 7), (1, 3, 8)
+    bad = W.MixedBatch(**{**base.__dict__})
+    bad.decode_pages = base.decode_pages.copy()
+    bad.decode_kv_len = base.decode_kv_len.copy()
+    for i in broken_page:
+        bad.decode_pages[bad.decode_page_indptr[i] + (lens[i] - 1) // 16] = -1 if i else bad.num_pages
+    for i in broken_len:
+        bad.decode_kv_len[i] = empty_len
+    good = [i for i in range(len(lens)) if i not in broken_page + broken_len]
+    keep = W.MixedBatch(**{**base.__dict__})
+    keep.decode_kv_len = base.decode_kv_len[good]
+    keep.decode_pages = np.concatenate([base.decode_pages[base.decode_page_indptr[i]:base.decode_page_indptr[i + 1]] for i in good])
+    keep.decode_page_indptr = np.concatenate([[0], np.cumsum([-(-lens[i] // 16) for i in good])]).astype(np.int32)
+    pool = t["pool"].copy()
+    assert oracle.kv_append(pool, keep, t["k_new"][good], t["v_new"][good]) == 0
+    ref, ref_lse, _ = oracle.mixed_attention(pool, keep, t["q"][good])
+    r = G.Runner(bad, t)
+    for _ in range(2):
+        r.iterate()
+        assert r.status()[0] == r.B.SW_ERR_OUT_OF_RANGE
+        out, lse = r.results()
+        assert np.array_equal(G.torch_to_bits(r.pool), pool)
+        G.compare(out[good].reshape(-1, shape.head_dim), lse[good].reshape(-1), ref, ref_lse, f"{heads} {empty_len}")
