@@ -478,14 +478,16 @@ sw_status copy_tables(const sw_batch* hb, const HostTables& t, int64_t n_dec_pag
     return SW_OK;
 }
 
-// Whether a page that chunk rows are written to is also the last page of a decode request (then a decode row and chunk rows may
-// attend each other, and the iteration is not taken apart).
-bool chunks_meet_decodes(const sw_batch* hb, const Chunks& ch) {
+// Whether two parts of the iteration would meet on a page: one that rows of two chunks are written to (tokens of one prompt, say; the
+// second chunk may attend the first one's rows of that page), or chunk rows and a decode request's last row.  Such an iteration is not
+// taken apart, since every row is written before anything is attended.
+bool parts_share_a_page(const sw_batch* hb, const Chunks& ch) {
     std::vector<int32_t> written;
     for (int j = 0; j < ch.n; ++j)
         for (int64_t pi = ch.P[j] / sw::kPageSize; pi <= ((int64_t)ch.P[j] + ch.C[j] - 1) / sw::kPageSize; ++pi)
             written.push_back(hb->prefill_pages[ch.page0[j] + pi]);
     std::sort(written.begin(), written.end());
+    if (std::adjacent_find(written.begin(), written.end()) != written.end()) return true;
     for (int i = 0; i < hb->num_decode; ++i) {
         const int pages = (int)(((int64_t)hb->decode_kv_len[i] + sw::kPageSize - 1) / sw::kPageSize);
         const int beg = hb->decode_page_indptr[i], end = hb->decode_page_indptr[i + 1];
@@ -498,18 +500,18 @@ bool chunks_meet_decodes(const sw_batch* hb, const Chunks& ch) {
 // Chunk rows of a part of a host-buffer iteration (0: it is run whole).  Parts are whole 256-row groups.  Where the chunks'
 // arithmetic (at 1.2 PFLOP/s) takes longer than the way up (at 46 GB/s), parts of fewer work items than there are SMs would cost
 // more than they hide.
-int host_part_rows(const sw_ctx* ctx, const sw_batch* hb, const Chunks& ch, size_t up_bytes) {
-    const sw_layout& l = ctx->layout;
+int host_part_rows(const sw_layout& l, int num_sms, const sw_batch* hb, const Chunks& ch) {
+    const size_t up_bytes = ((size_t)ch.rows + hb->num_decode) * (l.num_q_heads + 2 * l.num_kv_heads) * l.head_dim * 2;
     if (ch.rows == 0 || up_bytes < kHostPartBytes) return 0;
     const int group_rows = 256 / (l.num_q_heads / l.num_kv_heads);
     int groups = ((ch.rows + kHostParts - 1) / kHostParts + group_rows - 1) / group_rows;
     double pairs = 0.;   // attended (query, key) pairs
     for (int j = 0; j < ch.n; ++j) pairs += (double)ch.C[j] * ((double)ch.P[j] + 0.5 * (double)ch.C[j]);
     if (pairs * 4. * l.num_q_heads * l.head_dim / 1.2e15 > (double)up_bytes / 46e9)
-        groups = std::max(groups, ctx->num_sms / l.num_kv_heads);
+        groups = std::max(groups, num_sms / l.num_kv_heads);
     if (groups * group_rows >= ch.rows) return 0;
     try {
-        return chunks_meet_decodes(hb, ch) ? 0 : groups * group_rows;
+        return parts_share_a_page(hb, ch) ? 0 : groups * group_rows;
     } catch (...) {
         return 0;   // no host memory for the comparison
     }
@@ -641,7 +643,7 @@ sw_status sw_mixed_iteration_host(sw_ctx* ctx, void* kv_pool, const sw_batch* hb
     db.decode_pages = t.dec_pages;
     Chunks checked;
     if (check_batch(ctx, &db, "sw_mixed_iteration_run", &checked) == SW_OK && check_current_device(ctx, "sw_mixed_iteration_run") == SW_OK) {
-        const int per = host_part_rows(ctx, hb, hch, q_bytes + 2 * kv_bytes);
+        const int per = host_part_rows(ctx->layout, ctx->num_sms, hb, hch);
         if (per > 0 && ctx->copies) {
             st = iterate_parts(ctx, kv_pool, hb, hch, per, t, n_dec_pages, h_q, h_k_new, h_v_new, h_out, h_lse, s);
             // (after an error too: nothing may still be reading or writing the caller's buffers)
@@ -664,6 +666,12 @@ sw_status sw_mixed_iteration_host(sw_ctx* ctx, void* kv_pool, const sw_batch* hb
     if (h_lse) SW_CUDA(cudaMemcpyAsync(h_lse, d_lse, (size_t)rows * l.num_q_heads * 4, cudaMemcpyDeviceToHost, s));
     SW_CUDA(cudaStreamSynchronize(s));
     return SW_OK;
+}
+
+int sw_host_part_rows_of(const sw_layout* layout, int32_t num_sms, const sw_batch* hb) {
+    Chunks ch;
+    if (!layout || !hb || !layout_supported(*layout) || chunks_of(hb, "sw_host_part_rows_of", &ch) != SW_OK) return -1;
+    return host_part_rows(*layout, num_sms, hb, ch);
 }
 
 namespace {

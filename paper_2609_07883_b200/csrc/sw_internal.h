@@ -156,3 +156,7 @@ cudaError_t launch_selftest_wait(int32_t* ctrl, long long budget_cycles, cudaStr
 size_t mixed_attn_smem_bytes(int head_dim);
 
 }  // namespace sw
+
+// Not part of the ABI: the chunk rows that sw_mixed_iteration_host would give a part of this host batch on a device of num_sms SMs (0: the
+// iteration is run whole; -1: no valid batch).  Host arithmetic only; the tests look at it.
+extern "C" int sw_host_part_rows_of(const sw_layout* layout, int32_t num_sms, const sw_batch* h_batch);

@@ -30,10 +30,12 @@ def run_host(oracle, batch, pinned, with_lse, seed, rng):
         q, k, v, out, lse = (t.pin_memory() for t in (q, k, v, out, lse))
     hs, keep = B.host_batch_struct(batch)
     before = G.torch_to_bits(pool)
-    for _ in range(2):    # again on the same context: events and streams are kept
+    results = []
+    for _ in range(2):    # the first pass finds other rows in the pool; again on the same context: events and streams are kept
         out.zero_()
         B.sw_mixed_iteration_host(ctx, pool, hs, q, k, v, out, lse if with_lse else None)
         assert B.sw_check_status(ctx, raise_on_error=False) == (0, 0)
+        results.append((W.bf16_bits_to_f64(G.torch_to_bits(out)), lse.numpy().astype(np.float64)))
     want = before.copy()
     rows = 0
     if batch.chunk_lens is None:
@@ -49,7 +51,6 @@ def run_host(oracle, batch, pinned, with_lse, seed, rng):
                            batch.decode_pages)
         assert oracle.kv_append(want, dec, G.torch_to_bits(k[rows:]), G.torch_to_bits(v[rows:])) == 0
     assert np.array_equal(G.torch_to_bits(pool), want)
-    got, got_lse = W.bf16_bits_to_f64(G.torch_to_bits(out)), lse.numpy().astype(np.float64)
     # chunk by chunk (the oracle takes one), rows around the parts' edges and a few others, one head each
     edges = {r + d for r in range(0, batch.chunk_len, 64) for d in (-1, 0)} | set(range(batch.chunk_len, R))
     at = 0
@@ -64,7 +65,8 @@ def run_host(oracle, batch, pinned, with_lse, seed, rng):
         pairs = np.array([(r, int(rng.integers(sh.num_q_heads))) for r in take], dtype=np.int32)
         ref, ref_lse, _ = oracle.mixed_attention(want, one, G.torch_to_bits(q[at:at + C + n]), pairs=pairs)
         rr = pairs[:, 0] + at
-        G.compare(got[rr, pairs[:, 1]], got_lse[rr, pairs[:, 1]] if with_lse else None, ref, ref_lse, f"host parts, chunk {j}")
+        for got, got_lse in results:
+            G.compare(got[rr, pairs[:, 1]], got_lse[rr, pairs[:, 1]] if with_lse else None, ref, ref_lse, f"host parts, chunk {j}")
         at += C
 
 
@@ -96,3 +98,18 @@ def test_a_decode_row_on_a_page_of_the_chunk(oracle):
     batch.decode_kv_len = np.array([6 * 16 + 5], dtype=np.int32)   # its row is in slot 4 of that page
     batch.decode_page_indptr = np.array([0, 7], dtype=np.int32)
     run_host(oracle, batch, True, True, 92, rng)
+
+
+def two_chunks_of_one_prompt(rng, decode_lens=(300, 40)):
+    """Two chunks of one prompt whose rows meet on a page: 500 tokens at prefix 100, listed first, and the four tokens before them."""
+    one = W.make_batch(W.LLAMA, 200, decode_lens, 100, 500, rng)
+    n = one.prefill_pages.shape[0]
+    return W.MixedBatch(**{**one.__dict__, "chunk_len": 504, "prefill_pages": np.concatenate([one.prefill_pages, one.prefill_pages[:7]]),
+                           "chunk_prefix_lens": np.array([100, 96], np.int32), "chunk_lens": np.array([500, 4], np.int32),
+                           "chunk_page_indptr": np.array([0, n, n + 7], np.int32)})
+
+
+def test_chunks_that_share_a_page(oracle):
+    """The rows of the second chunk are attended by the first one's, whichever part those are in."""
+    rng = np.random.default_rng(4)
+    run_host(oracle, two_chunks_of_one_prompt(rng), True, True, 93, rng)
