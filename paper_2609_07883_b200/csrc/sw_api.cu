@@ -621,6 +621,8 @@ sw_status sw_mixed_iteration_host(sw_ctx* ctx, void* kv_pool, const sw_batch* hb
     const int n = hb->num_decode;
     if (n > 0 && (!hb->decode_kv_len || !hb->decode_page_indptr || !hb->decode_pages))
         return sw_fail(SW_ERR_INVALID_ARG, "sw_mixed_iteration_host: decode arrays missing");
+    if (hb->num_prefill_pages > 0 && !hb->prefill_pages)   // (the lists are also read here, see parts_share_a_page)
+        return sw_fail(SW_ERR_INVALID_ARG, "sw_mixed_iteration_host: prefill page list missing");
     const int64_t n_dec_pages = n > 0 ? hb->decode_page_indptr[n] : 0;
     if (n_dec_pages < 0 || n_dec_pages + hb->num_prefill_pages > ctx->max_pages)
         return sw_fail(SW_ERR_WORKSPACE, "sw_mixed_iteration_host: %lld page-table entries exceed max_pages %lld",

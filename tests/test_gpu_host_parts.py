@@ -113,3 +113,23 @@ def test_chunks_that_share_a_page(oracle):
     """The rows of the second chunk are attended by the first one's, whichever part those are in."""
     rng = np.random.default_rng(4)
     run_host(oracle, two_chunks_of_one_prompt(rng), True, True, 93, rng)
+
+
+@pytest.mark.parametrize("tokens", [40, 500])    # run whole, taken apart
+def test_a_missing_page_list_is_refused(tokens):
+    import torch
+
+    from paper_2609_07883_b200 import binding as B
+
+    batch = W.make_batch(W.LLAMA, 64, [], 0, tokens, np.random.default_rng(1))
+    ctx = B.Context(W.LLAMA, 64, tokens, 1, 64)
+    pool = torch.zeros(64 * W.LLAMA.page_elems, dtype=torch.bfloat16, device="cuda")
+    q, k, v, out = (torch.zeros(tokens, h, 128, dtype=torch.bfloat16) for h in (32, 8, 8, 32))
+    struct, keep = B.host_batch_struct(batch)
+    struct.prefill_pages = None
+    with pytest.raises(B.SwError) as e:
+        B.sw_mixed_iteration_host(ctx, pool, struct, q, k, v, out)
+    assert e.value.status == B.SW_ERR_INVALID_ARG
+    struct, keep = B.host_batch_struct(batch)         # the context is usable afterwards
+    B.sw_mixed_iteration_host(ctx, pool, struct, q, k, v, out)
+    assert B.sw_check_status(ctx, raise_on_error=False) == (0, 0)
