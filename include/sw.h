@@ -129,9 +129,12 @@ sw_status sw_mixed_attn_run(sw_ctx* ctx, const void* kv_pool, const sw_batch* ba
  * Arguments as for the two calls.  Contract beyond theirs: no page of a decode request other than its last, and no
  * page below the chunk's first row, is written by this call (true of any page table in which requests own their
  * pages, shared prompt prefixes included).  Asynchronous.
- * The waits need every CTA of the persistent grid to be resident at once.  sw_create checks that (occupancy of the
- * kernel times the SM count against the grid); on a device where it does not hold this call issues the append as a
- * launch of its own before the attention launch, with the same results. */
+ * The waits for the append (iterations with chunks) need every CTA of the persistent grid to be resident at once.  sw_create
+ * checks that (occupancy of the kernel times the SM count against the grid); on a device where it does not hold this
+ * call issues the append as a launch of its own before the attention launch, with the same results.  It cannot see what
+ * else will run: beside kernels that hold SMs for a second or more (launches of another context on another stream, waiting in the
+ * same way, among them) use sw_kv_append and sw_mixed_attn_run.  Those, decode-only iterations and sw_decode_attn_static
+ * wait for no CTA that has not started. */
 sw_status sw_mixed_iteration_run(sw_ctx* ctx, void* kv_pool, const sw_batch* batch, const void* k_new, const void* v_new,
                                  const void* q, void* out, float* lse, void* stream);
 

@@ -65,8 +65,8 @@ struct MixedParams {
     bool append_last;    // decode-only launches: a request's new row is written by the units that reach its last page
     // scratch
     int32_t* ctrl;
-    int32_t* tickets;   // [max_decode * Hkv]: order in which the units of a (request, kv head) near their end
-    int32_t* ready;     // [max_decode * Hkv]: how many of them have published their partial result
+    int32_t* tickets;   // [max_decode * Hkv]: order in which the units of a (request, kv head) near their end; shared merges: units started
+    int32_t* ready;     // [max_decode * Hkv]: how many of them have published their partial result (and more, see rows_to_merge)
     float* part_ml;     // [max_items][2 * kMaxGroup]  (m then l per query head of the group)
     float* part_o;      // [max_items][group * D]
     int max_items;      // partial-result slots available

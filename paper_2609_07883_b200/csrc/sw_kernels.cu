@@ -7,7 +7,8 @@
 //                           the context lengths; a warp's first unit is fixed by its index, further ones come from a
 //                           shared counter; a unit streams its K/V pages with TMA into the warp's shared-memory ring
 //                           and keeps an online softmax in registers; of the units of one (request, kv head) the one
-//                           that drew the last ticket merges the partial results.
+//                           that drew the last ticket merges the partial results or, where there are many, the last
+//                           ones one query-head row each.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -545,6 +546,40 @@ __device__ __forceinline__ void patch_page(const MixedParams& p, uint32_t smem, 
     __syncwarp();
 }
 
+// Shared merges (requests cut into many units): the calling unit, whose partial result is written, publishes it and learns which
+// query-head rows it has to merge, as a bit mask (0: none; -1: the bounded wait expired).  One lane calls it.  merge_row: the unit's
+// own row, -1 if it has none.
+//
+// A merger may only wait for units that run: one that has not started may be waiting for this merger's SM (another kernel can
+// hold an SM for as long as it likes, and two launches of this one can each hold a part of the SMs), or for its warp.  So every
+// unit counts itself in `started` when it begins, and a merger that finds units missing hands its row over and leaves; the unit
+// that publishes last, after which nobody has to wait, merges the rows that were handed over before.
+// `ready`: the low half counts the units that have published and then, once those are all, the rows that are merged; bit 16 + r:
+// row r is handed over.
+constexpr int kPublished = 0xffff;
+constexpr long long kPatienceCycles = 20000;   // ten microseconds: the CTAs of a launch start within two or three of each other
+__device__ __forceinline__ int rows_to_merge(int32_t* ready, const int32_t* started, int nsplit, int merge_row) {
+    const int own = merge_row < 0 ? 0 : 1 << merge_row;
+    const int before = atomicAdd(ready, 1);
+    if ((before & kPublished) == nsplit - 1) {
+        __threadfence();
+        return own | before >> 16;
+    }
+    if (own == 0) return 0;
+    const long long t0 = clock64();
+    while ((ld_acquire_gpu(ready) & kPublished) < nsplit) {
+        const long long waited = clock64() - t0;
+        if (waited > kWaitBudgetCycles) return -1;
+        if (waited > kPatienceCycles && ld_relaxed_gpu(started) < nsplit) {
+            if ((atomicOr(ready, own << 16) & kPublished) < nsplit) return 0;
+            __threadfence();   // the others have started and published meanwhile: the last one did not see it
+            return own;
+        }
+        __nanosleep(64);
+    }
+    return own;
+}
+
 // Runs one unit; returns false if a bounded wait expired.
 //
 // The products are transposed: the 16 rows of an mma.m16n8k16 are keys (of S = K Q^T) or output columns (of O^T = V^T P^T) and
@@ -616,14 +651,13 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
     // round trip hides behind the last pages, and no warp hoards a unit while others are still idle.
     // With the claim the unit draws its ticket among the units of its (request, kv head): the last ticket makes it
     // the one that merges.  Both answers are read at the end of the unit, when they have long arrived.
-    // A request cut into many units (kWideMergeSplits or more) has g mergers per kv head, fixed in advance: its last g
-    // units, one query-head row each (units of one request and head are Hkv apart in the order in which SMs take them, so
-    // the mergers sit on different SMs).  Such a unit will wait for the request's other units, so it must not hold a
-    // claimed unit meanwhile (another merger could be waiting for that one): it claims its next unit after the merge.
-    // Where every unit of the launch has a warp of its own (`resident`) nobody can wait for a unit that nobody runs, and the merge
-    // is shared as soon as there are g units.
+    // A request cut into many units (kWideMergeSplits or more; g where every unit of the launch has a warp of its own, `resident`)
+    // has g mergers per kv head, fixed in advance: its last g units, one query-head row each (units of one request and head are
+    // Hkv apart in the order in which SMs take them, so the mergers sit on different SMs).  They claim their next unit after
+    // the merge.  What they wait for: see rows_to_merge.
     const bool wide = g > 1 && u.nsplit >= (resident ? g : kWideMergeSplits);
     const int merge_row = wide && u.nsplit - 1 - u.split < g ? u.nsplit - 1 - u.split : -1;
+    if (wide && lane == 0) atomicAdd(&p.tickets[u.ticket], 1);   // started
     bool claimed = merge_row >= 0;
     int ticket = 0;  // lane 0
     auto claim_next = [&]() {
@@ -792,34 +826,24 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
     if (wide) {
         // Many splits (one long context cut for all the warps): a single warp would load their partial outputs a few
         // at a time.  Every unit publishes its partial result; g of the request's last units then merge one row of
-        // the group each.  A waiting merger holds no claimed unit, and the units it waits for are run by warps that wait
-        // for nothing or are claimed by such warps: a request has 24 units or more only if it holds 23 units' worth
-        // of pages, so at most target_items / 23 (request, kv head) pairs have mergers, fewer than 1500 warps even
-        // with groups of 8, and some warp is always free to claim.  The last merger to finish re-arms the counter.
+        // the group each.  The last merger to finish re-arms the counters.
         __threadfence();
         __syncwarp();
-        if (lane == 0) atomicAdd(&p.ready[u.ticket], 1);
-        if (merge_row < 0) return true;
-        int ok = 1;
-        if (lane == 0) {
-            const long long t0 = clock64();
-            while (ld_acquire_gpu(&p.ready[u.ticket]) < u.nsplit) {
-                if (clock64() - t0 > kWaitBudgetCycles) {
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(64);
-            }
-        }
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        if (!ok) {
+        int rows = 0;
+        if (lane == 0) rows = rows_to_merge(&p.ready[u.ticket], &p.tickets[u.ticket], u.nsplit, merge_row);
+        rows = __shfl_sync(0xffffffffu, rows, 0);
+        if (rows < 0) {
             if (lane == 0) report(p.ctrl, SW_ERR_DEVICE_TIMEOUT, kSiteWait, u.q_row);
             return false;
         }
-        merge_splits<D, 1, 16>(p, u, merge_row, 1);
+        const int merged = __popc(rows);
+        for (; rows != 0; rows &= rows - 1) merge_splits<D, 1, 16>(p, u, __ffs(rows) - 1, 1);
         if (lane == 0) {
-            if (atomicAdd(&p.ready[u.ticket], 1) == u.nsplit + g - 1) p.ready[u.ticket] = 0;  // ready for the next launch
-            next_item = pulls ? fixed_items + atomicAdd(work, 1) : 0x7fffffff;
+            if (merged > 0 && (atomicAdd(&p.ready[u.ticket], merged) & kPublished) + merged == u.nsplit + g) {
+                p.ready[u.ticket] = 0;      // ready for the next launch
+                p.tickets[u.ticket] = 0;
+            }
+            if (merge_row >= 0) next_item = pulls ? fixed_items + atomicAdd(work, 1) : 0x7fffffff;
         }
         return true;
     }
@@ -1026,9 +1050,10 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
         ring.bar = base + Geo<D>::kBarOffset + warp * Geo<D>::kStages * 8;
         ring.it = 0;
         const int fixed_items = ((int)gridDim.x - prefill_ctas) * kWarps;  // units handed out without the counter
-        // with two unit sizes the early CTAs run their one large unit each and leave the counter to the late CTAs
-        const bool pulls = !plan.two_sizes || (int)blockIdx.x < prefill_ctas;
-        const bool resident = plan.total_items <= fixed_items;   // every unit has a warp of its own in a CTA that started with units
+        const bool resident = plan.total_items <= fixed_items;   // every unit has a warp of its own in a CTA that starts with units
+        // With two unit sizes the early CTAs run their one large unit each and leave the counter to the late CTAs; where every unit
+        // has a warp of its own the counter has none to give (asking it costs a merger 0.7 us at its end).
+        const bool pulls = !resident && (!plan.two_sizes || (int)blockIdx.x < prefill_ctas);
         // neighbouring units go to different SMs: a batch with fewer units than warps is spread over all of them
         int item = warp * ((int)gridDim.x - prefill_ctas) + (int)blockIdx.x - prefill_ctas;
         if ((int)blockIdx.x < prefill_ctas) {
