@@ -29,9 +29,11 @@ __device__ __forceinline__ void report(int32_t* ctrl, int code, int site, int in
 // ---------------------------------------------------------------------------------------------------------------
 // KV append
 // ---------------------------------------------------------------------------------------------------------------
-// A warp takes 32 of the 16-byte pieces of a row's Hkv*D elements, of K and of V, kAppendBatch times at once: what the append
-// costs is its chain of latencies (position, page id, row, store), not its bytes.  `first` and `stride` spread the pieces over
-// the calling warps.  (One piece per thread and pass, with 64-bit divisions, took 7.6-11 us of a launch with 2048 chunk rows.)
+// A warp takes 32 of the 16-byte pieces of a row's Hkv*D elements (of several rows where a row has fewer), of K and of V, and
+// kAppendBatch times as many at once: what the append costs is its chain of latencies (position, page id, row, store), not its
+// bytes.  `first` and `stride` spread the pieces over the calling warps.  (One piece per thread and pass, with 64-bit divisions,
+// took 7.6-11 us of a launch with 2048 chunk rows.  With one row per warp, 8192 rows of 16 pieces made the fused launch of 8/2/64
+// 151 us and that of 8/1/128 156 instead of 139 and 148.)
 // (P is AppendParams or MixedParams: the fields have the same names; every index into the chunk arrays is a
 // compile-time constant so that the kernel parameters stay in constant memory.)
 constexpr int kAppendBatch = 4;
@@ -40,7 +42,8 @@ __device__ __forceinline__ void append_rows(const P& p, int head_dim, int first,
     const int lane = threadIdx.x & 31;
     const int pieces_per_row = p.Hkv * head_dim / 8;
     const int per_row = (pieces_per_row + 31) / 32;   // warp-wide parts of a row
-    const int total = (p.C + p.n) * per_row;
+    const int rows_at_once = max(1, 32 / pieces_per_row), sub = lane / pieces_per_row, sub_lane = lane - sub * pieces_per_row;
+    const int rows = p.C + p.n, total = (rows + rows_at_once - 1) / rows_at_once * per_row;
 #pragma unroll 1
     for (int c0 = first; c0 < total; c0 += kAppendBatch * stride) {
         uint4 k[kAppendBatch], v[kAppendBatch];
@@ -50,12 +53,11 @@ __device__ __forceinline__ void append_rows(const P& p, int head_dim, int first,
             const int c = c0 + b * stride;
             slot[b] = -1;
             if (c >= total) break;
-            const int row = c / per_row, piece = (c - row * per_row) * 32 + lane;
-            if (piece < pieces_per_row) {
-                const int64_t src = ((int64_t)row * pieces_per_row + piece) * 8;
-                k[b] = *reinterpret_cast<const uint4*>(p.k_new + src);
-                v[b] = *reinterpret_cast<const uint4*>(p.v_new + src);
-            }
+            const int part = c / per_row, row = part * rows_at_once + sub, piece = (c - part * per_row) * 32 + sub_lane;
+            if (piece >= pieces_per_row || sub >= rows_at_once || row >= rows) continue;
+            const int64_t src = ((int64_t)row * pieces_per_row + piece) * 8;
+            k[b] = *reinterpret_cast<const uint4*>(p.k_new + src);
+            v[b] = *reinterpret_cast<const uint4*>(p.v_new + src);
             unsigned pos;
             const int32_t* pages;
             int npages;
@@ -93,10 +95,10 @@ __device__ __forceinline__ void append_rows(const P& p, int head_dim, int first,
         for (int b = 0; b < kAppendBatch; ++b) {
             const int c = c0 + b * stride;
             if (c >= total) break;
-            const int row = c / per_row, e0 = ((c - row * per_row) * 32 + lane) * 8;   // element offset inside the row's [Hkv][D]
-            if (slot[b] < 0 || e0 >= pieces_per_row * 8) continue;
+            if (slot[b] < 0) continue;
+            const int part = c / per_row, e0 = ((c - part * per_row) * 32 + sub_lane) * 8;   // element offset inside the row's [Hkv][D]
             if (page[b] < 0 || page[b] >= p.num_pages) {
-                report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAppendPage, row);
+                report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAppendPage, part * rows_at_once + sub);
                 continue;
             }
             const int64_t block = ((int64_t)page[b] * 2 * p.Hkv + e0 / head_dim) * kPageSize + slot[b];   // K; V is Hkv blocks further
@@ -115,7 +117,8 @@ __global__ void sw_kv_append_kernel(const AppendParams p) {
 }
 
 cudaError_t launch_kv_append(const AppendParams& p, int num_sms, cudaStream_t stream) {
-    const int64_t total = (int64_t)(p.C + p.n) * ((p.Hkv * p.D / 8 + 31) / 32);   // warp-wide parts of rows
+    const int pieces_per_row = p.Hkv * p.D / 8, rows_at_once = pieces_per_row < 32 ? 32 / pieces_per_row : 1;
+    const int64_t total = (int64_t)((p.C + p.n + rows_at_once - 1) / rows_at_once) * ((pieces_per_row + 31) / 32);   // warp-wide parts
     if (total == 0) return cudaSuccess;
     const int threads = 256;
     int64_t blocks = (total + threads / 32 - 1) / (threads / 32);
