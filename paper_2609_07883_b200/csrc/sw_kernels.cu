@@ -36,8 +36,8 @@ __device__ __forceinline__ void report(int32_t* ctrl, int code, int site, int in
 // 151 us and that of 8/1/128 156 instead of 139 and 148.)
 // (P is AppendParams or MixedParams: the fields have the same names; every index into the chunk arrays is a
 // compile-time constant so that the kernel parameters stay in constant memory.)
-constexpr int kAppendBatch = 4;
-template <bool kMulti, class P>
+constexpr int kAppendBatch = 4;   // in the fused launch, with 11 warps an SM; the stand-alone kernel has 64 of one part each
+template <bool kMulti, int kBatch, class P>
 __device__ __forceinline__ void append_rows(const P& p, int head_dim, int first, int stride) {
     const int lane = threadIdx.x & 31;
     const int pieces_per_row = p.Hkv * head_dim / 8;
@@ -45,11 +45,11 @@ __device__ __forceinline__ void append_rows(const P& p, int head_dim, int first,
     const int rows_at_once = max(1, 32 / pieces_per_row), sub = lane / pieces_per_row, sub_lane = lane - sub * pieces_per_row;
     const int rows = p.C + p.n, total = (rows + rows_at_once - 1) / rows_at_once * per_row;
 #pragma unroll 1
-    for (int c0 = first; c0 < total; c0 += kAppendBatch * stride) {
-        uint4 k[kAppendBatch], v[kAppendBatch];
-        int page[kAppendBatch], slot[kAppendBatch];   // slot: -1 = no such position in the list (reported)
+    for (int c0 = first; c0 < total; c0 += kBatch * stride) {
+        uint4 k[kBatch], v[kBatch];
+        int page[kBatch], slot[kBatch];   // slot: -1 = no such position in the list (reported)
 #pragma unroll
-        for (int b = 0; b < kAppendBatch; ++b) {
+        for (int b = 0; b < kBatch; ++b) {
             const int c = c0 + b * stride;
             slot[b] = -1;
             if (c >= total) break;
@@ -92,7 +92,7 @@ __device__ __forceinline__ void append_rows(const P& p, int head_dim, int first,
             }
         }
 #pragma unroll
-        for (int b = 0; b < kAppendBatch; ++b) {
+        for (int b = 0; b < kBatch; ++b) {
             const int c = c0 + b * stride;
             if (c >= total) break;
             if (slot[b] < 0) continue;
@@ -108,21 +108,24 @@ __device__ __forceinline__ void append_rows(const P& p, int head_dim, int first,
     }
 }
 
-__global__ void sw_kv_append_kernel(const AppendParams p) {
+constexpr int kAppendThreads = 256, kAppendBlocksPerSm = 8;
+__global__ void __launch_bounds__(kAppendThreads, kAppendBlocksPerSm) sw_kv_append_kernel(const AppendParams p) {
     // launched with programmatic stream serialization: it may start while the previous kernel (the attention of
     // the previous iteration, possibly still reading this pool) drains; nothing is touched before this wait
     grid_launch_dependents();
     grid_dependency_wait();
-    append_rows<true>(p, p.D, (int)(blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32), (int)(gridDim.x * (blockDim.x / 32)));
+    append_rows<true, 1>(p, p.D, (int)(blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32), (int)(gridDim.x * (blockDim.x / 32)));
 }
 
 cudaError_t launch_kv_append(const AppendParams& p, int num_sms, cudaStream_t stream) {
     const int pieces_per_row = p.Hkv * p.D / 8, rows_at_once = pieces_per_row < 32 ? 32 / pieces_per_row : 1;
     const int64_t total = (int64_t)((p.C + p.n + rows_at_once - 1) / rows_at_once) * ((pieces_per_row + 31) / 32);   // warp-wide parts
     if (total == 0) return cudaSuccess;
-    const int threads = 256;
+    const int threads = kAppendThreads;
     int64_t blocks = (total + threads / 32 - 1) / (threads / 32);
-    if (blocks > (int64_t)num_sms * 8) blocks = (int64_t)num_sms * 8;   // eight 256-thread blocks fill an SM
+    // The grid is resident at once, so that the launch after this one is released at once too.  (With four parts a warp a thread has
+    // 64 registers and half the blocks wait: 3000 rows of 32/8/128 5.5 -> 6.3 us, 8192 12.2 -> 14.1.)
+    if (blocks > (int64_t)num_sms * kAppendBlocksPerSm) blocks = (int64_t)num_sms * kAppendBlocksPerSm;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3(threads);
@@ -965,7 +968,7 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
     if (p.append_first) {
         // fused launch with chunks: this CTA's share of the new K/V rows (the planning warp has none), then its mark on the
         // counter the readers wait for
-        if (warp != 2) append_rows<kMulti>(p, D, (int)blockIdx.x * (kWarps - 1) + warp - (warp > 2), (int)gridDim.x * (kWarps - 1));
+        if (warp != 2) append_rows<kMulti, kAppendBatch>(p, D, (int)blockIdx.x * (kWarps - 1) + warp - (warp > 2), (int)gridDim.x * (kWarps - 1));
         fence_proxy_async_global();
         __threadfence();
         __syncthreads();
