@@ -1,0 +1,34 @@
+"""Decode contexts around the edges of the split and of the merge: numbers of units that fill, miss and exceed a batch of the merge."""
+import numpy as np
+import pytest
+
+from paper_2609_07883_b200 import workloads as W
+from tests import gpu_util as G
+
+pytestmark = pytest.mark.gpu
+
+
+def run(oracle, heads, lens, what, fused=True):
+    rng = np.random.default_rng(51)
+    shape = W.AttnShape(*heads)
+    batch = W.make_batch(shape, sum(-(-x // 16) for x in lens) + 3, lens, 0, 0, rng)
+    t = W.host_tensors(batch, rng)
+    pool = t["pool"].copy()
+    assert oracle.kv_append(pool, batch, t["k_new"], t["v_new"]) == 0
+    ref, ref_lse, _ = oracle.mixed_attention(pool, batch, t["q"])
+    r = G.Runner(batch, t)
+    for _ in range(2):
+        if fused:
+            r.iterate()
+        else:
+            r.append()
+            r.attend()
+        assert r.status() == (0, 0)
+        out, lse = r.results()
+        G.compare(out.reshape(-1, shape.head_dim), lse.reshape(-1), ref, ref_lse, what)
+
+
+@pytest.mark.parametrize("heads", [(4, 4, 64), (2, 2, 128), (4, 2, 64), (8, 2, 128), (8, 1, 64)])
+def test_numbers_of_splits_around_a_batch_of_the_merge(oracle, heads):
+    for splits in (2, 7, 8, 9, 15, 16, 17, 31, 32, 33):   # units of 64 tokens
+        run(oracle, heads, [64 * splits - 3], f"{heads}, {splits} splits")
