@@ -381,6 +381,7 @@ sw_status run_mixed(sw_ctx* ctx, void* kv_pool, const sw_batch* batch, const voi
     p.step_us = ctx->step_us;
     p.stages_per_us = 1.f / ctx->stage_us;
     p.steps_per_stage = ctx->stage_us / ctx->step_us;
+    sw::small_batch_limits(batch->num_decode, l.num_kv_heads, ctx->num_sms, &p.small_from, &p.small_to);
     p.C = ch.rows;
     p.n = batch->num_decode;
     p.nchunks = ch.n;

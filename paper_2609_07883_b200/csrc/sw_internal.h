@@ -42,6 +42,7 @@ struct MixedParams {
     // (page, kv head) stage of K and V, and microseconds of one 128-key step of a chunk-prefill entry
     float stage_us, step_us;
     float stages_per_us, steps_per_stage;   // 1 / stage_us and stage_us / step_us, worked out on the host
+    int small_from, small_to;   // pages of the decode requests between which a batch may be cut into units of half the smallest size
     // batch.  C is the number of chunk rows of the iteration: the rows of its prefill chunks, one chunk after the
     // other.  Chunk j has cC[j] tokens at prefix cP[j], starts at row cRow0[j] and its prompt's page list starts at
     // prefill_pages[cPage0[j]] (cPage0[nchunks] = num_prefill_pages).
@@ -146,6 +147,11 @@ inline void device_timing(int mem_clock_khz, int bus_width_bits, int sm_clock_kh
     const double stage_bytes = 2.0 * kPageSize * head_dim * 2;   // K and V rows of one head in a page
     *stage_us = (float)(stage_bytes / bytes_per_us);
     *step_us = (float)(4300.0 / ((double)sm_clock_khz / 1e3));
+}
+// MixedParams::small_from / small_to: more than eight pages a request (four, up to four requests), at most 16 stages per CTA.
+inline void small_batch_limits(int num_decode, int num_kv_heads, int num_ctas, int* from, int* to) {
+    *from = 8 * num_decode - (num_decode < 5 ? 4 : 0) + 1;
+    *to = 16 * num_ctas / num_kv_heads;
 }
 cudaError_t launch_mixed_attn(int head_dim, const KvMaps& kv_maps, const CUtensorMap& q_map, const CUtensorMap& out_map,
                               const MixedParams& p,

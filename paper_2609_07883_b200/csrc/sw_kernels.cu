@@ -238,20 +238,23 @@ __device__ __forceinline__ int block_sum(int v, int* ctr) {
     return *reinterpret_cast<volatile int*>(ctr);
 }
 
+constexpr int kLongPages = 512;   // from this many pages on a context is not cut into units of half the smallest size
 // One-class unit size: pages per unit when `warps_per_head` warps share `total_pages`.  Small batches are
 // latency-bound: one round of units, as many as there are warps, gets every warp streaming at once.  Large batches are
 // bandwidth-bound: a few rounds of smaller units shorten the tail.  Every request adds at most one ragged unit per
 // head, hence the "- n".
-__device__ __forceinline__ int plan_split_pages(const MixedParams& p, int total_pages, int warps_per_head) {
+__device__ __forceinline__ int plan_split_pages(const MixedParams& p, int total_pages, bool any_long, int warps_per_head) {
     const int one_round = (total_pages + warps_per_head - 1) / warps_per_head;  // pages per unit if run in one round
     const int rounds = one_round <= kOneRoundMaxPages ? 1 : (one_round <= 160 ? 2 : 4);
     int units_target = max(1, rounds * warps_per_head - p.n);
     units_target = min(units_target, max(1, p.target_items / p.Hkv));
     // Where the batch is at most 16 stages per SM its time is the chain of a unit's pages, and units of half the smallest size
     // are faster although more of them are merged: one 1024-token context 14.8 -> 12.5 us, one of 4096 16.0 -> 14.9, four of 256-2048
-    // 15.6 -> 13.9 (8192 tokens, 28 stages per SM: 18.3 -> 20.1); not for contexts of a few pages, which would be split for
-    // nothing (200 of 16-100 tokens 11.3 -> 12.3).
-    const bool small = (int64_t)total_pages * p.Hkv <= 16 * (int64_t)gridDim.x && total_pages >= 5 * p.n;
+    // 15.6 -> 13.9 (8192 tokens, 28 stages per SM: 18.3 -> 20.1).  Not for contexts of up to eight pages (one unit of the usual
+    // size, which needs no merge), unless there are four of them or fewer: 32 of 81 tokens, 8/2/64, 12.3 us split and 10.6 whole, one
+    // of 128, 32/8/128, 10.6 and 12.2.  And not where a context would be cut into 128 units or more, whose merge is the longer chain: one
+    // of 32768 tokens, 8/1/128, 33.5 us and 25.8, one of 16384, 8/2/64, 21.9 and 19.7 (8192: 17.0 and 16.8).
+    const bool small = total_pages >= p.small_from && total_pages <= p.small_to && !any_long;
     return max((total_pages + units_target - 1) / units_target, kMinSplitTokens / kPageSize / (small ? 2 : 1));
 }
 
@@ -282,22 +285,28 @@ __device__ __forceinline__ Plan make_plan(const MixedParams& p, int* unit_prefix
     const int end = min(p.n, beg + per_thread);
     // total context in pages (fits an int: n <= 2048 requests of < 2^27 pages)
     int pages_local = 0;
+    bool long_local = false;
     for (int i = beg; i < end; ++i) {
         const int len = p.decode_kv_len[i];
-        pages_local += len > 0 ? (len + kPageSize - 1) / kPageSize : 0;
+        const int pg = len > 0 ? (len + kPageSize - 1) / kPageSize : 0;
+        pages_local += pg;
+        long_local |= pg >= kLongPages;
         len_s[i] = len;                              // the units read these from shared memory later
         indptr_s[i] = p.decode_page_indptr[i];
     }
     if (threadIdx.x == 0 && p.n > 0) indptr_s[p.n] = p.decode_page_indptr[p.n];
     int* ctr = scratch + 64;  // kPlanCounters counters zeroed in the kernel prologue, one per block sum
-    const int total_pages = block_sum(pages_local, ctr++);
+    const int warp_pages = __reduce_add_sync(0xffffffffu, pages_local);
+    if ((threadIdx.x & 31) == 0 && warp_pages != 0) atomicAdd(ctr, warp_pages);
+    const bool any_long = __syncthreads_or(long_local);   // (the barrier of the sum, see block_sum)
+    const int total_pages = *reinterpret_cast<volatile int*>(ctr++);
 
     const int G = (int)gridDim.x;
     constexpr int kMinPages = kMinSplitTokens / kPageSize;
     int split_a = 0, split_b = 0;  // pages per unit of the first requests / of the rest
     int a_pages = 0x7fffffff;      // requests whose pages start below this (per head) are cut with split_a
     if (late.ctas <= 0 || late.ctas >= G) {
-        split_a = split_b = plan_split_pages(p, total_pages, max(1, G * kWarps / p.Hkv));
+        split_a = split_b = plan_split_pages(p, total_pages, any_long, max(1, G * kWarps / p.Hkv));
     } else {
         const float early = (float)((G - late.ctas) * kWarps), all = (float)(G * kWarps);
         const float pages = (float)total_pages * p.Hkv;
@@ -312,12 +321,12 @@ __device__ __forceinline__ Plan make_plan(const MixedParams& p, int* unit_prefix
         if (G - late.ctas < kMinEarlyCtas || late.ctas < kMinLateCtas || streamed < 0.25f * pages) {
             // Too few early CTAs to keep the memory system busy on their own (the estimate of what they stream would
             // not hold), or a head start that is small next to the whole phase: one unit size, every warp pulls.
-            split_a = split_b = plan_split_pages(p, total_pages, max(1, G * kWarps / p.Hkv));
+            split_a = split_b = plan_split_pages(p, total_pages, any_long, max(1, G * kWarps / p.Hkv));
         } else if (pages - streamed < (float)(late.ctas * kWarps * kMinPages)) {
-            split_a = split_b = plan_split_pages(p, total_pages, max(1, (G - late.ctas) * kWarps / p.Hkv));
+            split_a = split_b = plan_split_pages(p, total_pages, any_long, max(1, (G - late.ctas) * kWarps / p.Hkv));
         } else if (a_ragged > 0.25f * a_units || b_ragged > 0.25f * b_units) {
             // too many requests per warp for one even unit each: units pulled by every warp balance better
-            split_a = split_b = plan_split_pages(p, total_pages, max(1, G * kWarps / p.Hkv));
+            split_a = split_b = plan_split_pages(p, total_pages, any_long, max(1, G * kWarps / p.Hkv));
         } else {
             split_a = max(kMinPages, (int)ceilf(a_share / (a_units - a_ragged)));
             split_b = max(kMinPages, (int)ceilf(b_share / (b_units - b_ragged)));

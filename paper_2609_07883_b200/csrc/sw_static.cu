@@ -139,6 +139,7 @@ extern "C" sw_status sw_decode_attn_static(const sw_layout* layout, int device, 
     sw::device_timing(st->mem_khz, st->bus_bits, st->sm_khz, l.head_dim, &p.stage_us, &p.step_us);
     p.stages_per_us = 1.f / p.stage_us;
     p.steps_per_stage = p.stage_us / p.step_us;
+    sw::small_batch_limits(batch->num_decode, l.num_kv_heads, st->num_sms, &p.small_from, &p.small_to);
     p.C = 0;
     p.n = batch->num_decode;
     p.decode_kv_len = batch->decode_kv_len;

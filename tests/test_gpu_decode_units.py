@@ -32,3 +32,13 @@ def run(oracle, heads, lens, what, fused=True):
 def test_numbers_of_splits_around_a_batch_of_the_merge(oracle, heads):
     for splits in (2, 7, 8, 9, 15, 16, 17, 31, 32, 33):   # units of 64 tokens
         run(oracle, heads, [64 * splits - 3], f"{heads}, {splits} splits")
+
+
+@pytest.mark.parametrize("heads,lens", [
+    ((8, 2, 64), [128] * 9), ((8, 2, 64), [128] * 8 + [129]),                      # eight pages a context, and one more
+    ((8, 1, 128), [128] * 4), ((8, 1, 128), [128] * 5), ((8, 1, 128), [112] * 4),  # four contexts or fewer
+    ((8, 1, 64), [511 * 16]), ((8, 1, 64), [511 * 16 + 1]), ((8, 1, 64), [20, 512 * 16 + 5, 3]),   # 128 units of four pages and more
+    ((4, 4, 64), [64]), ((4, 4, 64), [65]), ((4, 4, 64), [1, 1, 300]),
+])
+def test_contexts_at_the_edges_of_the_small_batch_rule(oracle, heads, lens):
+    run(oracle, heads, lens, f"{heads} {len(lens)} x {max(lens)}")
