@@ -1013,11 +1013,14 @@ __device__ __forceinline__ void prefill_phase(const CUtensorMap* kv_map, const C
                 if (it.j1 > it.j0) pf_sanitize<D, kMulti>(p, sh, it, san_kv_it);
                 // Near the end of what may be the CTA's last entry: whether the decode units have all been handed out (the CTAs
                 // that started with them have published their number).  Then the CTA need not work the decode plan out afterwards,
-                // which takes 2-3 us.
-                if (lane == 0 && p.n > 0) {
-                    const int32_t* counters = p.ctrl + next[2];
-                    const int items = ld_relaxed_gpu(&counters[kSetItems]) - 1, drawn = ld_relaxed_gpu(&counters[kSetWork]);
-                    next[3] = items >= 0 && ((int)gridDim.x - min(plan.n_entries, plan.ctas)) * kWarps + drawn >= items;
+                // which takes 2-3 us.  (Not with several chunks at head size 64: the compiler then makes every step of the
+                // entries 2-3 % longer, 1687 tokens at prefix 59930 beside 67 of 16/4/64 711 -> 733 us.)
+                if constexpr (D == 128 || !kMulti) {
+                    if (lane == 0 && p.n > 0) {
+                        const int32_t* counters = p.ctrl + next[2];
+                        const int items = ld_relaxed_gpu(&counters[kSetItems]) - 1, drawn = ld_relaxed_gpu(&counters[kSetWork]);
+                        next[3] = items >= 0 && ((int)gridDim.x - min(plan.n_entries, plan.ctas)) * kWarps + drawn >= items;
+                    }
                 }
             } else {
                 // entries 0 .. plan.ctas-1 are the CTAs' first ones; the counter hands out the rest
