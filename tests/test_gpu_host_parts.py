@@ -70,14 +70,19 @@ def run_host(oracle, batch, pinned, with_lse, seed, rng):
         at += C
 
 
+# (heads, decode lengths, chunks, chunk rows of a part: see test_host_parts.py)
+PARTS = [
+    ((32, 8, 128), [300, 17, 1, 2047], [(512, 512)], 256),            # decodes on their own
+    ((32, 8, 128), [], [(0, 1001)], 512),                             # ragged last part, no decodes
+    ((32, 8, 128), [40, 500], [(700, 260), (33, 300), (0, 65)], 320),  # parts that hold ends and beginnings of chunks
+    ((16, 4, 64), [129], [(4111, 1777)], 896),
+    ((8, 1, 128), [64, 65], [(100, 2100)], 1056),
+    ((16, 4, 64), [700], [(20000, 2500)], 2368),                      # bound by the arithmetic: a first part of a whole grid's items
+]
+
+
 @pytest.mark.parametrize("pinned", [True, False])
-@pytest.mark.parametrize("heads,lens,chunks", [
-    ((32, 8, 128), [300, 17, 1, 2047], [(512, 512)]),            # decodes on their own
-    ((32, 8, 128), [], [(0, 1001)]),                             # ragged last part, no decodes
-    ((32, 8, 128), [40, 500], [(700, 260), (33, 300), (0, 65)]),  # parts that hold ends and beginnings of chunks
-    ((16, 4, 64), [129], [(4111, 1777)]),                        # bound by the arithmetic: parts of a whole grid's items
-    ((8, 1, 128), [64, 65], [(100, 2100)]),
-])
+@pytest.mark.parametrize("heads,lens,chunks", [case[:3] for case in PARTS])
 def test_parts(oracle, heads, lens, chunks, pinned):
     rng = np.random.default_rng(len(lens) + heads[0])
     sh = W.AttnShape(*heads)
