@@ -336,7 +336,6 @@ sw_status sw_kv_append(sw_ctx* ctx, void* kv_pool, const sw_batch* batch, const 
     p.n = batch->num_decode;
     p.nchunks = ch.n;
     std::memcpy(p.cP, ch.P, sizeof p.cP);
-    std::memcpy(p.cC, ch.C, sizeof p.cC);
     std::memcpy(p.cRow0, ch.row0, sizeof p.cRow0);
     std::memcpy(p.cPage0, ch.page0, sizeof p.cPage0);
     p.prefill_pages = batch->prefill_pages;

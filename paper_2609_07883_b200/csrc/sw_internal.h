@@ -14,7 +14,7 @@ constexpr int kMaxDecode = 2048;        // decode requests per iteration (prefix
 constexpr int kThreads = 384;           // 12 warps per CTA, one CTA per SM
 constexpr int kWarps = kThreads / 32;
 constexpr int kTargetItems = 4096;      // split-KV units aimed at per launch (bounds the partial-result scratch)
-constexpr int kMinSplitTokens = 128;    // never split a decode context finer than this
+constexpr int kMinSplitTokens = 128;    // decode contexts are not split finer than this (small batches: half of it, plan_split_pages)
 constexpr int kMaxGroup = 8;            // query heads per KV head
 constexpr int kMaxCtas = 192;           // persistent CTAs (one per SM) the scratch is sized for
 constexpr int kPfRoundSlots = 3 * kMaxCtas;  // partial results of chunk-prefill pieces that run in several rounds
@@ -84,7 +84,7 @@ struct AppendParams {
     int64_t num_pages;
     int C, n;
     int nchunks;
-    int cP[kMaxChunks], cC[kMaxChunks], cRow0[kMaxChunks], cPage0[kMaxChunks + 1];
+    int cP[kMaxChunks], cRow0[kMaxChunks], cPage0[kMaxChunks + 1];
     const int32_t* prefill_pages;
     int num_prefill_pages;
     const int32_t* decode_kv_len;

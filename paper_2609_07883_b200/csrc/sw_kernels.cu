@@ -168,6 +168,11 @@ __device__ __forceinline__ bool wait_append(const MixedParams& p, uint32_t set_a
 // ---------------------------------------------------------------------------------------------------------------
 constexpr int kPageHashBits = 2048;   // buckets of the hash that tells pages with one writer from pages that may have several
 
+// Words of the CTA's scratch from kMiscAt on: TMEM base, abort flag, the two tiles' ticket flags, the next entries (two, by the parity
+// of the current one), where the launch's counters start (words into ctrl), and whether no decode unit is left for the CTA.
+constexpr int kMiscAt = 32;
+enum MiscWord { kMiscTmem = 0, kMiscAbort = 1, kMiscFlags = 2, kMiscNext = 5, kMiscSet = 7, kMiscNoUnits = 8 };
+
 template <int D>
 struct Geo {
     static constexpr int kHalves = D / 64;                    // 128-byte swizzled column blocks per row
@@ -183,7 +188,7 @@ struct Geo {
     static constexpr int kIndptrOffset = kLenOffset + kMaxDecode * 4;           // int32 page_indptr[kMaxDecode+1]
     static constexpr int kLastOffset = kIndptrOffset + (kMaxDecode + 1) * 4 + 12; // int32 id of request i's last page
     static constexpr int kMiscOffset = kLastOffset + kMaxDecode * 4;              // scan scratch, TMEM base, abort flag
-    static constexpr int kSetOffset = kMiscOffset + (32 + 7) * 4;                 // where this launch's counters start (words into ctrl)
+    static constexpr int kSetOffset = kMiscOffset + (kMiscAt + kMiscSet) * 4;      // where this launch's counters start (words into ctrl)
     static constexpr int kSharedOffset = kMiscOffset + 768;   // after 64 ints scan scratch and flags, the plan's counters, the chunk table:
     static constexpr int kSmemBytes = kSharedOffset + 2 * kPageHashBits / 8;      // two bit sets over hashed last pages
 };
@@ -202,8 +207,7 @@ struct Plan {
     const int* len;     // shared-memory copies of the context lengths and page-list offsets
     const int* indptr;
     bool two_sizes;     // large units handed out by index to the early CTAs, small ones pulled by the late CTAs only
-    int decode_units;   // units of all requests
-    int total_items;
+    int total_items;    // units of all requests, times the KV heads
 };
 
 // Block-wide exclusive scan of one value per thread (kThreads threads): a warp scan, one barrier, then every thread
@@ -375,7 +379,6 @@ __device__ __forceinline__ Plan make_plan(const MixedParams& p, int* unit_prefix
     }
     if (threadIdx.x == 0) unit_prefix[p.n] = total_units;
     __syncthreads();
-    plan.decode_units = total_units;
     plan.total_items = total_units * p.Hkv;
     return plan;
 }
@@ -419,8 +422,8 @@ __device__ __forceinline__ void issue_page(const CUtensorMap* kvp_map, const War
 // units share the merge).  J splits at a time: lane j fetches (m, l) of split j while all lanes fetch their four (two) columns
 // of the J partial outputs, so a merge of up to J splits costs one round trip to L2; it is the round trips (about a
 // microsecond each) that a merge consists of: with eight at a time instead of sixteen a 32768-token context of one query head per KV
-// head took 32.8 us per launch instead of 25.6 (4/4/64) and 43.8 instead of 38.1 (8/8/128).  G >= nrows is a compile-time bound: rows beyond the group read row 0 with
-// weight zero, which keeps the loops free of branches.  Slots of the splits are Hkv apart.
+// head took 32.8 us per launch instead of 25.6 (4/4/64) and 43.8 instead of 38.1 (8/8/128).  G >= nrows is a compile-time bound:
+// rows beyond the group read row 0 with weight zero, which keeps the loops free of branches.  Slots of the splits are Hkv apart.
 template <int D, int G, int J = (G >= 8 ? 2 : (G == 4 ? 4 : (G == 2 ? 8 : 16)))>
 __device__ __forceinline__ void merge_splits(const MixedParams& p, const Unit& u, int row0, int nrows) {
     constexpr int V = D / 32;                 // output columns per lane
@@ -924,7 +927,7 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
     int* scratch = reinterpret_cast<int*>(smem + Geo<D>::kMiscOffset);
 
     const bool tensor_prefill = p.C > 0;
-    volatile int* misc = reinterpret_cast<volatile int*>(scratch + 32);  // [0] TMEM base, [1] abort flag, [2..3] ticket flags, [5..6] next entry, [7] where this launch's counters start, [8] no units left
+    volatile int* misc = reinterpret_cast<volatile int*>(scratch + kMiscAt);
     if (threadIdx.x >= 32 && threadIdx.x < 32 + kPlanCounters) scratch[64 + threadIdx.x - 32] = 0;  // block-sum counters
     if (threadIdx.x < kWarps * Geo<D>::kStages) {
         mbar_init(base + Geo<D>::kBarOffset + threadIdx.x * 8, 1);
@@ -941,9 +944,9 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
             tma_prefetch_desc(&out_map);
             pf_init_barriers(base + Geo<D>::kPfBarOffset);
         }
-        misc[0] = 0;
-        misc[1] = 0;
-        misc[8] = 0;
+        misc[kMiscTmem] = 0;
+        misc[kMiscAbort] = 0;
+        misc[kMiscNoUnits] = 0;
         fence_mbar_init();
     }
     // The plan of the chunk-prefill phase and, with several chunks, their descriptors go to shared memory: the roles look them
@@ -962,7 +965,7 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
     // grid - 1 uses set 0, one that reads more uses set 1, and it clears the other one for the launch after it.
     const int set = ld_relaxed_gpu(&p.ctrl[kCtrArrived]) >= (int)gridDim.x ? 1 : 0;
     int32_t* counters = p.ctrl + kCtrSets + set * kSetWords;
-    if (threadIdx.x == 0) misc[7] = kCtrSets + set * kSetWords;
+    if (threadIdx.x == 0) misc[kMiscSet] = kCtrSets + set * kSetWords;
     if (blockIdx.x == 0 && threadIdx.x < kSetWords) p.ctrl[kCtrSets + (set ^ 1) * kSetWords + threadIdx.x] = 0;
     if (tensor_prefill && warp == 2) {
         if constexpr (kMulti) {
@@ -978,7 +981,8 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
     if (p.append_first) {
         // fused launch with chunks: this CTA's share of the new K/V rows (the planning warp has none), then its mark on the
         // counter the readers wait for
-        if (warp != 2) append_rows<kMulti, kAppendBatch>(p, D, (int)blockIdx.x * (kWarps - 1) + warp - (warp > 2), (int)gridDim.x * (kWarps - 1));
+        if (warp != 2)
+            append_rows<kMulti, kAppendBatch>(p, D, (int)blockIdx.x * (kWarps - 1) + warp - (warp > 2), (int)gridDim.x * (kWarps - 1));
         fence_proxy_async_global();
         __threadfence();
         __syncthreads();
@@ -1002,7 +1006,7 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
         const int first_entry = blockIdx.x;
         if (first_entry < prefill_ctas) {  // CTA-uniform: this CTA has prefill work
             if (warp == 1) {
-                tmem_alloc(smem_u32(const_cast<int*>(&misc[0])), 512);
+                tmem_alloc(smem_u32(const_cast<int*>(&misc[kMiscTmem])), 512);
                 tmem_relinquish();
             }
             tc_fence_before_sync();
@@ -1011,21 +1015,21 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
             PfShared sh;
             sh.smem = base;
             sh.bars = base + Geo<D>::kPfBarOffset;
-            sh.tmem = (uint32_t)misc[0];
-            sh.abort_flag = &misc[1];
+            sh.tmem = (uint32_t)misc[kMiscTmem];
+            sh.abort_flag = &misc[kMiscAbort];
             PfScratch scr;
             scr.ml = p.pf_ml;
             scr.o = p.pf_o;
             scr.tickets = p.pf_tickets;
-            scr.flags = &misc[2];
-            prefill_phase<D, kMulti>(&kv_map, &q_map, &out_map, p, sh, pplan, scr, first_entry, &misc[5]);
+            scr.flags = &misc[kMiscFlags];
+            prefill_phase<D, kMulti>(&kv_map, &q_map, &out_map, p, sh, pplan, scr, first_entry, &misc[kMiscNext]);
             tc_fence_before_sync();
             __syncthreads();
             if (warp == 1) tmem_dealloc(sh.tmem, 512);
         }
         __syncthreads();
     }
-    if (p.n == 0 || misc[8]) {   // no decode units, or none left for this CTA
+    if (p.n == 0 || misc[kMiscNoUnits]) {   // no decode units, or none left for this CTA
         if (threadIdx.x == 0) atomicInc(reinterpret_cast<unsigned*>(&p.ctrl[kCtrArrived]), 2 * gridDim.x - 1);
         return;
     }
@@ -1056,7 +1060,7 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
         __syncwarp();
         if (lane == 0) mbar_arrive(base + Geo<D>::kLastBarOffset);
     }
-    if ((int)blockIdx.x == prefill_ctas && threadIdx.x == 0) atomicExch(p.ctrl + misc[7] + kSetItems, plan.total_items + 1);
+    if ((int)blockIdx.x == prefill_ctas && threadIdx.x == 0) atomicExch(p.ctrl + misc[kMiscSet] + kSetItems, plan.total_items + 1);
     if (plan.total_items > p.max_items) {
         if (threadIdx.x == 0) report(p.ctrl, SW_ERR_WORKSPACE, kSiteScratch, plan.total_items);
     } else {
@@ -1139,6 +1143,8 @@ cudaError_t launch_selftest_wait(int32_t* ctrl, long long budget_cycles, cudaStr
     return cudaGetLastError();
 }
 
+// 226.7 KB at head size 128, 288 bytes below what a CTA may have
+static_assert(Geo<128>::kSmemBytes + 1024 <= 227 * 1024 && Geo<64>::kSmemBytes + 1024 <= 227 * 1024, "shared memory of a CTA");
 size_t mixed_attn_smem_bytes(int head_dim) {
     return (head_dim == 64 ? Geo<64>::kSmemBytes : Geo<128>::kSmemBytes) + 1024;
 }

@@ -979,8 +979,8 @@ __device__ __forceinline__ bool pf_softmax(const CUtensorMap* out_map, const Mix
 }
 
 // ---- the prefill phase of one CTA ----------------------------------------------------------------------------------
-// `next` points at two shared-memory ints (after them: where the launch's counters start, and whether no decode unit is left): the idle warp fetches the following entry from the global counter while
-// the current one is processed and leaves it in next[iteration parity]; everyone reads it after the piece barrier.
+// `next` points at the scratch words from kMiscNext on: the idle warp fetches the following entry from the global counter while the
+// current one is processed and leaves it in next[iteration parity]; everyone reads it after the piece barrier.
 template <int D, bool kMulti>
 __device__ __forceinline__ void prefill_phase(const CUtensorMap* kv_map, const CUtensorMap* q_map, const CUtensorMap* out_map,
                                               const MixedParams& p, const PfShared& sh, const PfPlan& plan,
@@ -1017,14 +1017,15 @@ __device__ __forceinline__ void prefill_phase(const CUtensorMap* kv_map, const C
                 // entries 2-3 % longer, 1687 tokens at prefix 59930 beside 67 of 16/4/64 711 -> 733 us.)
                 if constexpr (D == 128 || !kMulti) {
                     if (lane == 0 && p.n > 0) {
-                        const int32_t* counters = p.ctrl + next[2];
+                        const int32_t* counters = p.ctrl + next[kMiscSet - kMiscNext];
                         const int items = ld_relaxed_gpu(&counters[kSetItems]) - 1, drawn = ld_relaxed_gpu(&counters[kSetWork]);
-                        next[3] = items >= 0 && ((int)gridDim.x - min(plan.n_entries, plan.ctas)) * kWarps + drawn >= items;
+                        next[kMiscNoUnits - kMiscNext] = items >= 0 && ((int)gridDim.x - min(plan.n_entries, plan.ctas)) * kWarps + drawn >= items;
                     }
                 }
             } else {
                 // entries 0 .. plan.ctas-1 are the CTAs' first ones; the counter hands out the rest
-                if (lane == 0) next[iter & 1] = plan.ctas + atomicAdd(p.ctrl + lds_s32(sh.smem + Geo<D>::kSetOffset) + kSetPrefill, 1);
+                if (lane == 0)
+                    next[iter & 1] = plan.ctas + atomicAdd(p.ctrl + lds_s32(sh.smem + Geo<D>::kSetOffset) + kSetPrefill, 1);
             }
             if (!piece_sync()) break;
             entry = next[iter & 1];
