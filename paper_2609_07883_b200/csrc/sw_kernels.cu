@@ -36,7 +36,7 @@ __device__ __forceinline__ void report(int32_t* ctrl, int code, int site, int in
 // 151 us and that of 8/1/128 156 instead of 139 and 148.)
 // (P is AppendParams or MixedParams: the fields have the same names; every index into the chunk arrays is a
 // compile-time constant so that the kernel parameters stay in constant memory.)
-constexpr int kAppendBatch = 4;   // in the fused launch, with 11 warps an SM; the stand-alone kernel has 64 of one part each
+constexpr int kAppendBatch = 4;   // in the fused launch, with 11 warps an SM; the stand-alone kernel has 32 of one part each
 template <bool kMulti, int kBatch, class P>
 __device__ __forceinline__ void append_rows(const P& p, int head_dim, int first, int stride) {
     const int lane = threadIdx.x & 31;
@@ -108,7 +108,7 @@ __device__ __forceinline__ void append_rows(const P& p, int head_dim, int first,
     }
 }
 
-constexpr int kAppendThreads = 256, kAppendBlocksPerSm = 8;
+constexpr int kAppendThreads = 256, kAppendBlocksPerSm = 4;
 __global__ void __launch_bounds__(kAppendThreads, kAppendBlocksPerSm) sw_kv_append_kernel(const AppendParams p) {
     // launched with programmatic stream serialization: it may start while the previous kernel (the attention of
     // the previous iteration, possibly still reading this pool) drains; nothing is touched before this wait
@@ -123,8 +123,9 @@ cudaError_t launch_kv_append(const AppendParams& p, int num_sms, cudaStream_t st
     if (total == 0) return cudaSuccess;
     const int threads = kAppendThreads;
     int64_t blocks = (total + threads / 32 - 1) / (threads / 32);
-    // The grid is resident at once, so that the launch after this one is released at once too.  (With four parts a warp a thread has
-    // 64 registers and half the blocks wait: 3000 rows of 32/8/128 5.5 -> 6.3 us, 8192 12.2 -> 14.1.)
+    // The grid is resident at once, so that the launch after this one is released at once too.  (Four parts a warp and grids of eight
+    // blocks per SM: 3000 rows of 32/8/128 5.5 us instead of 5.2, 8192 10.7 instead of 10.3.  Eight blocks of 32 registers are as
+    // fast alone and 1 us slower with the attention launch behind them, 461 rows 20.2 instead of 19.3 us.)
     if (blocks > (int64_t)num_sms * kAppendBlocksPerSm) blocks = (int64_t)num_sms * kAppendBlocksPerSm;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks);
@@ -193,7 +194,12 @@ struct Geo {
     static constexpr int kSmemBytes = kSharedOffset + 2 * kPageHashBits / 8;      // two bit sets over hashed last pages
 };
 
-constexpr int kWideMergeSplits = 24;  // from this many units of a request on, its last g units share the merge
+// From this many units of a request on, its last g units share the merge.  A merge of groups of eight by one warp takes two splits a
+// round trip, of groups of four four: sharing it from eight units on instead of 24 took 64 contexts of 2000-20000 tokens of 32/4/128
+// from 242 to 225 us, 128 of 8/1/128 from 136 to 123, 97 of them beside 423 tokens from 55 to 48; at head size 64, whose pages are
+// half as long, 40 of 8/2/64 beside 700 tokens from 61 to 57.  (Groups of four at head size 128: 20 contexts of 20000 tokens of 32/8/128
+// 263 -> 252, but 64 log-normal ones beside 256 tokens 143.7 -> 145.5; groups of two: 4/2/64 in place of 8/2/64 56 -> 58.)
+__device__ __forceinline__ constexpr int wide_merge_splits(int head_dim, int g) { return g == 8 || (g == 4 && head_dim == 64) ? 8 : 24; }
 constexpr int kOneRoundMaxPages = 48;  // longest unit (pages) for which one round of units is planned
 constexpr int kPlanCounters = 8;       // shared counters of the plan's block sums, zeroed in the kernel prologue
 // When the CTAs of a single wave of prefill entries turn to decode units: a fixed start-up plus the time of the longest
@@ -670,11 +676,11 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
     // round trip hides behind the last pages, and no warp hoards a unit while others are still idle.
     // With the claim the unit draws its ticket among the units of its (request, kv head): the last ticket makes it
     // the one that merges.  Both answers are read at the end of the unit, when they have long arrived.
-    // A request cut into many units (kWideMergeSplits or more; g where every unit of the launch has a warp of its own, `resident`)
+    // A request cut into many units (wide_merge_splits or more; g where every unit of the launch has a warp of its own, `resident`)
     // has g mergers per kv head, fixed in advance: its last g units, one query-head row each (units of one request and head are
     // Hkv apart in the order in which SMs take them, so the mergers sit on different SMs).  They claim their next unit after
     // the merge.  What they wait for: see rows_to_merge.
-    const bool wide = g > 1 && u.nsplit >= (resident ? g : kWideMergeSplits);
+    const bool wide = g > 1 && u.nsplit >= (resident ? g : wide_merge_splits(D, g));
     const int merge_row = wide && u.nsplit - 1 - u.split < g ? u.nsplit - 1 - u.split : -1;
     if (wide && lane == 0) atomicAdd(&p.tickets[u.ticket], 1);   // started
     bool claimed = merge_row >= 0;

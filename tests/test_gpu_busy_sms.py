@@ -8,7 +8,7 @@ from tests import gpu_util as G
 
 pytestmark = pytest.mark.gpu
 
-HOLD_CYCLES = 100_000_000   # about 50 ms per SM held, a thousand times a launch
+HOLD_CYCLES = 300_000_000   # about 150 ms per SM held, thousands of times a launch
 
 
 @pytest.mark.parametrize("form", ["fused", "two", "static"])

@@ -42,3 +42,27 @@ def test_numbers_of_splits_around_a_batch_of_the_merge(oracle, heads):
 ])
 def test_contexts_at_the_edges_of_the_small_batch_rule(oracle, heads, lens):
     run(oracle, heads, lens, f"{heads} {len(lens)} x {max(lens)}")
+
+
+@pytest.mark.parametrize("heads", [(8, 1, 64), (16, 2, 128), (8, 2, 64), (4, 2, 64), (8, 2, 128)])
+def test_requests_of_1_to_30_units_beside_a_chunk(oracle, heads):
+    """Beside chunk-prefill entries not every unit has a warp of its own: merges by the last ticket and shared ones in one launch."""
+    rng = np.random.default_rng(52)
+    shape = W.AttnShape(*heads)
+    lens = [int(x) for x in np.linspace(20, 3900, 40)]
+    for fused in (True, False):
+        batch = W.make_batch(shape, sum(-(-x // 16) for x in lens) + 40, lens, 100, 400, rng)
+        t = W.host_tensors(batch, rng)
+        pool = t["pool"].copy()
+        assert oracle.kv_append(pool, batch, t["k_new"], t["v_new"]) == 0
+        ref, ref_lse, _ = oracle.mixed_attention(pool, batch, t["q"])
+        r = G.Runner(batch, t)
+        for _ in range(2):
+            if fused:
+                r.iterate()
+            else:
+                r.append()
+                r.attend()
+            assert r.status() == (0, 0)
+            out, lse = r.results()
+            G.compare(out.reshape(-1, shape.head_dim), lse.reshape(-1), ref, ref_lse, f"{heads} fused={fused}")
