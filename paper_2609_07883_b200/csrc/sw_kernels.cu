@@ -209,11 +209,33 @@ constexpr int kPlanCounters = 8;       // shared counters of the plan's block su
 constexpr float kLateBaseUs = 1.0f;
 constexpr int kMinEarlyCtas = 64;  // CTAs whose rings of page copies keep the memory system busy on their own
 constexpr int kMinLateCtas = 24;   // fewer late CTAs than this: their delay is not worth units of two sizes
+
+// Decode-only launches of up to kLinePages pages a warp run without units: the stages (pages of one KV head) of all requests lie in a
+// line, KV head by KV head and request by request, and every CTA gets an equal stretch of it, every warp an equal part of that.  So all
+// warps stream the same number of pages, and the results of a (request, KV head) pair that lies on several warps meet in shared
+// memory: what goes through global memory is one partial result per CTA that a pair reaches beyond, not one per warp.
+// Per launch of 32/8/128, units -> line: one context of 8192 tokens 18.0 -> 15.9 us (33.5 MB: 2.1 TB/s), of 32768 38.7 -> 30.3, 16 of 256-2048
+// 22.2 -> 21.8, 64 of those 58.3 -> 55.2, 256 of 100-500 64.5 -> 61.2, 16 of 8192 90.0 -> 85.5, four of 49152 (55 pages a warp, which were two
+// rounds of units) 141.5 -> 122.0 (6.6 TB/s); 8 of 200-400 12.6 -> 11.5; 20 of 256-4096 tokens of 16/4/64 18.7 -> 16.7, of 16/8/128 37.2 -> 35.7.
+// A static share: beyond kLinePages the spread of the SMs' rates (their stretches of the four long contexts end between 100 and 133 us)
+// costs more than drawing units does.
+constexpr int kLinePages = 64;
+constexpr int kLineMaxDecode = 432;
+constexpr int kLineGroups = kWarps + 1, kLineWords = 4, kLineTable = 88;   // (where the chunk table was: the entries are done)
+// Up to 432 requests, whose lengths, offsets, first stages and last pages take 1732 bytes of the four arrays of the plan; what is left
+// of each holds three partial results (O of the group, m, l) of at most 2 KB + 64 bytes.
+constexpr int kStashBytes = 2048 + 2 * kMaxGroup * 4;
+__device__ __forceinline__ bool use_line(const MixedParams& p, int head_dim, int total_pages) {
+    return p.n <= kLineMaxDecode && p.group * head_dim <= 512 && total_pages > 0 && total_pages <= kLinePages * kWarps * kMaxCtas &&
+           total_pages * p.Hkv <= kLinePages * kWarps * (int)gridDim.x && (int)gridDim.x + p.n * p.Hkv <= p.max_items;
+}
 struct Plan {
     const int* len;     // shared-memory copies of the context lengths and page-list offsets
     const int* indptr;
     bool two_sizes;     // large units handed out by index to the early CTAs, small ones pulled by the late CTAs only
     int total_items;    // units of all requests, times the KV heads
+    int line_ctas;      // CTAs that share the line of stages (0: units are drawn)
+    int head_stages;    // the line: stages of one KV head
 };
 
 // Block-wide exclusive scan of one value per thread (kThreads threads): a warp scan, one barrier, then every thread
@@ -284,12 +306,14 @@ struct LateJoin {
 // run them, so that no warp starts a second unit.  If the early warps are nearly done by the time the late ones arrive,
 // the plan is sized for the early warps alone; if the early CTAs are few, their head start is small or there are many
 // requests per warp, it falls back to units of one size pulled by everybody.
+template <int D, bool kLine>
 __device__ __forceinline__ Plan make_plan(const MixedParams& p, int* unit_prefix, int* len_s, int* indptr_s, int* scratch,
                                           LateJoin late, float pages_per_us) {
     Plan plan;
     plan.len = len_s;
     plan.indptr = indptr_s;
     plan.two_sizes = false;
+    plan.line_ctas = 0;
     const int per_thread = (p.n + kThreads - 1) / kThreads;
     const int beg = min(p.n, (int)threadIdx.x * per_thread);
     const int end = min(p.n, beg + per_thread);
@@ -306,12 +330,25 @@ __device__ __forceinline__ Plan make_plan(const MixedParams& p, int* unit_prefix
     }
     if (threadIdx.x == 0 && p.n > 0) indptr_s[p.n] = p.decode_page_indptr[p.n];
     int* ctr = scratch + 64;  // kPlanCounters counters zeroed in the kernel prologue, one per block sum
-    const int warp_pages = __reduce_add_sync(0xffffffffu, pages_local);
-    if ((threadIdx.x & 31) == 0 && warp_pages != 0) atomicAdd(ctr, warp_pages);
-    const bool any_long = __syncthreads_or(long_local);   // (the barrier of the sum, see block_sum)
-    const int total_pages = *reinterpret_cast<volatile int*>(ctr++);
+    if (__any_sync(0xffffffffu, long_local) && (threadIdx.x & 31) == 0) atomicOr(ctr, 1);
+    int total_pages;
+    int pages_before = block_exclusive_scan(pages_local, scratch + 16, &total_pages);
+    const bool any_long = *reinterpret_cast<volatile int*>(ctr++) != 0;
 
     const int G = (int)gridDim.x;
+    if (kLine && late.ctas == 0 && use_line(p, D, total_pages)) {
+        for (int i = beg, at = pages_before; i < end; ++i) {
+            unit_prefix[i] = at;
+            at += len_s[i] > 0 ? (len_s[i] + kPageSize - 1) / kPageSize : 0;
+        }
+        if (threadIdx.x == 0) unit_prefix[p.n] = total_pages;
+        if (threadIdx.x == 32) scratch[kLineTable + kLineGroups * kLineWords] = 0;
+        plan.head_stages = total_pages;
+        plan.total_items = total_pages * p.Hkv;
+        plan.line_ctas = max(1, min(G, plan.total_items / kWarps));
+        __syncthreads();
+        return plan;
+    }
     constexpr int kMinPages = kMinSplitTokens / kPageSize;
     int split_a = 0, split_b = 0;  // pages per unit of the first requests / of the rest
     int a_pages = 0x7fffffff;      // requests whose pages start below this (per head) are cut with split_a
@@ -344,10 +381,7 @@ __device__ __forceinline__ Plan make_plan(const MixedParams& p, int* unit_prefix
             plan.two_sizes = true;
         }
     }
-    int pages_before = 0;
     if (plan.two_sizes) {
-        int unused;
-        pages_before = block_exclusive_scan(pages_local, scratch + 16, &unused);
         // count the units of either size and grow the size until they fit their warps (the estimates are rarely off)
         const int a_units = (G - late.ctas) * kWarps / p.Hkv, b_units = late.ctas * kWarps / p.Hkv;
         for (int pass = 0; pass < (kPlanCounters - 1) / 2; ++pass) {
@@ -605,47 +639,175 @@ __device__ __forceinline__ int rows_to_merge(int32_t* ready, const int32_t* star
     return own;
 }
 
-// Runs one unit; returns false if a bounded wait expired.
+// A decode unit's queries as B fragments of Q^T: the lane holds head lane / 4, elements 2 (lane % 4) + {0, 1} (+ 8) of every 16.
+template <int D>
+__device__ __forceinline__ void load_query(const MixedParams& p, int q_row, int kvh, uint32_t (&qb)[D / 16][2]) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(p.q + ((int64_t)q_row * p.Hq + kvh * p.group + (lane >> 2)) * D + (lane & 3) * 2);
+    const bool live = (lane >> 2) < p.group;
+#pragma unroll
+    for (int ks = 0; ks < D / 16; ++ks) {
+        qb[ks][0] = live ? src[ks * 8] : 0u;
+        qb[ks][1] = live ? src[ks * 8 + 4] : 0u;
+    }
+}
+
+// O^T of the keys so far: columns 16 t + lane / 4 (+ 8) of heads 2 (lane % 4) + {0, 1}; m of those two heads; l over the lane's own keys.
+template <int D>
+struct DecodeState {
+    float o[D / 16][4];
+    float m0, m1, l0, l1;
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int i = 0; i < D / 16; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
+        m0 = m1 = -INFINITY;
+        l0 = l1 = 0.f;
+    }
+};
+
+// One page (K and V of a head at sK, `valid` keys of it attended) on one warp.
 //
 // The products are transposed: the 16 rows of an mma.m16n8k16 are keys (of S = K Q^T) or output columns (of O^T = V^T P^T) and
 // its 8 columns are the query heads of the group (columns past the group are zero queries), half the instructions of the form
 // with the heads as rows, which would be padded to 16.
 template <int D>
+__device__ __forceinline__ void attend_page(const MixedParams& p, uint32_t sK, int valid, const uint32_t (&qb)[D / 16][2], DecodeState<D>& st) {
+    constexpr int KS = D / 16;  // k-slices of K Q^T; also 16-column tiles of O
+    const int lane = threadIdx.x & 31;
+    // Per-lane offsets of the ldmatrix rows: the four 8x8 matrices are keys 0-7 / 8-15 of one 8-element block, then of the next
+    // (K), or the two blocks of keys 0-7, then of keys 8-15 (V, transposed).  In the 128-byte swizzle 16-byte chunk c of row r
+    // lies at c ^ (r % 8), so a step of two chunks flips address bits 5 and 6.
+    const uint32_t k_addr = sK + (lane & 15) * 128 + (((lane >> 4) ^ (lane & 7)) << 4);
+    const uint32_t v_addr = sK + Geo<D>::kHalves * Geo<D>::kBlockBytes + ((lane & 7) + ((lane >> 4) << 3)) * 128 +
+                            ((((lane >> 3) & 1) ^ (lane & 7)) << 4);
+    // S^T = K Q^T for 16 keys, in two chains
+    float s[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks) {
+        uint32_t a0, a1, a2, a3;
+        ldmatrix_x4((k_addr ^ ((ks & 3) * 32)) + (ks >> 2) * Geo<D>::kBlockBytes, a0, a1, a2, a3);
+        mma_bf16_16816(ks & 1 ? s2 : s, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
+    }
+    // the lane's keys are lane / 4 and lane / 4 + 8; keys past the context are masked
+    const bool ok0 = (lane >> 2) < valid, ok1 = (lane >> 2) + 8 < valid;
+    s[0] = ok0 ? s[0] + s2[0] : -INFINITY;
+    s[1] = ok0 ? s[1] + s2[1] : -INFINITY;
+    s[2] = ok1 ? s[2] + s2[2] : -INFINITY;
+    s[3] = ok1 ? s[3] + s2[3] : -INFINITY;
+    float mx0 = fmaxf(s[0], s[2]), mx1 = fmaxf(s[1], s[3]);
+#pragma unroll
+    for (int w = 4; w < 32; w <<= 1) {
+        mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, w));
+        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, w));
+    }
+    mx0 = fmaxf(st.m0, mx0);
+    mx1 = fmaxf(st.m1, mx1);
+    const float c0 = fast_exp2((st.m0 - mx0) * p.sm_scale_log2), c1 = fast_exp2((st.m1 - mx1) * p.sm_scale_log2);
+    st.m0 = mx0;
+    st.m1 = mx1;
+    const float b0 = mx0 * p.sm_scale_log2, b1 = mx1 * p.sm_scale_log2;
+    s[0] = fast_exp2(fmaf(s[0], p.sm_scale_log2, -b0));
+    s[1] = fast_exp2(fmaf(s[1], p.sm_scale_log2, -b1));
+    s[2] = fast_exp2(fmaf(s[2], p.sm_scale_log2, -b0));
+    s[3] = fast_exp2(fmaf(s[3], p.sm_scale_log2, -b1));
+    st.l0 = st.l0 * c0 + (s[0] + s[2]);
+    st.l1 = st.l1 * c1 + (s[1] + s[3]);
+#pragma unroll
+    for (int i = 0; i < KS; ++i) {
+        st.o[i][0] *= c0;
+        st.o[i][1] *= c1;
+        st.o[i][2] *= c0;
+        st.o[i][3] *= c1;
+    }
+    // P^T [keys][heads] as the B operand: keys along the fragment's registers, so the 8x8 blocks are transposed
+    const uint32_t p0 = movmatrix_trans(pack_bf16x2(s[0], s[1])), p1 = movmatrix_trans(pack_bf16x2(s[2], s[3]));
+
+    // the unwritten slots of a partly filled last page hold whatever the pool held: zero those V rows so that
+    // 0 * garbage cannot produce NaN
+    if (valid < kPageSize) {
+        __syncwarp();
+        const int dead_rows = kPageSize - valid;
+        for (int c = lane; c < dead_rows * (D / 8); c += 32) {
+            const int row_i = valid + c / (D / 8);
+            const int chunk = c % (D / 8);
+            sts_v4(sK + (Geo<D>::kHalves + (chunk >> 3)) * Geo<D>::kBlockBytes + row_i * 128 + (((chunk & 7) ^ (row_i & 7)) << 4),
+                   0u, 0u, 0u, 0u);
+        }
+        __syncwarp();
+    }
+
+    // O^T += V^T P^T
+#pragma unroll
+    for (int dn = 0; dn < KS; ++dn) {
+        uint32_t a0, a1, a2, a3;
+        ldmatrix_x4_trans((v_addr ^ ((dn & 3) * 32)) + (dn >> 2) * Geo<D>::kBlockBytes, a0, a1, a2, a3);
+        mma_bf16_16816(st.o[dn], a0, a1, a2, a3, p0, p1);
+    }
+}
+
+// The end of a unit: the row sums over the keys of all lanes, then O through shared memory, so that rows leave in whole lines:
+// O[head][D] with the 32-byte groups of a row rotated by half the head (the lanes' four head pairs then fall on different banks).
+template <int D>
+__device__ __forceinline__ void stage_result(uint32_t dst, int g, DecodeState<D>& st) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int w = 4; w < 32; w <<= 1) {
+        st.l0 += __shfl_xor_sync(0xffffffffu, st.l0, w);
+        st.l1 += __shfl_xor_sync(0xffffffffu, st.l1, w);
+    }
+    const int h = (lane & 3) * 2;
+    const uint32_t addr = dst + (h * D + (lane >> 2)) * 4;
+#pragma unroll
+    for (int t = 0; t < D / 16; ++t) {
+        const uint32_t a0 = addr + ((16 * t) ^ (h * 4)) * 4, a1 = addr + ((16 * t + 8) ^ (h * 4)) * 4;
+        if (h < g) {
+            sts_f32(a0, st.o[t][0]);
+            sts_f32(a1, st.o[t][2]);
+        }
+        if (h + 1 < g) {
+            sts_f32(a0 + D * 4, st.o[t][1]);
+            sts_f32(a1 + D * 4, st.o[t][3]);
+        }
+    }
+    __syncwarp();
+}
+// Output rows of a (request, KV head) pair that one unit did alone, from the staged result.
+template <int D>
+__device__ __forceinline__ void write_rows(const MixedParams& p, uint32_t src, int q_row, int kvh, const DecodeState<D>& st) {
+    constexpr int kRowLanes = D / 4;   // lanes that hold a row, four columns each
+    const int lane = threadIdx.x & 31, g = p.group, col = (lane % kRowLanes) * 4;
+    for (int r0 = 0; r0 < g; r0 += 32 / kRowLanes) {
+        const int r = r0 + lane / kRowLanes;
+        const float ma = __shfl_sync(0xffffffffu, st.m0, r >> 1), mb = __shfl_sync(0xffffffffu, st.m1, r >> 1);
+        const float la = __shfl_sync(0xffffffffu, st.l0, r >> 1), lb = __shfl_sync(0xffffffffu, st.l1, r >> 1);
+        if (r < g) {
+            const float4 x = lds_f4(src + (r * D + (col ^ ((r >> 1) * 8))) * 4);
+            const float inv = 1.f / (r & 1 ? lb : la);
+            const int head = kvh * g + r;
+            *reinterpret_cast<uint2*>(p.out + ((int64_t)q_row * p.Hq + head) * D + col) =
+                make_uint2(pack_bf16x2(x.x * inv, x.y * inv), pack_bf16x2(x.z * inv, x.w * inv));
+            if (p.lse && col == 0) p.lse[(int64_t)q_row * p.Hq + head] = (r & 1 ? mb : ma) * p.sm_scale + __logf(r & 1 ? lb : la);
+        }
+    }
+}
+
+// Runs one unit; returns false if a bounded wait expired.
+template <int D>
 __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const Unit& u, WarpRing<D>& ring, uint32_t smem,
                          int32_t* work, int fixed_items, bool pulls, bool resident, int& next_item) {
-    constexpr int KS = D / 16;  // k-slices of K Q^T; also 16-column tiles of O
     constexpr int kStages = Geo<D>::kStages;
     const int lane = threadIdx.x & 31;
     const int g = p.group;
     const bool patch = p.append_last;   // the new rows are written here; with chunks they were written before
 
-    // B fragments of Q^T: the lane holds head lane / 4, elements 2 (lane % 4) + {0, 1} (+ 8) of every 16
-    uint32_t qb[KS][2];
-    {
-        const uint32_t* src = reinterpret_cast<const uint32_t*>(p.q + ((int64_t)u.q_row * p.Hq + u.kvh * g + (lane >> 2)) * D + (lane & 3) * 2);
-        const bool live = (lane >> 2) < g;
-#pragma unroll
-        for (int ks = 0; ks < KS; ++ks) {
-            qb[ks][0] = live ? src[ks * 8] : 0u;
-            qb[ks][1] = live ? src[ks * 8 + 4] : 0u;
-        }
-    }
-
-    float o[KS][4];   // O^T: columns 16 t + lane / 4 (+ 8) of heads 2 (lane % 4) + {0, 1}
-#pragma unroll
-    for (int i = 0; i < KS; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
-    float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;   // of those two heads; l over the lane's own keys
+    uint32_t qb[D / 16][2];
+    load_query<D>(p, u.q_row, u.kvh, qb);
+    DecodeState<D> st;
+    st.clear();
 
     const int pg0 = u.t_begin / kPageSize;
     const int pg1 = (u.t_end + kPageSize - 1) / kPageSize;
     const int npg = pg1 - pg0;
-
-    // Per-lane offsets of the ldmatrix rows: the four 8x8 matrices are keys 0-7 / 8-15 of one 8-element block, then of the next
-    // (K), or the two blocks of keys 0-7, then of keys 8-15 (V, transposed).  In the 128-byte swizzle 16-byte chunk c of row r
-    // lies at c ^ (r % 8), so a step of two chunks flips address bits 5 and 6.
-    const uint32_t k_lane = (lane & 15) * 128 + (((lane >> 4) ^ (lane & 7)) << 4);
-    const uint32_t v_lane = Geo<D>::kHalves * Geo<D>::kBlockBytes + ((lane & 7) + ((lane >> 4) << 3)) * 128 +
-                            ((((lane >> 3) & 1) ^ (lane & 7)) << 4);
 
     int ids = 0;
     int issued = 0;
@@ -719,117 +881,18 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
             patch_page<D>(p, smem, sK, u.q_row, u.kvh, valid, row);
         }
 
-        // S^T = K Q^T for 16 keys, in two chains
-        float s[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f};
-        const uint32_t k_addr = sK + k_lane, v_addr = sK + v_lane;
-#pragma unroll
-        for (int ks = 0; ks < KS; ++ks) {
-            uint32_t a0, a1, a2, a3;
-            ldmatrix_x4((k_addr ^ ((ks & 3) * 32)) + (ks >> 2) * Geo<D>::kBlockBytes, a0, a1, a2, a3);
-            mma_bf16_16816(ks & 1 ? s2 : s, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
-        }
-        // the lane's keys are lane / 4 and lane / 4 + 8; keys past the context are masked
-        const bool ok0 = (lane >> 2) < valid, ok1 = (lane >> 2) + 8 < valid;
-        s[0] = ok0 ? s[0] + s2[0] : -INFINITY;
-        s[1] = ok0 ? s[1] + s2[1] : -INFINITY;
-        s[2] = ok1 ? s[2] + s2[2] : -INFINITY;
-        s[3] = ok1 ? s[3] + s2[3] : -INFINITY;
-        float mx0 = fmaxf(s[0], s[2]), mx1 = fmaxf(s[1], s[3]);
-#pragma unroll
-        for (int w = 4; w < 32; w <<= 1) {
-            mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, w));
-            mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, w));
-        }
-        mx0 = fmaxf(m0, mx0);
-        mx1 = fmaxf(m1, mx1);
-        const float c0 = fast_exp2((m0 - mx0) * p.sm_scale_log2), c1 = fast_exp2((m1 - mx1) * p.sm_scale_log2);
-        m0 = mx0;
-        m1 = mx1;
-        const float b0 = mx0 * p.sm_scale_log2, b1 = mx1 * p.sm_scale_log2;
-        s[0] = fast_exp2(fmaf(s[0], p.sm_scale_log2, -b0));
-        s[1] = fast_exp2(fmaf(s[1], p.sm_scale_log2, -b1));
-        s[2] = fast_exp2(fmaf(s[2], p.sm_scale_log2, -b0));
-        s[3] = fast_exp2(fmaf(s[3], p.sm_scale_log2, -b1));
-        l0 = l0 * c0 + (s[0] + s[2]);
-        l1 = l1 * c1 + (s[1] + s[3]);
-#pragma unroll
-        for (int i = 0; i < KS; ++i) {
-            o[i][0] *= c0;
-            o[i][1] *= c1;
-            o[i][2] *= c0;
-            o[i][3] *= c1;
-        }
-        // P^T [keys][heads] as the B operand: keys along the fragment's registers, so the 8x8 blocks are transposed
-        const uint32_t p0 = movmatrix_trans(pack_bf16x2(s[0], s[1])), p1 = movmatrix_trans(pack_bf16x2(s[2], s[3]));
-
-        // the unwritten slots of a partly filled last page hold whatever the pool held: zero those V rows so that
-        // 0 * garbage cannot produce NaN
-        if (valid < kPageSize) {
-            __syncwarp();
-            const int dead_rows = kPageSize - valid;
-            for (int c = lane; c < dead_rows * (D / 8); c += 32) {
-                const int row_i = valid + c / (D / 8);
-                const int chunk = c % (D / 8);
-                sts_v4(sK + (Geo<D>::kHalves + (chunk >> 3)) * Geo<D>::kBlockBytes + row_i * 128 + (((chunk & 7) ^ (row_i & 7)) << 4),
-                       0u, 0u, 0u, 0u);
-            }
-            __syncwarp();
-        }
-
-        // O^T += V^T P^T
-#pragma unroll
-        for (int dn = 0; dn < KS; ++dn) {
-            uint32_t a0, a1, a2, a3;
-            ldmatrix_x4_trans((v_addr ^ ((dn & 3) * 32)) + (dn >> 2) * Geo<D>::kBlockBytes, a0, a1, a2, a3);
-            mma_bf16_16816(o[dn], a0, a1, a2, a3, p0, p1);
-        }
+        attend_page<D>(p, sK, valid, qb, st);
         ring.it += 1;
         __syncwarp();  // every lane is done reading this stage before it is refilled
         if (issued < npg) issue_next();
         claim_next();
     }
 
-    // Finish: the row sums over the keys of all lanes, then (m, l, O) through the unit's last page buffer, so that rows leave in
-    // whole lines: O[head][D] with the 32-byte groups of a row rotated by half the head (the lanes' four head pairs then fall
-    // on different banks).
-#pragma unroll
-    for (int w = 4; w < 32; w <<= 1) {
-        l0 += __shfl_xor_sync(0xffffffffu, l0, w);
-        l1 += __shfl_xor_sync(0xffffffffu, l1, w);
-    }
-    {
-        const int h = (lane & 3) * 2;
-        const uint32_t addr = sK + (h * D + (lane >> 2)) * 4;
-#pragma unroll
-        for (int t = 0; t < KS; ++t) {
-            const uint32_t a0 = addr + ((16 * t) ^ (h * 4)) * 4, a1 = addr + ((16 * t + 8) ^ (h * 4)) * 4;
-            if (h < g) {
-                sts_f32(a0, o[t][0]);
-                sts_f32(a1, o[t][2]);
-            }
-            if (h + 1 < g) {
-                sts_f32(a0 + D * 4, o[t][1]);
-                sts_f32(a1 + D * 4, o[t][3]);
-            }
-        }
-    }
-    __syncwarp();
+    stage_result<D>(sK, g, st);
     constexpr int kRowLanes = D / 4;   // lanes that hold a row, four columns each
     const int col = (lane % kRowLanes) * 4;
     if (u.nsplit == 1) {
-        for (int r0 = 0; r0 < g; r0 += 32 / kRowLanes) {
-            const int r = r0 + lane / kRowLanes;
-            const float ma = __shfl_sync(0xffffffffu, m0, r >> 1), mb = __shfl_sync(0xffffffffu, m1, r >> 1);
-            const float la = __shfl_sync(0xffffffffu, l0, r >> 1), lb = __shfl_sync(0xffffffffu, l1, r >> 1);
-            if (r < g) {
-                const float4 x = lds_f4(sK + (r * D + (col ^ ((r >> 1) * 8))) * 4);
-                const float inv = 1.f / (r & 1 ? lb : la);
-                const int head = u.kvh * g + r;
-                *reinterpret_cast<uint2*>(p.out + ((int64_t)u.q_row * p.Hq + head) * D + col) =
-                    make_uint2(pack_bf16x2(x.x * inv, x.y * inv), pack_bf16x2(x.z * inv, x.w * inv));
-                if (p.lse && col == 0) p.lse[(int64_t)u.q_row * p.Hq + head] = (r & 1 ? mb : ma) * p.sm_scale + __logf(r & 1 ? lb : la);
-            }
-        }
+        write_rows<D>(p, sK, u.q_row, u.kvh, st);
         fence_proxy_async_smem();  // the buffer was written with plain stores and is refilled by the copy engine
         __syncwarp();
         return true;
@@ -843,8 +906,8 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
         *reinterpret_cast<float4*>(p.part_o + ((int64_t)u.slot * g + r) * D + col) = lds_f4(sK + (r * D + (col ^ ((r >> 1) * 8))) * 4);
     if (lane < 4) {
         float* ml = p.part_ml + (int64_t)u.slot * (2 * kMaxGroup) + lane * 2;
-        if (lane * 2 < g) ml[0] = m0, ml[kMaxGroup] = l0;
-        if (lane * 2 + 1 < g) ml[1] = m1, ml[kMaxGroup + 1] = l1;
+        if (lane * 2 < g) ml[0] = st.m0, ml[kMaxGroup] = st.l0;
+        if (lane * 2 + 1 < g) ml[1] = st.m1, ml[kMaxGroup + 1] = st.l1;
     }
     fence_proxy_async_smem();  // the buffer was written with plain stores and is refilled by the copy engine
     __syncwarp();
@@ -907,6 +970,255 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
         default: merge_splits<D, kMaxGroup>(p, u, 0, g); break;
     }
     return true;
+}
+
+// The line of stages (see use_line): CTA `cta` of plan.line_ctas streams its stretch and merges.
+//
+// Positions: x / head_stages is the KV head, x % head_stages the page in the order of the requests.  CTA c has [c T / C, (c + 1) T / C) of
+// the T stages, its warp w the same share of those; page copies run ahead of the (request, KV head) pair that is being worked on.  A pair
+// that begins and ends in the warp is finished by it.  Any other leaves a partial result in shared memory, in the warp's first page
+// buffer if it is the last thing the warp does and in the plan's unused space otherwise; when all warps are done, warps merge the
+// pairs row by row.  A pair that goes on beyond the CTA is published (slots of a pair's CTAs follow one another) and merged by the CTA
+// that publishes last, so nobody waits for another CTA.
+template <int D>
+__device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const MixedParams& p, const Plan& plan, const int* prefix, int* scratch,
+                                         uint32_t smem, int cta) {
+    constexpr int kStages = Geo<D>::kStages, V = D / 32;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int T = plan.total_items, C = plan.line_ctas, g = p.group;   // (T C < 2^25)
+    const int X0 = cta * T / C, X1 = cta < C ? (cta + 1) * T / C : X0, L = X1 - X0;
+    auto warp_begin = [&](int w) { return X0 + w * L / kWarps; };
+    auto ring_of = [&](int w) { return smem + w * kStages * Geo<D>::kStageBytes; };
+    auto stash_of = [&](int w) {   // array w / 3 of the plan, behind its first kLineMaxDecode + 1 words
+        const int at = w < 6 ? (w < 3 ? Geo<D>::kPlanOffset : Geo<D>::kLenOffset) : (w < 9 ? Geo<D>::kIndptrOffset : Geo<D>::kLastOffset);
+        return smem + ((at + (kLineMaxDecode + 1) * 4 + 15) & ~15) + (w % 3) * kStashBytes;
+    };
+    // (head, request, page) of a position
+    auto locate = [&](int x, int& kvh, int& i) {
+        kvh = x / plan.head_stages;
+        const int rem = x - kvh * plan.head_stages;
+        int lo = 0, hi = p.n;  // largest i with prefix[i] <= rem
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (prefix[mid] <= rem) lo = mid; else hi = mid;
+        }
+        i = lo;
+        return rem - prefix[lo];
+    };
+    int* table = scratch + kLineTable;   // pairs that are merged; their number behind them
+    WarpRing<D> ring;
+    ring.buf = ring_of(warp);
+    ring.bar = smem + Geo<D>::kBarOffset + warp * kStages * 8;
+    ring.it = 0;
+    const int x0 = warp_begin(warp), x1 = warp_begin(warp + 1), total = x1 - x0;
+    int id = 0, head = 0, issued = 0;   // lane l: page id and KV head of stage x0 + 32 n + l
+    auto issue_next = [&]() {
+        if ((issued & 31) == 0) {
+            const int x = x0 + issued + lane;
+            id = 0;
+            if (x < x1) {
+                int i;
+                const int page = locate(x, head, i), beg = plan.indptr[i];
+                if (prefix[i + 1] - prefix[i] <= plan.indptr[i + 1] - beg) {
+                    id = p.decode_pages[beg + page];
+                    if (id < 0 || (int64_t)id >= p.num_pages) {   // never reaches the copy engine
+                        report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAttnPage, p.C + i);
+                        id = 0;
+                    }
+                } else {
+                    report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAttnLen, p.C + i);
+                }
+            }
+        }
+        issue_page<D>(kvp_map, ring, issued, __shfl_sync(0xffffffffu, id, issued & 31), __shfl_sync(0xffffffffu, head, issued & 31));
+        ++issued;
+    };
+    for (int k = 0; k < kStages && k < total; ++k) issue_next();
+    bool ok = true;
+#pragma unroll 1
+    for (int x = x0; x < x1 && ok;) {
+        int kvh, i;
+        const int page = locate(x, kvh, i), pages = prefix[i + 1] - prefix[i];
+        const int a = x - page, b = a + pages, end = min(b, x1);   // the pair's stretch of the line; where the warp's part of it ends
+        const bool alone = a >= x0 && b <= x1, listed = pages <= plan.indptr[i + 1] - plan.indptr[i];
+        uint32_t qb[D / 16][2];
+        load_query<D>(p, p.C + i, kvh, qb);
+        DecodeState<D> st;
+        st.clear();
+        uint32_t sK = 0;
+        int valid = plan.len[i] - page * kPageSize;   // keys from the page on
+#pragma unroll 1
+        for (; x < end; ++x, valid -= kPageSize) {
+            const uint32_t stage = ring.it % kStages, parity = (ring.it / kStages) & 1;
+            sK = ring.buf + stage * Geo<D>::kStageBytes;
+            const bool patched = p.append_last && valid <= kPageSize;
+            uint4 row;
+            if (patched) row = load_new_row<D>(p, i, kvh);
+            if (!mbar_wait(ring.bar + stage * 8, parity) || (patched && !mbar_wait(smem + Geo<D>::kLastBarOffset, 0))) {
+                report(p.ctrl, SW_ERR_DEVICE_TIMEOUT, kSiteWait, p.C + i);
+                ok = false;
+                break;
+            }
+            if (patched) {
+                __syncwarp();
+                patch_page<D>(p, smem, sK, i, kvh, valid, row);
+            }
+            attend_page<D>(p, sK, valid, qb, st);
+            ring.it += 1;
+            __syncwarp();  // every lane is done reading this stage before it is refilled
+            if (x + 1 < end && issued < total) issue_next();
+        }
+        if (!listed) st.clear();   // nothing of this request counts
+        const uint32_t keep = alone ? sK : (end == x1 ? ring.buf : stash_of(warp));
+        stage_result<D>(keep, g, st);
+        if (alone) {
+            if (listed) write_rows<D>(p, keep, p.C + i, kvh, st);
+            fence_proxy_async_smem();  // the buffer was written with plain stores and is refilled by the copy engine
+            __syncwarp();
+        } else {
+            if (lane < 4) {   // m and l of the group behind O
+                sts_f32(keep + (g * D + 2 * lane) * 4, st.m0);
+                sts_f32(keep + (g * D + 2 * lane + 1) * 4, st.m1);
+                sts_f32(keep + (g * D + kMaxGroup + 2 * lane) * 4, st.l0);
+                sts_f32(keep + (g * D + kMaxGroup + 2 * lane + 1) * 4, st.l1);
+            }
+            if (lane == 0 && max(a, x0) == max(a, X0)) {   // the pair's first warp in this CTA
+                const int lb = min(b, X1), wb = ((lb - X0) * kWarps - 1) / L, ca = ((a + 1) * C - 1) / T, cb = (b * C - 1) / T;
+                int* e = table + atomicAdd(table + kLineGroups * kLineWords, 1) * kLineWords;
+                e[0] = i * p.Hkv + kvh;
+                e[1] = warp | wb << 8 | (lb == warp_begin(wb + 1) ? 1 << 16 : 0);
+                e[2] = ca;
+                e[3] = cb - ca + 1;
+            }
+        }
+        if (issued < total) issue_next();
+    }
+    __syncthreads();
+    const int lg = 31 - __clz(g), tasks = *reinterpret_cast<volatile int*>(table + kLineGroups * kLineWords) << lg;
+    bool beyond = false;   // some pair goes on in another CTA
+#pragma unroll 1
+    for (int t = lane; t < tasks; t += 32) beyond |= table[(t >> lg) * kLineWords + 3] > 1;
+    beyond = __any_sync(0xffffffffu, beyond);
+    auto finish_row = [&](int pair, int row, float m, float l, const float (&acc)[V]) {
+        if (l == 0.f) return;   // a request whose page list is too short
+        const int i = pair / p.Hkv, kvh = pair - i * p.Hkv;
+        const float inv = 1.f / l;
+        const int64_t out_row = (int64_t)(p.C + i) * p.Hq + kvh * g + row;
+        uint32_t* dst = reinterpret_cast<uint32_t*>(p.out + out_row * D + lane * V);
+#pragma unroll
+        for (int v = 0; v < V; v += 2) dst[v / 2] = pack_bf16x2(acc[v] * inv, acc[v + 1] * inv);
+        if (p.lse && lane == 0) p.lse[out_row] = m * p.sm_scale + __logf(l);
+    };
+#pragma unroll 1
+    for (int t = warp; t < tasks; t += kWarps) {
+        const int* e = table + (t >> lg) * kLineWords;
+        const int pair = e[0], row = t & (g - 1), wa = e[1] & 0xff, wb = e[1] >> 8 & 0xff;
+        const int w = min(wa + lane, wb);
+        const bool live = wa + lane <= wb && warp_begin(w) < warp_begin(w + 1);
+        const uint32_t at = w < wb || (e[1] >> 16) != 0 ? ring_of(w) : stash_of(w);
+        const float ms = live ? lds_f32(at + (g * D + row) * 4) : -INFINITY;
+        float mw = ms, lw = live ? lds_f32(at + (g * D + kMaxGroup + row) * 4) : 0.f;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) mw = fmaxf(mw, __shfl_xor_sync(0xffffffffu, mw, o));   // (kWarps <= 16)
+        const float wgt = ms == -INFINITY ? 0.f : fast_exp2((ms - mw) * p.sm_scale_log2);
+        lw *= wgt;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) lw += __shfl_xor_sync(0xffffffffu, lw, o);
+        mw = __shfl_sync(0xffffffffu, mw, 0);
+        lw = __shfl_sync(0xffffffffu, lw, 0);
+        float acc[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc[v] = 0.f;
+        const uint32_t col = (row * D + ((lane * V) ^ ((row >> 1) * 8))) * 4;
+#pragma unroll 2
+        for (int j = 0; j <= wb - wa; ++j) {
+            const float wj = __shfl_sync(0xffffffffu, wgt, j);
+            const uint32_t src = __shfl_sync(0xffffffffu, at, j) + col;
+            if (wj == 0.f) continue;   // (warps without a stage among them: their buffers hold anything)
+#pragma unroll
+            for (int v = 0; v < V; v += 2) {
+                const float2 y = lds_f2(src + v * 4);
+                acc[v] = fmaf(wj, y.x, acc[v]);
+                acc[v + 1] = fmaf(wj, y.y, acc[v + 1]);
+            }
+        }
+        if (e[3] == 1) {
+            finish_row(pair, row, mw, lw, acc);
+        } else {
+            const int slot = cta + (pair % p.Hkv) * p.n + pair / p.Hkv;
+            float2* dst = reinterpret_cast<float2*>(p.part_o + ((int64_t)slot * g + row) * D + lane * V);
+#pragma unroll
+            for (int v = 0; v < V; v += 2) dst[v / 2] = make_float2(acc[v], acc[v + 1]);
+            if (lane == 0) {
+                p.part_ml[(int64_t)slot * (2 * kMaxGroup) + row] = mw;
+                p.part_ml[(int64_t)slot * (2 * kMaxGroup) + kMaxGroup + row] = lw;
+            }
+        }
+    }
+    if (!beyond) return;
+    __syncthreads();
+    if (threadIdx.x < kLineGroups && threadIdx.x << lg < tasks) {
+        int* e = table + threadIdx.x * kLineWords;
+        if (e[3] > 1) {
+            __threadfence();
+            const bool last = atomicAdd(&p.tickets[e[0]], 1) == e[3] - 1;
+            if (last) p.tickets[e[0]] = 0;   // ready for the next launch
+            __threadfence();
+            e[1] = last;
+        }
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int t = warp; t < tasks; t += kWarps) {
+        const int* e = table + (t >> lg) * kLineWords;
+        if (e[3] == 1 || e[1] == 0) continue;
+        const int pair = e[0], row = t & (g - 1), ns = e[3], slot0 = e[2] + (pair % p.Hkv) * p.n + pair / p.Hkv;
+        const float* ml = p.part_ml + (int64_t)slot0 * (2 * kMaxGroup) + row;
+        const float2* po = reinterpret_cast<const float2*>(p.part_o + ((int64_t)slot0 * g + row) * D + lane * V);
+        float m = -INFINITY, l = 0.f, acc[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc[v] = 0.f;
+        // 32 partial results at a time, lane j holding m and l of the j-th; eight of O in flight
+#pragma unroll 1
+        for (int s0 = 0; s0 < ns; s0 += 32) {
+            const int here = min(32, ns - s0);
+            const float ms = lane < here ? __ldcg(ml + (s0 + lane) * (2 * kMaxGroup)) : -INFINITY;
+            const float ls = lane < here ? __ldcg(ml + (s0 + lane) * (2 * kMaxGroup) + kMaxGroup) : 0.f;
+            float wgt = 0.f;
+#pragma unroll 1
+            for (int j0 = 0; j0 < here; j0 += 8) {
+                float2 y[8][V / 2];
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+#pragma unroll
+                    for (int v = 0; v < V / 2; ++v) y[j][v] = __ldcg(po + (int64_t)(s0 + min(j0 + j, here - 1)) * (g * D / 2) + v);
+                if (j0 == 0) {
+                    float mw = fmaxf(m, ms);
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) mw = fmaxf(mw, __shfl_xor_sync(0xffffffffu, mw, o));
+                    wgt = ms == -INFINITY ? 0.f : fast_exp2((ms - mw) * p.sm_scale_log2);
+                    float lw = wgt * ls;
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) lw += __shfl_xor_sync(0xffffffffu, lw, o);
+                    const float f = m == -INFINITY ? 0.f : fast_exp2((m - mw) * p.sm_scale_log2);
+                    l = l * f + lw;
+                    m = mw;
+#pragma unroll
+                    for (int v = 0; v < V; ++v) acc[v] *= f;
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float wj = j0 + j < here ? __shfl_sync(0xffffffffu, wgt, j0 + j) : 0.f;
+#pragma unroll
+                    for (int v = 0; v < V; v += 2) {
+                        acc[v] = fmaf(wj, y[j][v / 2].x, acc[v]);
+                        acc[v + 1] = fmaf(wj, y[j][v / 2].y, acc[v + 1]);
+                    }
+                }
+            }
+        }
+        finish_row(pair, row, m, l, acc);
+    }
 }
 
 }  // namespace sw
@@ -1040,7 +1352,7 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
         return;
     }
 
-    const Plan plan = make_plan(p, unit_prefix, reinterpret_cast<int*>(smem + Geo<D>::kLenOffset),
+    const Plan plan = make_plan<D, !kMulti>(p, unit_prefix, reinterpret_cast<int*>(smem + Geo<D>::kLenOffset),
                                 reinterpret_cast<int*>(smem + Geo<D>::kIndptrOffset), scratch, late,
                                 p.stages_per_us);
     if (p.append_last) {
@@ -1067,8 +1379,10 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
         if (lane == 0) mbar_arrive(base + Geo<D>::kLastBarOffset);
     }
     if ((int)blockIdx.x == prefill_ctas && threadIdx.x == 0) atomicExch(p.ctrl + misc[kMiscSet] + kSetItems, plan.total_items + 1);
-    if (plan.total_items > p.max_items) {
+    if (plan.line_ctas == 0 && plan.total_items > p.max_items) {
         if (threadIdx.x == 0) report(p.ctrl, SW_ERR_WORKSPACE, kSiteScratch, plan.total_items);
+    } else if (!kMulti && plan.line_ctas > 0) {
+        if constexpr (!kMulti) run_line<D>(&kvp_map, p, plan, unit_prefix, scratch, base, (int)blockIdx.x);
     } else {
         int32_t* work = p.ctrl + lds_s32(base + Geo<D>::kSetOffset) + kSetWork;
         WarpRing<D> ring;

@@ -1,0 +1,69 @@
+"""Decode-only launches whose stages are shared out in a line: stretches shorter than a CTA's warps, pairs on one warp, on several and on
+several CTAs, the largest batch and the longest stretches of the rule and the first ones beyond it, page lists that are too short."""
+import numpy as np
+import pytest
+
+from paper_2609_07883_b200 import workloads as W
+from tests import gpu_util as G
+
+pytestmark = pytest.mark.gpu
+
+
+def run(oracle, heads, lens, what, fused=True, seed=71):
+    rng = np.random.default_rng(seed)
+    shape = W.AttnShape(*heads)
+    batch = W.make_batch(shape, sum(-(-x // 16) for x in lens) + 3, lens, 0, 0, rng)
+    t = W.host_tensors(batch, rng)
+    pool = t["pool"].copy()
+    assert oracle.kv_append(pool, batch, t["k_new"], t["v_new"]) == 0
+    ref, ref_lse, _ = oracle.mixed_attention(pool, batch, t["q"])
+    r = G.Runner(batch, t)
+    for _ in range(2):                      # the second launch finds the tickets re-armed
+        if fused:
+            r.iterate()
+        else:
+            r.append()
+            r.attend()
+        assert r.status() == (0, 0)
+        out, lse = r.results()
+        G.compare(out.reshape(-1, shape.head_dim), lse.reshape(-1), ref, ref_lse, what)
+        assert np.array_equal(G.torch_to_bits(r.pool).reshape(-1), pool.reshape(-1)), what
+
+
+@pytest.mark.parametrize("fused", [True, False])
+@pytest.mark.parametrize("heads", [(4, 1, 128), (2, 2, 128), (8, 1, 64), (4, 4, 64), (4, 2, 64)])
+def test_stretches_and_pairs(oracle, heads, fused):
+    for lens in ([1], [16 * 11], [16 * 12], [16 * 13 - 1], [1] * 13, [16 * 25, 1, 17, 16 * 40 - 3],   # up to a few CTAs
+                 [16 * 148 * 12], [16 * 148 * 12 + 1], [16 * 1777, 5],                                 # one page a warp of one head, and one more
+                 [int(x) for x in np.linspace(1, 1500, 60)]):                                          # pairs on one warp and on several
+        run(oracle, heads, lens, f"{heads} {len(lens)} x {max(lens)}", fused)
+
+
+@pytest.mark.parametrize("n", [432, 433])
+def test_largest_batch_of_the_line(oracle, n):
+    run(oracle, (4, 1, 128), [int(x) for x in np.random.default_rng(n).integers(1, 90, n)], f"{n} requests")
+
+
+@pytest.mark.parametrize("pages", [64 * 12 * 148, 64 * 12 * 148 + 1])
+def test_longest_stretches(oracle, pages):
+    run(oracle, (1, 1, 64), [16 * (pages - 100), 16 * 100 - 7], f"{pages} pages")
+
+
+def test_requests_with_short_page_lists(oracle):
+    """Requests whose list ends before their context are reported and get no output; the others' are right."""
+    rng = np.random.default_rng(5)
+    shape = W.AttnShape(8, 2, 128)
+    lens = [700, 16 * 30, 4000, 33, 9]
+    batch = W.make_batch(shape, sum(-(-x // 16) for x in lens) + 3, lens, 0, 0, rng)
+    t = W.host_tensors(batch, rng)
+    ref, ref_lse, _ = oracle.mixed_attention(t["pool"], batch, t["q"])
+    batch.decode_kv_len = batch.decode_kv_len.copy()
+    batch.decode_kv_len[[1, 3]] += 16
+    r = G.Runner(batch, t)
+    r.attend()
+    assert r.status()[0] == r.B.SW_ERR_OUT_OF_RANGE
+    out, lse = r.results()
+    good = [0, 2, 4]
+    ref, ref_lse = ref.reshape(5, 8, 128), ref_lse.reshape(5, 8)
+    G.compare(out[good].reshape(-1, 128), lse[good].reshape(-1), ref[good].reshape(-1, 128), ref_lse[good].reshape(-1), "good requests")
+    assert not out[[1, 3]].any() and not lse[[1, 3]].any()
