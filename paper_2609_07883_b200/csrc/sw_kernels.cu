@@ -4,8 +4,8 @@
 //   sw_mixed_attn_kernel    ONE persistent launch per iteration (Sec. 4.1).  Optionally it first writes the new K/V
 //                           rows itself (the fused form of the append).  CTAs with chunk-prefill entries run them on
 //                           the tensor cores (sw_prefill.cuh).  Every CTA then plans the split-KV decode units from
-//                           the context lengths; a warp's first unit is fixed by its index, further ones come from a
-//                           shared counter; a unit streams its K/V pages with TMA into the warp's shared-memory ring
+//                           the context lengths (without chunks: shares them out as a line, see use_line); a warp's first
+//                           unit is fixed by its index, further ones come from a shared counter; a unit streams its K/V pages with TMA into the warp's shared-memory ring
 //                           and keeps an online softmax in registers; of the units of one (request, kv head) the one
 //                           that drew the last ticket merges the partial results or, where there are many, the last
 //                           ones one query-head row each.
@@ -210,24 +210,25 @@ constexpr float kLateBaseUs = 1.0f;
 constexpr int kMinEarlyCtas = 64;  // CTAs whose rings of page copies keep the memory system busy on their own
 constexpr int kMinLateCtas = 24;   // fewer late CTAs than this: their delay is not worth units of two sizes
 
-// Decode-only launches of up to kLinePages pages a warp run without units: the stages (pages of one KV head) of all requests lie in a
-// line, KV head by KV head and request by request, and every CTA gets an equal stretch of it, every warp an equal part of that.  So all
-// warps stream the same number of pages, and the results of a (request, KV head) pair that lies on several warps meet in shared
-// memory: what goes through global memory is one partial result per CTA that a pair reaches beyond, not one per warp.
-// Per launch of 32/8/128, units -> line: one context of 8192 tokens 18.0 -> 15.9 us (33.5 MB: 2.1 TB/s), of 32768 38.7 -> 30.3, 16 of 256-2048
-// 22.2 -> 21.8, 64 of those 58.3 -> 55.2, 256 of 100-500 64.5 -> 61.2, 16 of 8192 90.0 -> 85.5, four of 49152 (55 pages a warp, which were two
-// rounds of units) 141.5 -> 122.0 (6.6 TB/s); 8 of 200-400 12.6 -> 11.5; 20 of 256-4096 tokens of 16/4/64 18.7 -> 16.7, of 16/8/128 37.2 -> 35.7.
-// A static share: beyond kLinePages the spread of the SMs' rates (their stretches of the four long contexts end between 100 and 133 us)
-// costs more than drawing units does.
-constexpr int kLinePages = 64;
+// Decode-only launches run without units where they can: the stages (pages of one KV head) of all requests lie in a line, KV head by KV
+// head and request by request, and every CTA gets an equal stretch of it, every warp an equal part of that.  So all warps stream the
+// same number of pages, and the results of a (request, KV head) pair that lies on several warps meet in shared memory: what goes
+// through global memory is one partial result per CTA that a pair reaches beyond, not one per warp.
+// Per launch of 32/8/128, units -> line: one context of 8192 tokens 18.0 -> 15.6 us (33.5 MB: 2.1 TB/s), of 32768 38.7 -> 30, 16
+// of 256-2048 22.1 -> 21.5, 64 of those 58.4 -> 55.3, 8 of 200-400 12.6 -> 11.3, four of 49152 (55 pages a warp, which were two rounds of
+// units) 140.7 -> 123.0 (6.5 TB/s), 128 log-normal ones 259 -> 252.4, 16 of 32k-131k 791 -> 774 (7.4 TB/s); 20 of 256-4096 tokens of 16/4/64
+// 18.6 -> 16.0.  What is left: 4 us to the first copies, CTAs that end up to 15 % apart (the SMs' rates differ), 2-4 us of merges.
+// (Beside chunk-prefill entries units stay: shares fixed by an estimate of when the late CTAs come were slower as often as faster, 16
+// contexts of 256-2048 beside 300 tokens 26.4 -> 31.8 us, 40 of 256-8192 of 16/4/64 beside 700 42.2 -> 40.1.)
+constexpr int kLineMaxStages = 1 << 23;   // 64 GB at head size 128; positions times CTAs fit 32 bits
 constexpr int kLineMaxDecode = 432;
 constexpr int kLineGroups = kWarps + 1, kLineWords = 4, kLineTable = 88;   // (where the chunk table was: the entries are done)
 // Up to 432 requests, whose lengths, offsets, first stages and last pages take 1732 bytes of the four arrays of the plan; what is left
 // of each holds three partial results (O of the group, m, l) of at most 2 KB + 64 bytes.
 constexpr int kStashBytes = 2048 + 2 * kMaxGroup * 4;
-__device__ __forceinline__ bool use_line(const MixedParams& p, int head_dim, int total_pages) {
-    return p.n <= kLineMaxDecode && p.group * head_dim <= 512 && total_pages > 0 && total_pages <= kLinePages * kWarps * kMaxCtas &&
-           total_pages * p.Hkv <= kLinePages * kWarps * (int)gridDim.x && (int)gridDim.x + p.n * p.Hkv <= p.max_items;
+inline bool line_form(const MixedParams& p, int head_dim) { return p.n <= kLineMaxDecode && p.group * head_dim <= 512; }   // on the host
+__device__ __forceinline__ bool use_line(const MixedParams& p, int total_pages) {
+    return total_pages > 0 && (int64_t)total_pages * p.Hkv <= kLineMaxStages && (int)gridDim.x + p.n * p.Hkv <= p.max_items;
 }
 struct Plan {
     const int* len;     // shared-memory copies of the context lengths and page-list offsets
@@ -306,7 +307,7 @@ struct LateJoin {
 // run them, so that no warp starts a second unit.  If the early warps are nearly done by the time the late ones arrive,
 // the plan is sized for the early warps alone; if the early CTAs are few, their head start is small or there are many
 // requests per warp, it falls back to units of one size pulled by everybody.
-template <int D, bool kLine>
+template <int D, bool kLineForm>
 __device__ __forceinline__ Plan make_plan(const MixedParams& p, int* unit_prefix, int* len_s, int* indptr_s, int* scratch,
                                           LateJoin late, float pages_per_us) {
     Plan plan;
@@ -330,13 +331,21 @@ __device__ __forceinline__ Plan make_plan(const MixedParams& p, int* unit_prefix
     }
     if (threadIdx.x == 0 && p.n > 0) indptr_s[p.n] = p.decode_page_indptr[p.n];
     int* ctr = scratch + 64;  // kPlanCounters counters zeroed in the kernel prologue, one per block sum
-    if (__any_sync(0xffffffffu, long_local) && (threadIdx.x & 31) == 0) atomicOr(ctr, 1);
-    int total_pages;
-    int pages_before = block_exclusive_scan(pages_local, scratch + 16, &total_pages);
-    const bool any_long = *reinterpret_cast<volatile int*>(ctr++) != 0;
+    int total_pages, pages_before = 0;
+    bool any_long;
+    if constexpr (kLineForm) {
+        if (__any_sync(0xffffffffu, long_local) && (threadIdx.x & 31) == 0) atomicOr(ctr, 1);
+        pages_before = block_exclusive_scan(pages_local, scratch + 16, &total_pages);
+        any_long = *reinterpret_cast<volatile int*>(ctr++) != 0;
+    } else {
+        const int warp_pages = __reduce_add_sync(0xffffffffu, pages_local);
+        if ((threadIdx.x & 31) == 0 && warp_pages != 0) atomicAdd(ctr, warp_pages);
+        any_long = __syncthreads_or(long_local);   // (the barrier of the sum, see block_sum)
+        total_pages = *reinterpret_cast<volatile int*>(ctr++);
+    }
 
     const int G = (int)gridDim.x;
-    if (kLine && late.ctas == 0 && use_line(p, D, total_pages)) {
+    if (kLineForm && use_line(p, total_pages)) {
         for (int i = beg, at = pages_before; i < end; ++i) {
             unit_prefix[i] = at;
             at += len_s[i] > 0 ? (len_s[i] + kPageSize - 1) / kPageSize : 0;
@@ -382,6 +391,8 @@ __device__ __forceinline__ Plan make_plan(const MixedParams& p, int* unit_prefix
         }
     }
     if (plan.two_sizes) {
+        int unused;
+        pages_before = block_exclusive_scan(pages_local, scratch + 16, &unused);
         // count the units of either size and grow the size until they fit their warps (the estimates are rarely off)
         const int a_units = (G - late.ctas) * kWarps / p.Hkv, b_units = late.ctas * kWarps / p.Hkv;
         for (int pass = 0; pass < (kPlanCounters - 1) / 2; ++pass) {
@@ -791,14 +802,14 @@ __device__ __forceinline__ void write_rows(const MixedParams& p, uint32_t src, i
     }
 }
 
-// Runs one unit; returns false if a bounded wait expired.
-template <int D>
+// Runs one unit; returns false if a bounded wait expired.  kAlone: of a launch without chunk rows, whose new rows are written here;
+// with chunks they are written before.
+template <int D, bool kAlone>
 __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const Unit& u, WarpRing<D>& ring, uint32_t smem,
                          int32_t* work, int fixed_items, bool pulls, bool resident, int& next_item) {
     constexpr int kStages = Geo<D>::kStages;
     const int lane = threadIdx.x & 31;
     const int g = p.group;
-    const bool patch = p.append_last;   // the new rows are written here; with chunks they were written before
 
     uint32_t qb[D / 16][2];
     load_query<D>(p, u.q_row, u.kvh, qb);
@@ -826,7 +837,7 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
             page = 0;
         }
         // the request's last page holds the row this iteration appends
-        if (p.append_first && (pg0 + issued + 1) * kPageSize >= u.len && !wait_append(p, smem + Geo<D>::kSetOffset)) {
+        if (!kAlone && p.append_first && (pg0 + issued + 1) * kPageSize >= u.len && !wait_append(p, smem + Geo<D>::kSetOffset)) {
             if (lane == 0) report(p.ctrl, SW_ERR_DEVICE_TIMEOUT, kSiteWait, u.q_row);
             append_timeout = true;
         }
@@ -865,7 +876,7 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
         const uint32_t parity = (ring.it / kStages) & 1;
         sK = ring.buf + stage * Geo<D>::kStageBytes;
         const int valid = u.len - (pg0 + k) * kPageSize;   // keys of this page that are attended (16 or more: all)
-        const bool patched = patch && valid <= kPageSize;
+        const bool patched = kAlone && p.append_last && valid <= kPageSize;
         uint4 row;
         if (patched) row = load_new_row<D>(p, u.q_row, u.kvh);   // (no chunk rows: q_row is the request)
         if (!mbar_wait(ring.bar + stage * 8, parity)) {
@@ -972,6 +983,30 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
     return true;
 }
 
+// The requests' last pages, which fused decode-only launches write, by id; whole CTA.  Only warps with a request wait for the load.
+template <int D>
+__device__ __forceinline__ void list_last_pages(const MixedParams& p, const Plan& plan, uint32_t smem, unsigned* sets) {
+    for (int i = threadIdx.x; i < p.n; i += kThreads) {
+        const int len = plan.len[i], pi = (len - 1) / kPageSize;
+        int id = -1;
+        if (len < 1 || pi >= p.decode_page_indptr[i + 1] - plan.indptr[i]) {
+            if (blockIdx.x == 0) report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAppendLen, i);
+        } else {
+            id = p.decode_pages[plan.indptr[i] + pi];
+            if (id < 0 || (int64_t)id >= p.num_pages) {
+                if (blockIdx.x == 0) report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAppendPage, i);
+                id = -1;
+            }
+        }
+        sts_s32(smem + Geo<D>::kLastOffset + i * 4, id);
+        // first request in its bucket: marked in the first set; any other: the bucket is marked in the second
+        const unsigned h = page_hash(id), bit = 1u << (h & 31);
+        if (atomicOr(&sets[h / 32], bit) & bit) atomicOr(&sets[(kPageHashBits + h) / 32], bit);
+    }
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(smem + Geo<D>::kLastBarOffset);
+}
+
 // The line of stages (see use_line): CTA `cta` of plan.line_ctas streams its stretch and merges.
 //
 // Positions: x / head_stages is the KV head, x % head_stages the page in the order of the requests.  CTA c has [c T / C, (c + 1) T / C) of
@@ -982,10 +1017,10 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
 // that publishes last, so nobody waits for another CTA.
 template <int D>
 __device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const MixedParams& p, const Plan& plan, const int* prefix, int* scratch,
-                                         uint32_t smem, int cta) {
+                                         unsigned* sets, uint32_t smem, int cta) {
     constexpr int kStages = Geo<D>::kStages, V = D / 32;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int T = plan.total_items, C = plan.line_ctas, g = p.group;   // (T C < 2^25)
+    const int T = plan.total_items, C = plan.line_ctas, g = p.group;   // (T C < 2^31)
     const int X0 = cta * T / C, X1 = cta < C ? (cta + 1) * T / C : X0, L = X1 - X0;
     auto warp_begin = [&](int w) { return X0 + w * L / kWarps; };
     auto ring_of = [&](int w) { return smem + w * kStages * Geo<D>::kStageBytes; };
@@ -1034,6 +1069,7 @@ __device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const Mixed
         ++issued;
     };
     for (int k = 0; k < kStages && k < total; ++k) issue_next();
+    if (p.append_last) list_last_pages<D>(p, plan, smem, sets);   // after the first copies are on their way
     bool ok = true;
 #pragma unroll 1
     for (int x = x0; x < x1 && ok;) {
@@ -1228,7 +1264,13 @@ namespace sw {
 // ---------------------------------------------------------------------------------------------------------------
 // the persistent kernel
 // ---------------------------------------------------------------------------------------------------------------
-template <int D, bool kMulti>
+// Forms of the kernel, chosen by the host: iterations with one prefill chunk, whose descriptors are then plain kernel parameters; with
+// several (descriptors looked up per work item); without any, where the decodes may be worked off as a line (line_form), and the others.
+// A form has only the code that it needs: with the line's code in the kernel of one chunk, the small mixed launch of 8/2/64 took 13.6 us and 64
+// contexts beside 512 tokens 63.7, with kernels of their own 12.8 and 62.3; 20 contexts
+// of 8/1/128, worked off as units, take 18.2 us in a kernel of their own and 21.6 beside the line's code.
+enum Form { kOneChunk, kSeveralChunks, kLine, kUnits };
+template <int D, Form kForm>
 __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid_constant__ CUtensorMap kv_map,
                                                                        const __grid_constant__ CUtensorMap kvp_map,
                                                                     const __grid_constant__ CUtensorMap q_map,
@@ -1244,7 +1286,8 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
     int* unit_prefix = reinterpret_cast<int*>(smem + Geo<D>::kPlanOffset);
     int* scratch = reinterpret_cast<int*>(smem + Geo<D>::kMiscOffset);
 
-    const bool tensor_prefill = p.C > 0;
+    constexpr bool kMulti = kForm == kSeveralChunks, tensor_prefill = kMulti || kForm == kOneChunk;
+    unsigned* sets = reinterpret_cast<unsigned*>(smem + Geo<D>::kSharedOffset);   // of hashed last pages
     volatile int* misc = reinterpret_cast<volatile int*>(scratch + kMiscAt);
     if (threadIdx.x >= 32 && threadIdx.x < 32 + kPlanCounters) scratch[64 + threadIdx.x - 32] = 0;  // block-sum counters
     if (threadIdx.x < kWarps * Geo<D>::kStages) {
@@ -1252,11 +1295,11 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
         fence_mbar_init();
     }
     if (threadIdx.x >= 128 && threadIdx.x < 128 + 2 * kPageHashBits / 32)
-        reinterpret_cast<unsigned*>(smem + Geo<D>::kSharedOffset)[threadIdx.x - 128] = 0;
+        sets[threadIdx.x - 128] = 0;
     if (threadIdx.x == 96) {
         tma_prefetch_desc(&kvp_map);
         mbar_init(base + Geo<D>::kLastBarOffset, kWarps);
-        if (tensor_prefill) {
+        if constexpr (tensor_prefill) {
             tma_prefetch_desc(&kv_map);
             tma_prefetch_desc(&q_map);
             tma_prefetch_desc(&out_map);
@@ -1296,7 +1339,7 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
         }
         __syncwarp();
     }
-    if (p.append_first) {
+    if (tensor_prefill && p.append_first) {
         // fused launch with chunks: this CTA's share of the new K/V rows (the planning warp has none), then its mark on the
         // counter the readers wait for
         if (warp != 2)
@@ -1313,7 +1356,7 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
     // waits for a counter.  CTAs that start with prefill work take all their decode units from the counter.
     int prefill_ctas = 0;
     LateJoin late{0, 0.f};
-    if (tensor_prefill) {
+    if constexpr (tensor_prefill) {
         const PfPlan pplan = pf_make_plan(base + Geo<D>::kMiscOffset + kChunkTable * 4);
         prefill_ctas = min(pplan.n_entries, pplan.ctas);
         late.ctas = prefill_ctas;
@@ -1352,38 +1395,16 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
         return;
     }
 
-    const Plan plan = make_plan<D, !kMulti>(p, unit_prefix, reinterpret_cast<int*>(smem + Geo<D>::kLenOffset),
+    const Plan plan = make_plan<D, kForm == kLine>(p, unit_prefix, reinterpret_cast<int*>(smem + Geo<D>::kLenOffset),
                                 reinterpret_cast<int*>(smem + Geo<D>::kIndptrOffset), scratch, late,
                                 p.stages_per_us);
-    if (p.append_last) {
-        // The requests' last pages, which fused decode-only launches write.  Only warps with a request wait for the load.
-        for (int i = threadIdx.x; i < p.n; i += kThreads) {
-            const int len = plan.len[i], pi = (len - 1) / kPageSize;
-            int id = -1;
-            if (len < 1 || pi >= p.decode_page_indptr[i + 1] - plan.indptr[i]) {
-                if (blockIdx.x == 0) report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAppendLen, i);
-            } else {
-                id = p.decode_pages[plan.indptr[i] + pi];
-                if (id < 0 || (int64_t)id >= p.num_pages) {
-                    if (blockIdx.x == 0) report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAppendPage, i);
-                    id = -1;
-                }
-            }
-            sts_s32(base + Geo<D>::kLastOffset + i * 4, id);
-            // first request in its bucket: marked in the first set; any other: the bucket is marked in the second
-            unsigned* sets = reinterpret_cast<unsigned*>(smem + Geo<D>::kSharedOffset);
-            const unsigned h = page_hash(id), bit = 1u << (h & 31);
-            if (atomicOr(&sets[h / 32], bit) & bit) atomicOr(&sets[(kPageHashBits + h) / 32], bit);
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(base + Geo<D>::kLastBarOffset);
-    }
     if ((int)blockIdx.x == prefill_ctas && threadIdx.x == 0) atomicExch(p.ctrl + misc[kMiscSet] + kSetItems, plan.total_items + 1);
     if (plan.line_ctas == 0 && plan.total_items > p.max_items) {
         if (threadIdx.x == 0) report(p.ctrl, SW_ERR_WORKSPACE, kSiteScratch, plan.total_items);
-    } else if (!kMulti && plan.line_ctas > 0) {
-        if constexpr (!kMulti) run_line<D>(&kvp_map, p, plan, unit_prefix, scratch, base, (int)blockIdx.x);
+    } else if (kForm == kLine && plan.line_ctas > 0) {
+        if constexpr (kForm == kLine) run_line<D>(&kvp_map, p, plan, unit_prefix, scratch, sets, base, (int)blockIdx.x);
     } else {
+        if (!tensor_prefill && p.append_last) list_last_pages<D>(p, plan, base, sets);
         int32_t* work = p.ctrl + lds_s32(base + Geo<D>::kSetOffset) + kSetWork;
         WarpRing<D> ring;
         ring.buf = base + warp * Geo<D>::kStages * Geo<D>::kStageBytes;
@@ -1434,7 +1455,7 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
                     report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAttnLen, u.q_row);
                     next_item = pulls ? fixed_items + atomicAdd(work, 1) : 0x7fffffff;
                 }
-            } else if (!run_unit<D>(&kvp_map, p, u, ring, base, work, fixed_items, pulls, resident, next_item)) {
+            } else if (!run_unit<D, !tensor_prefill>(&kvp_map, p, u, ring, base, work, fixed_items, pulls, resident, next_item)) {
                 break;
             }
             item = __shfl_sync(0xffffffffu, next_item, 0);
@@ -1469,38 +1490,31 @@ size_t mixed_attn_smem_bytes(int head_dim) {
     return (head_dim == 64 ? Geo<64>::kSmemBytes : Geo<128>::kSmemBytes) + 1024;
 }
 
-// The kernel exists in two forms per head size: for iterations with at most one prefill chunk, whose descriptors are
-// then plain kernel parameters, and for iterations with several (descriptors looked up per work item).
+template <int D, class F>
+cudaError_t for_each_form(F f) {
+    cudaError_t e = f(sw_mixed_attn_kernel<D, kOneChunk>);
+    if (e == cudaSuccess) e = f(sw_mixed_attn_kernel<D, kSeveralChunks>);
+    if (e == cudaSuccess) e = f(sw_mixed_attn_kernel<D, kLine>);
+    return e == cudaSuccess ? f(sw_mixed_attn_kernel<D, kUnits>) : e;
+}
+template <class F>
+cudaError_t for_each_form(int head_dim, F f) { return head_dim == 64 ? for_each_form<64>(f) : for_each_form<128>(f); }
 cudaError_t configure_kernels(int head_dim) {
     const int bytes = (int)mixed_attn_smem_bytes(head_dim);
-    cudaError_t e;
-    if (head_dim == 64) {
-        e = cudaFuncSetAttribute(sw_mixed_attn_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (e != cudaSuccess) return e;
-        return cudaFuncSetAttribute(sw_mixed_attn_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    }
-    e = cudaFuncSetAttribute(sw_mixed_attn_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(sw_mixed_attn_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    return for_each_form(head_dim, [&](auto* kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
 }
 
-// CTAs of the persistent kernel that one SM can hold at a time (the smaller figure of the two forms).  The fused launch
+// CTAs of the persistent kernel that one SM can hold at a time (the smallest figure of all forms).  The fused launch
 // makes CTAs wait for one another's share of the KV append, which is only safe when the whole grid is resident.
 cudaError_t mixed_attn_resident_ctas_per_sm(int head_dim, int* out) {
     const size_t bytes = mixed_attn_smem_bytes(head_dim);
-    int a = 0, b = 0;
-    cudaError_t e;
-    if (head_dim == 64) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, sw_mixed_attn_kernel<64, false>, kThreads, bytes);
-        if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, sw_mixed_attn_kernel<64, true>, kThreads, bytes);
-    } else {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, sw_mixed_attn_kernel<128, false>, kThreads, bytes);
-        if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, sw_mixed_attn_kernel<128, true>, kThreads, bytes);
-    }
-    *out = a < b ? a : b;
-    return e;
+    *out = 1 << 30;
+    return for_each_form(head_dim, [&](auto* kernel) {
+        int n = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThreads, bytes);
+        *out = n < *out ? n : *out;
+        return e;
+    });
 }
 
 cudaError_t launch_mixed_attn(int head_dim, const KvMaps& kv_maps, const CUtensorMap& q_map, const CUtensorMap& out_map,
@@ -1516,12 +1530,15 @@ cudaError_t launch_mixed_attn(int head_dim, const KvMaps& kv_maps, const CUtenso
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const bool multi = p.nchunks > 1;
+    auto launch = [&](auto* kernel) { return cudaLaunchKernelEx(&cfg, kernel, kv_maps.half, kv_maps.page, q_map, out_map, p); };
+    auto form = [&](auto* one, auto* several, auto* line, auto* units) {
+        return p.nchunks > 1 ? launch(several) : (p.nchunks == 1 ? launch(one) : (line_form(p, head_dim) ? launch(line) : launch(units)));
+    };
     if (head_dim == 64)
-        return multi ? cudaLaunchKernelEx(&cfg, sw_mixed_attn_kernel<64, true>, kv_maps.half, kv_maps.page, q_map, out_map, p)
-                     : cudaLaunchKernelEx(&cfg, sw_mixed_attn_kernel<64, false>, kv_maps.half, kv_maps.page, q_map, out_map, p);
-    return multi ? cudaLaunchKernelEx(&cfg, sw_mixed_attn_kernel<128, true>, kv_maps.half, kv_maps.page, q_map, out_map, p)
-                 : cudaLaunchKernelEx(&cfg, sw_mixed_attn_kernel<128, false>, kv_maps.half, kv_maps.page, q_map, out_map, p);
+        return form(sw_mixed_attn_kernel<64, kOneChunk>, sw_mixed_attn_kernel<64, kSeveralChunks>, sw_mixed_attn_kernel<64, kLine>,
+                    sw_mixed_attn_kernel<64, kUnits>);
+    return form(sw_mixed_attn_kernel<128, kOneChunk>, sw_mixed_attn_kernel<128, kSeveralChunks>, sw_mixed_attn_kernel<128, kLine>,
+                sw_mixed_attn_kernel<128, kUnits>);
 }
 
 }  // namespace sw
