@@ -1268,7 +1268,7 @@ namespace sw {
 // several (descriptors looked up per work item); without any, where the decodes may be worked off as a line (line_form), and the others.
 // A form has only the code that it needs: with the line's code in the kernel of one chunk, the small mixed launch of 8/2/64 took 13.6 us and 64
 // contexts beside 512 tokens 63.7, with kernels of their own 12.8 and 62.3; 20 contexts
-// of 8/1/128, worked off as units, take 18.2 us in a kernel of their own and 21.6 beside the line's code.
+// of 8/1/128, worked off as units, take 16.8 us in a kernel of their own and 21.6 beside the line's code (18.3 with all in one).
 enum Form { kOneChunk, kSeveralChunks, kLine, kUnits };
 template <int D, Form kForm>
 __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid_constant__ CUtensorMap kv_map,

@@ -32,13 +32,18 @@ struct PfGeo {
     static constexpr int kAtomBytes = 8 * 128;                   // K, V: one [8 slots][64 elements] swizzled block
     static constexpr int kGroupStride = kHalves * kAtomBytes;    // K, V: 8 keys, [head_dim/64 blocks][8][128 B]
     static constexpr int kPageStride = 2 * kGroupStride;         // K, V: one page = two 8-key groups
+    // TMEM columns: S of tile t (fp32) at 128 t, P (bf16) at kPColumn + kPStride t, O (fp32) at kOColumn + D t.  At head size 64 P has
+    // columns of its own, so that S of a tile's next step can be computed while the softmax warps work on this one (kAhead).  At head
+    // size 128 that would leave one S for both tiles, and the launches are 5 % slower than with P stored over S.
+    static constexpr bool kAhead = D == 64;
+    static constexpr int kPColumn = kAhead ? 256 : 0, kPStride = kAhead ? 64 : 128, kOColumn = kAhead ? 384 : 256;
 };
 
 // P of a tile is handed to the MMA warp in two halves (keys 0-63, then 64-127) so that the first four P V
 // instructions run while the second half is still being exponentiated.
 enum PfBar {
     kBarQFull = 0, kBarKFull = 1, kBarVLanded = 3, kBarVFull = 5, kBarKEmpty = 7, kBarVEmpty = 9,
-    kBarSFull = 11, kBarPHalf = 13 /* [tile][half] */, kBarODone = 17, kPfBars = 19
+    kBarSFull = 11, kBarPHalf = 13 /* [tile][half] */, kBarODone = 17, kBarSFree = 19 /* kAhead */, kPfBars = 21
 };
 
 // register budgets per warpgroup during the prefill phase: 128 * 72 + 256 * 216 <= 384 * 168
@@ -68,7 +73,7 @@ __device__ __forceinline__ int pf_chunk(const MixedParams& p, const PfShared& sh
 }
 
 __device__ __forceinline__ void pf_init_barriers(uint32_t bars) {
-    for (int i = 0; i < kPfBars; ++i) mbar_init(bars + i * 8, (i >= kBarPHalf && i < kBarPHalf + 4) ? 4 : 1);
+    for (int i = 0; i < kPfBars; ++i) mbar_init(bars + i * 8, ((i >= kBarPHalf && i < kBarPHalf + 4) || i >= kBarSFree) ? 4 : 1);
 }
 
 // Bounded wait that also gives up when another role of this CTA has given up.
@@ -611,8 +616,8 @@ __device__ __forceinline__ void pf_issue_pv_half(const PfShared& sh, int t, uint
     constexpr uint32_t idesc = umma_idesc_bf16(128, D, 0, 1);  // B = V is MN-major: [key][d] with d contiguous
     const uint64_t vd = umma_desc_sw128(sh.smem + G::kKVOffset + s * 2 * G::kTileBytes + G::kTileBytes + half * 4 * G::kPageStride,
                                         G::kAtomBytes, G::kGroupStride);
-    const uint32_t d_tmem = sh.tmem + 256 + t * D;
-    const uint32_t p_tmem = sh.tmem + t * 128 + half * 32;
+    const uint32_t d_tmem = sh.tmem + G::kOColumn + t * D;
+    const uint32_t p_tmem = sh.tmem + G::kPColumn + t * G::kPStride + half * 32;
     const uint32_t acc_first = first && half == 0 ? 0u : 1u;
     if (leader) {
 #pragma unroll
@@ -663,6 +668,55 @@ __device__ __forceinline__ bool pf_mma(const MixedParams& p, const PfShared& sh,
                 pf_issue_qk<D>(sh, t, s ^ 1, leader);
             }
             if (more && t == last_active(j + 1)) commit(kBarKEmpty + (s ^ 1));
+        }
+    }
+    st.kv_it += it.j1 - it.j0;
+    st.q_it += 1;
+    return true;
+}
+
+// The same with kAhead: S of a tile is issued after the other tile's P V, a step earlier, PV0(j), QK1(j + 1), PV1(j), QK0(j + 2), ..., so that
+// it lies ready when the tile's softmax warps have written P.  (4111 + 1777 tokens of 16/4/64: 80.4 -> 76.8 us; entries of a few steps
+// lose 0.2: four contexts beside 256 + 128 of 8/2/64 12.9 -> 13.1.)
+template <int D>
+__device__ __forceinline__ bool pf_mma_ahead(const MixedParams& p, const PfShared& sh, const PfItem& it, PfMmaState& st) {
+    const bool leader = elect_one();
+    auto act = [&](int t, int j) { return j < it.j1 && j < it.nkv[t]; };
+    auto commit = [&](int bar) {
+        if (leader) tc_commit(sh.bars + bar * 8);
+    };
+    // S of tile t, step j: the first tile of a step waits for K, the last one hands it back; the tile's S before (one ahead of its
+    // P V products) has been read
+    auto issue_qk = [&](int t, int j, bool used) {
+        const uint32_t cur = st.kv_it + (j - it.j0), s = cur & 1;
+        if ((t == 0 || !act(0, j)) && !pf_wait(sh, kBarKFull + s, (cur >> 1) & 1, p.ctrl, 5)) return false;
+        if (used && !pf_wait(sh, kBarSFree + t, st.p_cnt[t] & 1, p.ctrl, 7)) return false;
+        tc_fence_after_sync();
+        pf_issue_qk<D>(sh, t, s, leader);
+        if (t == 1 || !act(1, j)) commit(kBarKEmpty + s);
+        return true;
+    };
+    if (!pf_wait(sh, kBarQFull, st.q_it & 1, p.ctrl, 4)) return false;
+    const int j0 = it.j0;
+    if (act(0, j0) && !issue_qk(0, j0, false)) return false;
+    if (act(1, j0) && !issue_qk(1, j0, false)) return false;
+    if (act(0, j0 + 1) && !issue_qk(0, j0 + 1, true)) return false;
+    for (int j = j0; j < it.j1; ++j) {
+        const uint32_t cur = st.kv_it + (j - j0), s = cur & 1;
+        if (!pf_wait(sh, kBarVFull + s, (cur >> 1) & 1, p.ctrl, 6)) return false;
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            if (act(t, j)) {
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    if (!pf_wait(sh, kBarPHalf + 2 * t + half, st.p_cnt[t] & 1, p.ctrl, 8)) return false;
+                    tc_fence_after_sync();
+                    pf_issue_pv_half<D>(sh, t, s, half, j == j0, leader);
+                }
+                st.p_cnt[t] += 1;
+                if (t == 1 || !act(1, j)) commit(kBarVEmpty + s);
+            }
+            if (act(1 - t, j + 1 + t) && !issue_qk(1 - t, j + 1 + t, true)) return false;
         }
     }
     st.kv_it += it.j1 - it.j0;
@@ -722,8 +776,9 @@ __device__ __forceinline__ bool pf_softmax(const CUtensorMap* out_map, const Mix
     const int head = it.kvh * p.group + row % p.group;
     const int pos = pf_chunk<D, kMulti>(p, sh, 0, it.chunk) + tok;
     const uint32_t lane_addr = sh.tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const uint32_t s_addr = lane_addr + t * 128;  // P (bf16) aliases the first 64 columns of S
-    const uint32_t o_addr = lane_addr + 256 + t * D;
+    const uint32_t s_addr = lane_addr + t * 128;
+    const uint32_t p_addr = lane_addr + G::kPColumn + t * G::kPStride;
+    const uint32_t o_addr = lane_addr + G::kOColumn + t * D;
     const float sl2 = p.sm_scale_log2;
     float m_ref = -INFINITY, l_sum = 0.f;
     uint32_t v[32];
@@ -738,6 +793,11 @@ __device__ __forceinline__ bool pf_softmax(const CUtensorMap* out_map, const Mix
 #pragma unroll
         for (int c = 0; c < 4; ++c) tmem_ld_32x32b_x32(s_addr + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
         tc_wait_ld();
+        if constexpr (G::kAhead) {   // S may be overwritten
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(sh.bars + (kBarSFree + t) * 8);
+        }
         if (limit < 128) {
 #pragma unroll
             for (int i = 0; i < 128; ++i) s[i] = i < limit ? s[i] : 0xff800000u;  // -inf: exp2 gives exactly 0
@@ -763,9 +823,12 @@ __device__ __forceinline__ bool pf_softmax(const CUtensorMap* out_map, const Mix
             // lazy rescale: keep the old reference unless some row's maximum grew by more than 2^8
             // (a row whose keys were all masked so far has m_ref = -inf and no weight yet: it just adopts m_new)
             const bool need = m_new - m_ref > 8.0f;
-            if (__any_sync(0xffffffffu, need)) {
+            const bool any = __any_sync(0xffffffffu, need);
+            if (G::kAhead || any) {   // the step before has updated O (and, with kAhead, read P)
                 if (!pf_wait(sh, kBarODone + t, (st.o_cnt + (j - it.j0) - 1) & 1, p.ctrl, 10)) return false;
                 tc_fence_after_sync();
+            }
+            if (any) {
                 const float f = need ? fast_exp2(m_ref - m_new) : 1.f;
 #pragma unroll
                 for (int c = 0; c < D / 32; ++c) {
@@ -782,7 +845,7 @@ __device__ __forceinline__ bool pf_softmax(const CUtensorMap* out_map, const Mix
                 }
             }
         }
-        // P = exp2(S * scale - m_ref), packed to bf16 over the columns of S (all of S is already in registers)
+        // P = exp2(S * scale - m_ref), packed to bf16 (all of S is already in registers)
         const float neg_m = m_ref == -INFINITY ? 0.f : -m_ref;
         const uint64_t scale2 = pack_f32x2(sl2, sl2), negm2 = pack_f32x2(neg_m, neg_m);
         uint64_t sum_a = pack_f32x2(0.f, 0.f), sum_b = sum_a;
@@ -806,7 +869,7 @@ __device__ __forceinline__ bool pf_softmax(const CUtensorMap* out_map, const Mix
                 if (i & 1) sum_b = add_f32x2(sum_b, pack_f32x2(p0, p1)); else sum_a = add_f32x2(sum_a, pack_f32x2(p0, p1));
                 pk[i] = pack_bf16x2(p0, p1);
             }
-            tmem_st_32x32b_x16(s_addr + c * 16, pk);
+            tmem_st_32x32b_x16(p_addr + c * 16, pk);
             if (c == 1) {  // the first 64 keys of P are in place: the first half of P V may start
                 tc_wait_st();
                 tc_fence_before_sync();
@@ -1008,7 +1071,7 @@ __device__ __forceinline__ void prefill_phase(const CUtensorMap* kv_map, const C
             if (warp == 0) {
                 if (it.j1 > it.j0) pf_produce<D, kMulti>(kv_map, q_map, p, sh, it, prod_kv_it);
             } else if (warp == 1) {
-                if (it.j1 > it.j0) pf_mma<D>(p, sh, it, mma_state);
+                if (it.j1 > it.j0) PfGeo<D>::kAhead ? pf_mma_ahead<D>(p, sh, it, mma_state) : pf_mma<D>(p, sh, it, mma_state);
             } else if (warp == 2) {
                 if (it.j1 > it.j0) pf_sanitize<D, kMulti>(p, sh, it, san_kv_it);
                 // Near the end of what may be the CTA's last entry: whether the decode units have all been handed out (the CTAs
