@@ -496,7 +496,7 @@ def run_ours(args) -> dict:
     clocks = sampler.window(*windows["mixed"][1])
     launch_bytes = work["attn_bytes"] + work["append_bytes"]
     tensor_bound = work["prefill_flops"] / (NOMINAL_BF16_TFLOPS * 1e12) > launch_bytes / (NOMINAL_HBM_GBS * 1e9)
-    kernel = f"sw_mixed_attn_kernel<{batch.shape.head_dim}, 1> (one prefill chunk; KV append fused in)"
+    kernel = f"sw_mixed_attn_kernel<{batch.shape.head_dim}, kOneChunk> (one prefill chunk; KV append fused in)"
     key = (args.workload, args.decodes, args.chunk, args.prefix)
     if tensor_bound:
         tf = work["prefill_flops"] / (us * 1e-6) / 1e12

@@ -222,7 +222,7 @@ constexpr int kMinLateCtas = 24;   // fewer late CTAs than this: their delay is 
 // contexts of 256-2048 beside 300 tokens 26.4 -> 31.8 us, 40 of 256-8192 of 16/4/64 beside 700 42.2 -> 40.1.)
 constexpr int kLineMaxStages = 1 << 23;   // 64 GB at head size 128; positions times CTAs fit 32 bits
 constexpr int kLineMaxDecode = 432;
-constexpr int kLineGroups = kWarps + 1, kLineWords = 4, kLineTable = 88;   // (where the chunk table was: the entries are done)
+constexpr int kLineGroups = kWarps + 1, kLineWords = 4, kLineTable = 88;   // (where launches with chunks keep their table)
 // Up to 432 requests, whose lengths, offsets, first stages and last pages take 1732 bytes of the four arrays of the plan; what is left
 // of each holds three partial results (O of the group, m, l) of at most 2 KB + 64 bytes.
 constexpr int kStashBytes = 2048 + 2 * kMaxGroup * 4;
@@ -831,7 +831,7 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
         }
         int page = __shfl_sync(0xffffffffu, ids, issued & 31);
         if (page < 0 || (int64_t)page >= p.num_pages) {
-            // a bad id never reaches the copy engine: the problem is reported and page 0 is fetched in its place, so
+// The line of stages (see use_line): CTA `cta` of plan.line_ctas streams its stretch and merges (CTAs beyond those have none).
             // the barrier still receives the bytes it expects
             if (lane == 0) report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAttnPage, u.q_row);
             page = 0;
