@@ -831,7 +831,7 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
         }
         int page = __shfl_sync(0xffffffffu, ids, issued & 31);
         if (page < 0 || (int64_t)page >= p.num_pages) {
-// The line of stages (see use_line): CTA `cta` of plan.line_ctas streams its stretch and merges (CTAs beyond those have none).
+            // a bad id never reaches the copy engine: the problem is reported and page 0 is fetched in its place, so
             // the barrier still receives the bytes it expects
             if (lane == 0) report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAttnPage, u.q_row);
             page = 0;
