@@ -37,6 +37,7 @@ __device__ __forceinline__ void report(int32_t* ctrl, int code, int site, int in
 // (P is AppendParams or MixedParams: the fields have the same names; every index into the chunk arrays is a
 // compile-time constant so that the kernel parameters stay in constant memory.)
 constexpr int kAppendBatch = 4;   // in the fused launch, with 11 warps an SM; the stand-alone kernel has 32 of one part each
+// (six: 2048 rows without a prefix 51.6 -> 50.7 us, but 64 contexts beside 512 tokens 62.8 -> 64.8)
 template <bool kMulti, int kBatch, class P>
 __device__ __forceinline__ void append_rows(const P& p, int head_dim, int first, int stride) {
     const int lane = threadIdx.x & 31;
