@@ -1110,8 +1110,6 @@ __device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const Mixed
         stage_result<D>(keep, g, st);
         if (alone) {
             if (listed) write_rows<D>(p, keep, p.C + i, kvh, st);
-            fence_proxy_async_smem();  // the buffer was written with plain stores and is refilled by the copy engine
-            __syncwarp();
         } else {
             if (lane < 4) {   // m and l of the group behind O
                 sts_f32(keep + (g * D + 2 * lane) * 4, st.m0);
@@ -1128,6 +1126,10 @@ __device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const Mixed
                 e[3] = cb - ca + 1;
             }
         }
+        // The pair's last page buffer was written with plain stores (the new row, zeroed rows of V, the result), wherever the result
+        // went, and is refilled by the copy engine.
+        fence_proxy_async_smem();
+        __syncwarp();
         if (issued < total) issue_next();
     }
     __syncthreads();

@@ -44,6 +44,42 @@ def test_largest_batch_of_the_line(oracle, n):
     run(oracle, (4, 1, 128), [int(x) for x in np.random.default_rng(n).integers(1, 90, n)], f"{n} requests")
 
 
+@pytest.mark.parametrize("fused", [True, False])
+@pytest.mark.parametrize("heads,lens", [
+    ((8, 2, 128), [16 * 13 - 9] * 300),                                        # four or five pages a warp: nearly every pair is cut
+    ((32, 8, 128), [int(x) for x in np.random.default_rng(6).integers(150, 330, 90)]),
+    ((8, 2, 64), [16 * 17 + 1, 16 * 11 - 1] * 130),
+])
+def test_page_buffers_are_refilled_behind_pairs_that_end_in_a_warp(oracle, heads, lens, fused):
+    """A pair that an earlier warp began ends in a partly filled page whose buffer is written with plain stores (the new row, zeroed rows)
+    and then refilled with the next pair's page: no such store may land on that page.  The unwritten slots of the pool hold NaNs."""
+    rng = np.random.default_rng(79)
+    shape = W.AttnShape(*heads)
+    batch = W.make_batch(shape, sum(-(-x // 16) for x in lens) + 3, lens, 0, 0, rng)
+    t = W.host_tensors(batch, rng)
+    pool = t["pool"].reshape(batch.num_pages, 2, shape.num_kv_heads, 16, shape.head_dim)
+    for i, x in enumerate(lens):
+        page = batch.decode_pages[batch.decode_page_indptr[i + 1] - 1]
+        pool[page, :, :, (x - 1) % 16 + 1:] = 0x7FC0
+    after = t["pool"].copy()
+    assert oracle.kv_append(after, batch, t["k_new"], t["v_new"]) == 0
+    ref, ref_lse, _ = oracle.mixed_attention(after, batch, t["q"])
+    r = G.Runner(batch, t)
+    first = None
+    for _ in range(10):
+        if fused:
+            r.iterate()
+        else:
+            r.append()
+            r.attend()
+        out, lse = r.results()
+        if first is None:
+            assert r.status() == (0, 0)
+            G.compare(out.reshape(-1, shape.head_dim), lse.reshape(-1), ref, ref_lse, f"{heads}")
+            first = out, lse
+        assert np.array_equal(out, first[0]) and np.array_equal(lse, first[1])
+
+
 def test_long_stretches(oracle):
     """Two pairs of 100000 and 13000 pages: 64 pages a warp and more."""
     batch = W.make_batch(W.AttnShape(1, 1, 64), 113003, [16 * 100000 - 3, 16 * 13000 - 7], 0, 0, np.random.default_rng(3))
