@@ -82,6 +82,7 @@ struct sw_ctx {
     int device = 0;
     int num_sms = 0;
     float stage_us = 0.f, step_us = 0.f;  // planning estimates from the device's clocks (sw::device_timing)
+    long long line_wait_cycles = sw::kLineWaitCycles;
     bool grid_resident = false;  // the persistent grid fits the device at once (needed by the fused append + attention launch)
     int max_chunk = 0, max_decode = 0;
     int64_t max_pages = 0;
@@ -410,6 +411,7 @@ sw_status run_mixed(sw_ctx* ctx, void* kv_pool, const sw_batch* batch, const voi
     p.part_o = reinterpret_cast<float*>(ctx->ws + ctx->w.part_o);
     p.max_items = ctx->w.max_items;
     p.target_items = sw::kTargetItems;
+    p.line_wait_cycles = ctx->line_wait_cycles;
     p.pf_ml = reinterpret_cast<float*>(ctx->ws + ctx->w.pf_ml);
     p.pf_o = reinterpret_cast<float*>(ctx->ws + ctx->w.pf_o);
     p.pf_slots = ctx->w.pf_slots;
@@ -674,6 +676,12 @@ int sw_host_part_rows_of(const sw_layout* layout, int32_t num_sms, const sw_batc
     Chunks ch;
     if (!layout || !hb || !layout_supported(*layout) || chunks_of(hb, "sw_host_part_rows_of", &ch) != SW_OK) return -1;
     return host_part_rows(*layout, num_sms, hb, ch);
+}
+
+int sw_ctx_set_line_wait(sw_ctx* ctx, int64_t cycles) {
+    if (!ctx || cycles < 0 || cycles > sw::kLineWaitCycles) return SW_ERR_INVALID_ARG;
+    ctx->line_wait_cycles = cycles;
+    return SW_OK;
 }
 
 namespace {

@@ -21,6 +21,8 @@ constexpr int kPfRoundSlots = 3 * kMaxCtas;  // partial results of chunk-prefill
 constexpr int kMaxChunks = 8;           // prefill chunks (of different prompts) in one iteration
 constexpr int kMaxChunk = 65536;        // chunk tokens per iteration (256-row groups are planned in shared memory)
 
+constexpr long long kLineWaitCycles = 2000000000LL;   // limit of a wait in the line of decode stages (about a second)
+
 // Control words at the start of the workspace.
 // kCtrArrived counts the CTAs that have ended, modulo two grids; launches use the two counter sets at kCtrSets in turn.
 enum CtrlWord { kCtrArrived = 0, kCtrStatus = 2, kCtrDetail = 3, kCtrSets = 16, kCtrWords = 64 };
@@ -72,6 +74,7 @@ struct MixedParams {
     float* part_o;      // [max_items][group * D]
     int max_items;      // partial-result slots available
     int target_items;   // split-KV units aimed at (<= max_items - n*Hkv)
+    long long line_wait_cycles;   // kLineWaitCycles; 0: what has not arrived at the first look has expired
     // scratch of prefill items finished by several CTAs
     float* pf_ml;        // [pf_slots][2][2][128]
     float* pf_o;         // [pf_slots][2][D / 4][128][4]
@@ -166,3 +169,6 @@ size_t mixed_attn_smem_bytes(int head_dim);
 // Not part of the ABI: the chunk rows that sw_mixed_iteration_host would give a part of this host batch on a device of num_sms SMs (0: the
 // iteration is run whole; -1: no valid batch).  Host arithmetic only; the tests look at it.
 extern "C" int sw_host_part_rows_of(const sw_layout* layout, int32_t num_sms, const sw_batch* h_batch);
+// Likewise: the limit of the waits in this context's decode-only launches (kLineWaitCycles otherwise).  With 0 they expire, and the tests
+// see what such a launch leaves behind.
+extern "C" int sw_ctx_set_line_wait(sw_ctx* ctx, int64_t cycles);

@@ -1015,7 +1015,8 @@ __device__ __forceinline__ void list_last_pages(const MixedParams& p, const Plan
 // that begins and ends in the warp is finished by it.  Any other leaves a partial result in shared memory, in the warp's first page
 // buffer if it is the last thing the warp does and in the plan's unused space otherwise; when all warps are done, warps merge the
 // pairs row by row.  A pair that goes on beyond the CTA is published (slots of a pair's CTAs follow one another) and merged by the CTA
-// that publishes last, so nobody waits for another CTA.
+// that publishes last, so nobody waits for another CTA.  If a wait expires, the warp ends (its own copies awaited) and the CTA merges and
+// publishes nothing: the launch is reported, and the pairs that it did not finish keep what their rows held before.
 template <int D>
 __device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const MixedParams& p, const Plan& plan, const int* prefix, int* scratch,
                                          unsigned* sets, uint32_t smem, int cta) {
@@ -1071,9 +1072,12 @@ __device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const Mixed
     };
     for (int k = 0; k < kStages && k < total; ++k) issue_next();
     if (p.append_last) list_last_pages<D>(p, plan, smem, sets);   // after the first copies are on their way
-    bool ok = true;
+    bool expired = false;
+    auto wait = [&](uint32_t bar, uint32_t parity) {
+        return mbar_test_wait(bar, parity) || (p.line_wait_cycles > 0 && mbar_wait(bar, parity, p.line_wait_cycles));
+    };
 #pragma unroll 1
-    for (int x = x0; x < x1 && ok;) {
+    for (int x = x0; x < x1;) {
         int kvh, i;
         const int page = locate(x, kvh, i), pages = prefix[i + 1] - prefix[i];
         const int a = x - page, b = a + pages, end = min(b, x1);   // the pair's stretch of the line; where the warp's part of it ends
@@ -1091,19 +1095,22 @@ __device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const Mixed
             const bool patched = p.append_last && valid <= kPageSize;
             uint4 row;
             if (patched) row = load_new_row<D>(p, i, kvh);
-            if (!mbar_wait(ring.bar + stage * 8, parity) || (patched && !mbar_wait(smem + Geo<D>::kLastBarOffset, 0))) {
-                report(p.ctrl, SW_ERR_DEVICE_TIMEOUT, kSiteWait, p.C + i);
-                ok = false;
+            expired = !wait(ring.bar + stage * 8, parity) || (patched && !wait(smem + Geo<D>::kLastBarOffset, 0));
+            if (__any_sync(0xffffffffu, expired)) {
+                expired = true;
                 break;
             }
-            if (patched) {
-                __syncwarp();
-                patch_page<D>(p, smem, sK, i, kvh, valid, row);
-            }
+            if (patched) patch_page<D>(p, smem, sK, i, kvh, valid, row);
             attend_page<D>(p, sK, valid, qb, st);
             ring.it += 1;
             __syncwarp();  // every lane is done reading this stage before it is refilled
             if (x + 1 < end && issued < total) issue_next();
+        }
+        if (expired) {
+            report(p.ctrl, SW_ERR_DEVICE_TIMEOUT, kSiteWait, p.C + i);
+#pragma unroll 1
+            for (; ring.it < (uint32_t)issued; ++ring.it) mbar_wait(ring.bar + ring.it % kStages * 8, (ring.it / kStages) & 1);
+            break;
         }
         if (!listed) st.clear();   // nothing of this request counts
         const uint32_t keep = alone ? sK : (end == x1 ? ring.buf : stash_of(warp));
@@ -1132,7 +1139,7 @@ __device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const Mixed
         __syncwarp();
         if (issued < total) issue_next();
     }
-    __syncthreads();
+    if (__syncthreads_or(expired)) return;
     const int lg = 31 - __clz(g), tasks = *reinterpret_cast<volatile int*>(table + kLineGroups * kLineWords) << lg;
     bool beyond = false;   // some pair goes on in another CTA
 #pragma unroll 1

@@ -155,6 +155,7 @@ extern "C" sw_status sw_decode_attn_static(const sw_layout* layout, int device, 
     p.part_o = reinterpret_cast<float*>(st->scratch + kOffPartO);
     p.max_items = kStaticMaxItems;
     p.target_items = kStaticTargetItems;
+    p.line_wait_cycles = sw::kLineWaitCycles;
     SW_CUDA(sw::launch_mixed_attn(l.head_dim, kv_maps, kv_maps.half, kv_maps.half, p, st->num_sms, s));
     return SW_OK;
 }

@@ -1,5 +1,7 @@
 """Decode-only launches whose stages are shared out in a line: stretches shorter than a CTA's warps, pairs on one warp, on several and on
 several CTAs, the largest batch of the rule and the first one beyond it, CTAs that come late, page lists that are too short."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -78,6 +80,39 @@ def test_page_buffers_are_refilled_behind_pairs_that_end_in_a_warp(oracle, heads
             G.compare(out.reshape(-1, shape.head_dim), lse.reshape(-1), ref, ref_lse, f"{heads}")
             first = out, lse
         assert np.array_equal(out, first[0]) and np.array_equal(lse, first[1])
+
+
+@pytest.mark.parametrize("fused", [True, False])
+@pytest.mark.parametrize("heads,lens", [((32, 8, 128), [2000] * 64), ((8, 2, 64), [30000, 500] * 12), ((4, 1, 128), [200000])])
+def test_expired_waits_leave_no_wrong_rows(oracle, heads, lens, fused):
+    """With a limit of zero most waits for a page expire.  The launch is reported, and every row of the output is right or untouched."""
+    rng = np.random.default_rng(80)
+    shape = W.AttnShape(*heads)
+    batch = W.make_batch(shape, sum(-(-x // 16) for x in lens) + 3, lens, 0, 0, rng)
+    t = W.host_tensors(batch, rng)
+    pool = t["pool"].copy()
+    assert oracle.kv_append(pool, batch, t["k_new"], t["v_new"]) == 0
+    ref, ref_lse, _ = oracle.mixed_attention(pool, batch, t["q"])
+    r = G.Runner(batch, t)
+    if not fused:
+        r.append()
+    launch = r.iterate if fused else r.attend
+    assert r.B._lib.sw_ctx_set_line_wait(r.ctx.handle, ctypes.c_int64(0)) == r.B.SW_OK
+    for _ in range(3):
+        r.out.zero_()
+        r.lse.zero_()
+        launch()
+        assert r.status()[0] == r.B.SW_ERR_DEVICE_TIMEOUT
+        out, lse = (x.reshape(ref.shape[0], -1) for x in r.results())
+        done = (out != 0).any(1) | (lse[:, 0] != 0)
+        assert not done.all()
+        if done.any():
+            G.compare(out[done], lse[done, 0], ref[done], ref_lse[done], f"{heads}: {done.sum()} rows")
+    assert r.B._lib.sw_ctx_set_line_wait(r.ctx.handle, ctypes.c_int64(2_000_000_000)) == r.B.SW_OK
+    launch()                                # the tickets are re-armed
+    assert r.status() == (0, 0)
+    out, lse = r.results()
+    G.compare(out.reshape(-1, shape.head_dim), lse.reshape(-1), ref, ref_lse, f"{heads} afterwards")
 
 
 def test_long_stretches(oracle):
