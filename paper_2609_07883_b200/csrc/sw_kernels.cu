@@ -4,8 +4,9 @@
 //   sw_mixed_attn_kernel    ONE persistent launch per iteration (Sec. 4.1).  Optionally it first writes the new K/V
 //                           rows itself (the fused form of the append).  CTAs with chunk-prefill entries run them on
 //                           the tensor cores (sw_prefill.cuh).  Every CTA then plans the split-KV decode units from
-//                           the context lengths (without chunks: shares them out as a line, see use_line); a warp's first
-//                           unit is fixed by its index, further ones come from a shared counter; a unit streams its K/V pages with TMA into the warp's shared-memory ring
+//                           the context lengths (without chunks, where line_form allows it: shares the pages out as a
+//                           line instead, run_line); a warp's first unit is fixed by its index, further ones come from a
+//                           shared counter; a unit streams its K/V pages with TMA into the warp's shared-memory ring
 //                           and keeps an online softmax in registers; of the units of one (request, kv head) the one
 //                           that drew the last ticket merges the partial results or, where there are many, the last
 //                           ones one query-head row each.
@@ -221,23 +222,35 @@ constexpr int kMinLateCtas = 24;   // fewer late CTAs than this: their delay is 
 // 18.6 -> 16.0.  What is left: 4 us to the first copies, CTAs that end up to 15 % apart (the SMs' rates differ), 2-4 us of merges.
 // (Beside chunk-prefill entries units stay: shares fixed by an estimate of when the late CTAs come were slower as often as faster, 16
 // contexts of 256-2048 beside 300 tokens 26.4 -> 31.8 us, 40 of 256-8192 of 16/4/64 beside 700 42.2 -> 40.1.)
-constexpr int kLineMaxStages = 1 << 23;   // 64 GB at head size 128; positions times CTAs fit 32 bits
+constexpr int kLineMaxStages = 0x7fffff00;   // 16 TB at head size 128
 constexpr int kLineMaxDecode = 432;
 constexpr int kLineGroups = kWarps + 1, kLineWords = 4, kLineTable = 88;   // (where launches with chunks keep their table)
+static_assert((kLineTable + kLineGroups * kLineWords + 1) * 4 <= 768, "the table of the line lies in the CTA's scratch");
 // Up to 432 requests, whose lengths, offsets, first stages and last pages take 1732 bytes of the four arrays of the plan; what is left
 // of each holds three partial results (O of the group, m, l) of at most 2 KB + 64 bytes.
-constexpr int kStashBytes = 2048 + 2 * kMaxGroup * 4;
-inline bool line_form(const MixedParams& p, int head_dim) { return p.n <= kLineMaxDecode && p.group * head_dim <= 512; }   // on the host
-__device__ __forceinline__ bool use_line(const MixedParams& p, int total_pages) {
-    return total_pages > 0 && (int64_t)total_pages * p.Hkv <= kLineMaxStages && (int)gridDim.x + p.n * p.Hkv <= p.max_items;
+constexpr int kLineGroupElems = 512, kStashBytes = kLineGroupElems * 4 + 2 * kMaxGroup * 4, kStashesPerArray = 3, kPlanArrays = 4;
+constexpr int kLineArrayBytes = ((kLineMaxDecode + 1) * 4 + 15) / 16 * 16;
+static_assert(kPlanArrays * kStashesPerArray >= kWarps, "one partial result per warp");
+static_assert(kLineArrayBytes + 15 + kStashesPerArray * kStashBytes <= kMaxDecode * 4, "behind an array's first entries lie its partial results");
+static_assert(kLineGroupElems * 4 + 2 * kMaxGroup * 4 <= Geo<64>::kStageBytes, "a partial result fits a page buffer");
+static_assert(kMaxCtas <= kTargetItems, "the line has a slot for every CTA and every (request, KV head) pair");
+inline bool line_form(const MixedParams& p, int head_dim) {   // on the host
+    return p.n <= kLineMaxDecode && p.group * head_dim <= kLineGroupElems;
 }
+struct Line {
+    const int* len;     // shared-memory copies of the context lengths and page-list offsets
+    const int* indptr;
+    const int* prefix;  // stages before a request's, of one KV head
+    int stages;         // of one KV head
+    int total;          // of all KV heads
+    int ctas;           // that share the line, in steps of 2^shift stages
+    int coarse, shift;  // steps: 2^23 at most
+};
 struct Plan {
     const int* len;     // shared-memory copies of the context lengths and page-list offsets
     const int* indptr;
     bool two_sizes;     // large units handed out by index to the early CTAs, small ones pulled by the late CTAs only
     int total_items;    // units of all requests, times the KV heads
-    int line_ctas;      // CTAs that share the line of stages (0: units are drawn)
-    int head_stages;    // the line: stages of one KV head
 };
 
 // Block-wide exclusive scan of one value per thread (kThreads threads): a warp scan, one barrier, then every thread
@@ -308,14 +321,12 @@ struct LateJoin {
 // run them, so that no warp starts a second unit.  If the early warps are nearly done by the time the late ones arrive,
 // the plan is sized for the early warps alone; if the early CTAs are few, their head start is small or there are many
 // requests per warp, it falls back to units of one size pulled by everybody.
-template <int D, bool kLineForm>
 __device__ __forceinline__ Plan make_plan(const MixedParams& p, int* unit_prefix, int* len_s, int* indptr_s, int* scratch,
                                           LateJoin late, float pages_per_us) {
     Plan plan;
     plan.len = len_s;
     plan.indptr = indptr_s;
     plan.two_sizes = false;
-    plan.line_ctas = 0;
     const int per_thread = (p.n + kThreads - 1) / kThreads;
     const int beg = min(p.n, (int)threadIdx.x * per_thread);
     const int end = min(p.n, beg + per_thread);
@@ -332,33 +343,13 @@ __device__ __forceinline__ Plan make_plan(const MixedParams& p, int* unit_prefix
     }
     if (threadIdx.x == 0 && p.n > 0) indptr_s[p.n] = p.decode_page_indptr[p.n];
     int* ctr = scratch + 64;  // kPlanCounters counters zeroed in the kernel prologue, one per block sum
-    int total_pages, pages_before = 0;
-    bool any_long;
-    if constexpr (kLineForm) {
-        if (__any_sync(0xffffffffu, long_local) && (threadIdx.x & 31) == 0) atomicOr(ctr, 1);
-        pages_before = block_exclusive_scan(pages_local, scratch + 16, &total_pages);
-        any_long = *reinterpret_cast<volatile int*>(ctr++) != 0;
-    } else {
-        const int warp_pages = __reduce_add_sync(0xffffffffu, pages_local);
-        if ((threadIdx.x & 31) == 0 && warp_pages != 0) atomicAdd(ctr, warp_pages);
-        any_long = __syncthreads_or(long_local);   // (the barrier of the sum, see block_sum)
-        total_pages = *reinterpret_cast<volatile int*>(ctr++);
-    }
+    int pages_before = 0;
+    const int warp_pages = __reduce_add_sync(0xffffffffu, pages_local);
+    if ((threadIdx.x & 31) == 0 && warp_pages != 0) atomicAdd(ctr, warp_pages);
+    const bool any_long = __syncthreads_or(long_local);   // (the barrier of the sum, see block_sum)
+    const int total_pages = *reinterpret_cast<volatile int*>(ctr++);
 
     const int G = (int)gridDim.x;
-    if (kLineForm && use_line(p, total_pages)) {
-        for (int i = beg, at = pages_before; i < end; ++i) {
-            unit_prefix[i] = at;
-            at += len_s[i] > 0 ? (len_s[i] + kPageSize - 1) / kPageSize : 0;
-        }
-        if (threadIdx.x == 0) unit_prefix[p.n] = total_pages;
-        if (threadIdx.x == 32) scratch[kLineTable + kLineGroups * kLineWords] = 0;
-        plan.head_stages = total_pages;
-        plan.total_items = total_pages * p.Hkv;
-        plan.line_ctas = max(1, min(G, plan.total_items / kWarps));
-        __syncthreads();
-        return plan;
-    }
     constexpr int kMinPages = kMinSplitTokens / kPageSize;
     int split_a = 0, split_b = 0;  // pages per unit of the first requests / of the rest
     int a_pages = 0x7fffffff;      // requests whose pages start below this (per head) are cut with split_a
@@ -433,6 +424,48 @@ __device__ __forceinline__ Plan make_plan(const MixedParams& p, int* unit_prefix
     __syncthreads();
     plan.total_items = total_units * p.Hkv;
     return plan;
+}
+
+// The line of a decode-only launch.  A request whose page list ends before its context has no stages in it, and no output.
+__device__ __forceinline__ Line make_line(const MixedParams& p, int* prefix, int* len_s, int* indptr_s, int* scratch) {
+    const int per_thread = (p.n + kThreads - 1) / kThreads;
+    const int first = min(p.n, (int)threadIdx.x * per_thread), last = min(p.n, first + per_thread);
+    auto stages_of = [&](int len, int listed) {
+        const int pages = len > 0 ? (len - 1) / kPageSize + 1 : 0;
+        return pages <= listed ? pages : 0;
+    };
+    int here = 0;
+    for (int i = first; i < last; ++i) {
+        const int len = p.decode_kv_len[i], at = p.decode_page_indptr[i], listed = p.decode_page_indptr[i + 1] - at;
+        len_s[i] = len;
+        indptr_s[i] = at;
+        prefix[i] = stages_of(len, listed);
+        here += prefix[i];
+        if (i == p.n - 1) indptr_s[p.n] = at + listed;
+        if (len > 0 && prefix[i] == 0 && blockIdx.x == 0) report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAttnLen, p.C + i);
+    }
+    Line line;
+    line.len = len_s;
+    line.indptr = indptr_s;
+    line.prefix = prefix;
+    int before = block_exclusive_scan(here, scratch + 16, &line.stages);
+    for (int i = first; i < last; ++i) {
+        const int stages = prefix[i];
+        prefix[i] = before;
+        before += stages;
+    }
+    if (line.stages < 0 || (int64_t)line.stages * p.Hkv > kLineMaxStages) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) report(p.ctrl, SW_ERR_WORKSPACE, kSiteScratch, line.stages);
+        line.stages = 0;
+    }
+    if (threadIdx.x == 0) prefix[p.n] = line.stages;
+    if (threadIdx.x == 32) scratch[kLineTable + kLineGroups * kLineWords] = 0;
+    line.total = line.stages * p.Hkv;
+    line.ctas = max(1, min((int)gridDim.x, line.total / kWarps));
+    line.shift = max(0, 9 - __clz(line.total));
+    line.coarse = ((line.total - 1) >> line.shift) + 1;
+    __syncthreads();
+    return line;
 }
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -986,14 +1019,14 @@ __device__ bool run_unit(const CUtensorMap* kvp_map, const MixedParams& p, const
 
 // The requests' last pages, which fused decode-only launches write, by id; whole CTA.  Only warps with a request wait for the load.
 template <int D>
-__device__ __forceinline__ void list_last_pages(const MixedParams& p, const Plan& plan, uint32_t smem, unsigned* sets) {
+__device__ __forceinline__ void list_last_pages(const MixedParams& p, const int* lens, const int* indptr, uint32_t smem, unsigned* sets) {
     for (int i = threadIdx.x; i < p.n; i += kThreads) {
-        const int len = plan.len[i], pi = (len - 1) / kPageSize;
+        const int len = lens[i], pi = (len - 1) / kPageSize;
         int id = -1;
-        if (len < 1 || pi >= p.decode_page_indptr[i + 1] - plan.indptr[i]) {
+        if (len < 1 || pi >= indptr[i + 1] - indptr[i]) {
             if (blockIdx.x == 0) report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAppendLen, i);
         } else {
-            id = p.decode_pages[plan.indptr[i] + pi];
+            id = p.decode_pages[indptr[i] + pi];
             if (id < 0 || (int64_t)id >= p.num_pages) {
                 if (blockIdx.x == 0) report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAppendPage, i);
                 id = -1;
@@ -1008,32 +1041,38 @@ __device__ __forceinline__ void list_last_pages(const MixedParams& p, const Plan
     if ((threadIdx.x & 31) == 0) mbar_arrive(smem + Geo<D>::kLastBarOffset);
 }
 
-// The line of stages (see use_line): CTA `cta` of plan.line_ctas streams its stretch and merges.
+// The line of stages (see line_form): CTA `cta` of line.ctas streams its stretch and merges.
 //
-// Positions: x / head_stages is the KV head, x % head_stages the page in the order of the requests.  CTA c has [c T / C, (c + 1) T / C) of
-// the T stages, its warp w the same share of those; page copies run ahead of the (request, KV head) pair that is being worked on.  A pair
+// Position x of the line is page x % stages, in the order of the requests, of KV head x / stages.  CTA c has [c T / C, (c + 1) T / C) of the T
+// stages, its warp w the same share of those.  (Lines of 2^23 stages and more are shared out in steps of 2^shift stages, so that
+// positions times CTAs fit 32 bits.  This arithmetic stands in a chain of instructions that are executed once, and fetched for it: with
+// shares that need no product, and 64-bit divisions, one 8192-token context took 16.6 us instead of 15.1.)  Page copies run ahead of the (request, KV head) pair that is being worked on.  A pair
 // that begins and ends in the warp is finished by it.  Any other leaves a partial result in shared memory, in the warp's first page
 // buffer if it is the last thing the warp does and in the plan's unused space otherwise; when all warps are done, warps merge the
 // pairs row by row.  A pair that goes on beyond the CTA is published (slots of a pair's CTAs follow one another) and merged by the CTA
 // that publishes last, so nobody waits for another CTA.  If a wait expires, the warp ends (its own copies awaited) and the CTA merges and
 // publishes nothing: the launch is reported, and the pairs that it did not finish keep what their rows held before.
 template <int D>
-__device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const MixedParams& p, const Plan& plan, const int* prefix, int* scratch,
+__device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const MixedParams& p, const Line& line, int* scratch,
                                          unsigned* sets, uint32_t smem, int cta) {
     constexpr int kStages = Geo<D>::kStages, V = D / 32;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int T = plan.total_items, C = plan.line_ctas, g = p.group;   // (T C < 2^31)
-    const int X0 = cta * T / C, X1 = cta < C ? (cta + 1) * T / C : X0, L = X1 - X0;
-    auto warp_begin = [&](int w) { return X0 + w * L / kWarps; };
+    const int g = p.group, C = line.ctas;
+    auto cta_begin = [&](int c) { return min(line.total, c * line.coarse / C << line.shift); };
+    auto cta_of = [&](int x) { return (((x >> line.shift) + 1) * C - 1) / line.coarse; };
+    const int X0 = cta_begin(min(cta, C)), X1 = cta_begin(min(cta + 1, C));
+    const unsigned L = X1 - X0;
+    auto warp_begin = [&](int w) { return X0 + (int)(w * L / kWarps); };
+    const int* prefix = line.prefix;
     auto ring_of = [&](int w) { return smem + w * kStages * Geo<D>::kStageBytes; };
     auto stash_of = [&](int w) {   // array w / 3 of the plan, behind its first kLineMaxDecode + 1 words
         const int at = w < 6 ? (w < 3 ? Geo<D>::kPlanOffset : Geo<D>::kLenOffset) : (w < 9 ? Geo<D>::kIndptrOffset : Geo<D>::kLastOffset);
-        return smem + ((at + (kLineMaxDecode + 1) * 4 + 15) & ~15) + (w % 3) * kStashBytes;
+        return smem + ((at + 15) & ~15) + kLineArrayBytes + (w % kStashesPerArray) * kStashBytes;
     };
     // (head, request, page) of a position
     auto locate = [&](int x, int& kvh, int& i) {
-        kvh = x / plan.head_stages;
-        const int rem = x - kvh * plan.head_stages;
+        kvh = x / line.stages;
+        const int rem = x - kvh * line.stages;
         int lo = 0, hi = p.n;  // largest i with prefix[i] <= rem
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
@@ -1055,15 +1094,11 @@ __device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const Mixed
             id = 0;
             if (x < x1) {
                 int i;
-                const int page = locate(x, head, i), beg = plan.indptr[i];
-                if (prefix[i + 1] - prefix[i] <= plan.indptr[i + 1] - beg) {
-                    id = p.decode_pages[beg + page];
-                    if (id < 0 || (int64_t)id >= p.num_pages) {   // never reaches the copy engine
-                        report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAttnPage, p.C + i);
-                        id = 0;
-                    }
-                } else {
-                    report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAttnLen, p.C + i);
+                const int page = locate(x, head, i);
+                id = p.decode_pages[line.indptr[i] + page];
+                if (id < 0 || (int64_t)id >= p.num_pages) {   // never reaches the copy engine
+                    report(p.ctrl, SW_ERR_OUT_OF_RANGE, kSiteAttnPage, p.C + i);
+                    id = 0;
                 }
             }
         }
@@ -1071,7 +1106,7 @@ __device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const Mixed
         ++issued;
     };
     for (int k = 0; k < kStages && k < total; ++k) issue_next();
-    if (p.append_last) list_last_pages<D>(p, plan, smem, sets);   // after the first copies are on their way
+    if (p.append_last) list_last_pages<D>(p, line.len, line.indptr, smem, sets);   // after the first copies are on their way
     bool expired = false;
     auto wait = [&](uint32_t bar, uint32_t parity) {
         return mbar_test_wait(bar, parity) || (p.line_wait_cycles > 0 && mbar_wait(bar, parity, p.line_wait_cycles));
@@ -1081,13 +1116,13 @@ __device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const Mixed
         int kvh, i;
         const int page = locate(x, kvh, i), pages = prefix[i + 1] - prefix[i];
         const int a = x - page, b = a + pages, end = min(b, x1);   // the pair's stretch of the line; where the warp's part of it ends
-        const bool alone = a >= x0 && b <= x1, listed = pages <= plan.indptr[i + 1] - plan.indptr[i];
+        const bool alone = a >= x0 && b <= x1;
         uint32_t qb[D / 16][2];
         load_query<D>(p, p.C + i, kvh, qb);
         DecodeState<D> st;
         st.clear();
         uint32_t sK = 0;
-        int valid = plan.len[i] - page * kPageSize;   // keys from the page on
+        int valid = line.len[i] - page * kPageSize;   // keys from the page on
 #pragma unroll 1
         for (; x < end; ++x, valid -= kPageSize) {
             const uint32_t stage = ring.it % kStages, parity = (ring.it / kStages) & 1;
@@ -1112,11 +1147,10 @@ __device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const Mixed
             for (; ring.it < (uint32_t)issued; ++ring.it) mbar_wait(ring.bar + ring.it % kStages * 8, (ring.it / kStages) & 1);
             break;
         }
-        if (!listed) st.clear();   // nothing of this request counts
         const uint32_t keep = alone ? sK : (end == x1 ? ring.buf : stash_of(warp));
         stage_result<D>(keep, g, st);
         if (alone) {
-            if (listed) write_rows<D>(p, keep, p.C + i, kvh, st);
+            write_rows<D>(p, keep, p.C + i, kvh, st);
         } else {
             if (lane < 4) {   // m and l of the group behind O
                 sts_f32(keep + (g * D + 2 * lane) * 4, st.m0);
@@ -1125,7 +1159,7 @@ __device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const Mixed
                 sts_f32(keep + (g * D + kMaxGroup + 2 * lane + 1) * 4, st.l1);
             }
             if (lane == 0 && max(a, x0) == max(a, X0)) {   // the pair's first warp in this CTA
-                const int lb = min(b, X1), wb = ((lb - X0) * kWarps - 1) / L, ca = ((a + 1) * C - 1) / T, cb = (b * C - 1) / T;
+                const int lb = min(b, X1), wb = ((lb - X0) * kWarps - 1u) / L, ca = cta_of(a), cb = cta_of(b - 1);
                 int* e = table + atomicAdd(table + kLineGroups * kLineWords, 1) * kLineWords;
                 e[0] = i * p.Hkv + kvh;
                 e[1] = warp | wb << 8 | (lb == warp_begin(wb + 1) ? 1 << 16 : 0);
@@ -1146,7 +1180,6 @@ __device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const Mixed
     for (int t = lane; t < tasks; t += 32) beyond |= table[(t >> lg) * kLineWords + 3] > 1;
     beyond = __any_sync(0xffffffffu, beyond);
     auto finish_row = [&](int pair, int row, float m, float l, const float (&acc)[V]) {
-        if (l == 0.f) return;   // a request whose page list is too short
         const int i = pair / p.Hkv, kvh = pair - i * p.Hkv;
         const float inv = 1.f / l;
         const int64_t out_row = (int64_t)(p.C + i) * p.Hq + kvh * g + row;
@@ -1405,16 +1438,20 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
         return;
     }
 
-    const Plan plan = make_plan<D, kForm == kLine>(p, unit_prefix, reinterpret_cast<int*>(smem + Geo<D>::kLenOffset),
-                                reinterpret_cast<int*>(smem + Geo<D>::kIndptrOffset), scratch, late,
-                                p.stages_per_us);
+    int* lens = reinterpret_cast<int*>(smem + Geo<D>::kLenOffset);
+    int* indptr = reinterpret_cast<int*>(smem + Geo<D>::kIndptrOffset);
+    if constexpr (kForm == kLine) {
+        const Line line = make_line(p, unit_prefix, lens, indptr, scratch);
+        run_line<D>(&kvp_map, p, line, scratch, sets, base, (int)blockIdx.x);
+        if (threadIdx.x == 0) atomicInc(reinterpret_cast<unsigned*>(&p.ctrl[kCtrArrived]), 2 * gridDim.x - 1);
+        return;
+    }
+    const Plan plan = make_plan(p, unit_prefix, lens, indptr, scratch, late, p.stages_per_us);
     if ((int)blockIdx.x == prefill_ctas && threadIdx.x == 0) atomicExch(p.ctrl + misc[kMiscSet] + kSetItems, plan.total_items + 1);
-    if (plan.line_ctas == 0 && plan.total_items > p.max_items) {
+    if (plan.total_items > p.max_items) {
         if (threadIdx.x == 0) report(p.ctrl, SW_ERR_WORKSPACE, kSiteScratch, plan.total_items);
-    } else if (kForm == kLine && plan.line_ctas > 0) {
-        if constexpr (kForm == kLine) run_line<D>(&kvp_map, p, plan, unit_prefix, scratch, sets, base, (int)blockIdx.x);
     } else {
-        if (!tensor_prefill && p.append_last) list_last_pages<D>(p, plan, base, sets);
+        if (!tensor_prefill && p.append_last) list_last_pages<D>(p, plan.len, plan.indptr, base, sets);
         int32_t* work = p.ctrl + lds_s32(base + Geo<D>::kSetOffset) + kSetWork;
         WarpRing<D> ring;
         ring.buf = base + warp * Geo<D>::kStages * Geo<D>::kStageBytes;

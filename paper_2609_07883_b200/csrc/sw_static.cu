@@ -28,6 +28,7 @@ constexpr size_t kOffPartMl = kOffTickets + (size_t)kStaticMaxDecode * kStaticMa
 constexpr size_t kOffPartO = kOffPartMl + (size_t)kStaticMaxItems * 2 * sw::kMaxGroup * 4;
 constexpr size_t kScratchBytes = kOffPartO + (size_t)kStaticMaxItems * kPartOBytesPerItem;
 static_assert(kOffPartMl % 256 == 0 && kOffPartO % 256 == 0, "regions stay 256-byte aligned");
+static_assert(sw::kMaxCtas <= kStaticTargetItems, "the line of decode stages has a slot for every CTA and every (request, KV head) pair");
 static_assert(kScratchBytes <= SW_STATIC_SCRATCH_BYTES, "the header states the size of the static scratch");
 
 // In host code this name is only a stand-in for the symbol; the device address comes from cudaGetSymbolAddress.

@@ -140,18 +140,49 @@ def test_beside_a_chunk(oracle, heads, lens, P, C, fused):
         G.run_device_case(oracle, batch, pairs, seed, f"{heads} {len(lens)} beside {P}+{C}", fused=fused)
 
 
-def test_requests_with_short_page_lists(oracle):
-    """Requests whose list ends before their context are reported and get no output; the others' are right."""
+@pytest.mark.parametrize("heads", [(8, 8, 64), (32, 8, 128)])
+def test_more_than_two_to_the_23_stages(oracle, heads):
+    """Page lists that name the same pages again and again: 1.1 million pages per KV head of a pool of 4000."""
+    rng = np.random.default_rng(81)
+    shape = W.AttnShape(*heads)
+    batch = W.make_batch(shape, 4000, [16 * 3000 - 5, 16 * 900 - 1, 33], 0, 0, rng)
+    times = [240, 430, 1]                                           # the list of request i is its pages, that often, last page last
+    lists = [np.tile(batch.decode_pages[a:b], k) for a, b, k in zip(batch.decode_page_indptr, batch.decode_page_indptr[1:], times)]
+    for x in lists[:2]:                                             # full pages in the middle: other ones than the last
+        x[:-1][x[:-1] == x[-1]] = x[0]
+    pages = np.array([len(x) for x in lists])
+    batch.decode_kv_len = (16 * pages - np.array([5, 1, 15])).astype(np.int32)
+    batch.decode_page_indptr = np.concatenate([[0], np.cumsum(pages)]).astype(np.int32)
+    batch.decode_pages = np.concatenate(lists).astype(np.int32)
+    assert pages.sum() * shape.num_kv_heads > 1 << 23
+    pairs = [(0, 0), (0, heads[0] - 1), (1, heads[0] // 2), (2, 1)]
+    G.run_device_case(oracle, batch, pairs, 82, f"{heads}, {pages.sum()} pages", fused=True)
+
+
+@pytest.mark.parametrize("fused", [True, False])
+def test_requests_with_short_page_lists(oracle, fused):
+    """Requests whose list ends before their context are reported and get no output (and no new row); the others' are right."""
     rng = np.random.default_rng(5)
     shape = W.AttnShape(8, 2, 128)
     lens = [700, 16 * 30, 4000, 33, 9]
     batch = W.make_batch(shape, sum(-(-x // 16) for x in lens) + 3, lens, 0, 0, rng)
     t = W.host_tensors(batch, rng)
-    ref, ref_lse, _ = oracle.mixed_attention(t["pool"], batch, t["q"])
+    pool = t["pool"].copy()
+    if fused:
+        assert oracle.kv_append(pool, batch, t["k_new"], t["v_new"]) == 0
+    ref, ref_lse, _ = oracle.mixed_attention(pool, batch, t["q"])
     batch.decode_kv_len = batch.decode_kv_len.copy()
     batch.decode_kv_len[[1, 3]] += 16
     r = G.Runner(batch, t)
-    r.attend()
+    if fused:
+        r.iterate()
+        per_page = t["pool"].size // batch.num_pages
+        for i in (1, 3):                                            # their pages hold what they held
+            ids = batch.decode_pages[batch.decode_page_indptr[i]:batch.decode_page_indptr[i + 1]]
+            pool.reshape(-1, per_page)[ids] = t["pool"].reshape(-1, per_page)[ids]
+        assert np.array_equal(G.torch_to_bits(r.pool).reshape(-1), pool.reshape(-1))
+    else:
+        r.attend()
     assert r.status()[0] == r.B.SW_ERR_OUT_OF_RANGE
     out, lse = r.results()
     good = [0, 2, 4]
