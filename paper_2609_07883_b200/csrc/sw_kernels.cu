@@ -223,6 +223,15 @@ constexpr int kMinLateCtas = 24;   // fewer late CTAs than this: their delay is 
 // (Beside chunk-prefill entries units stay: shares fixed by an estimate of when the late CTAs come were slower as often as faster, 16
 // contexts of 256-2048 beside 300 tokens 26.4 -> 31.8 us, 40 of 256-8192 of 16/4/64 beside 700 42.2 -> 40.1.)
 constexpr int kLineMaxStages = 0x7fffff00;   // 16 TB at head size 128
+// Where no pair is longer than a few stages, none is cut: the boundaries of warps and CTAs move to the nearest end of a pair, there are as many
+// CTAs as pairs, and nothing is merged.  `Few' is eight (what a unit has at least) and three times a warp's share of the line, up
+// to 24 (at head size 64, where a partial result is half as long, 20).  Cut -> whole, us of 32/8/128: 16 contexts of 16-64 tokens 11.1 -> 8.9, 100 of
+// 16-100 16.9 -> 12.3, 256 of 16-60 22.0 -> 17.9, 400 of 16-200 42.6 -> 38.4, 48 of 130-200 16.8 -> 14.5, 128 of 16-320 26.3 -> 22.5, 430 of
+// 100-380 78.7 -> 77.0; of 8/2/64 256 of 16-60 11.6 -> 9.0, 400 of 16-200 17.9 -> 15.7; but 430 of 100-380 21.9 -> 22.8, hence the
+// 20.  (Whole pairs beside cut ones gain nothing: 48 of 16-400 17.5 -> 18.3 and more.  32 of 81, which stretches of 12 pages cut at
+// ends of pairs only: 9.0 -> 9.7.)
+constexpr int kLineWhole = 8;
+__device__ __forceinline__ constexpr int line_whole_max(int head_dim) { return head_dim == 64 ? 20 : 24; }
 constexpr int kLineMaxDecode = 432;
 constexpr int kLineGroups = kWarps + 1, kLineWords = 4, kLineTable = 88;   // (where launches with chunks keep their table)
 static_assert((kLineTable + kLineGroups * kLineWords + 1) * 4 <= 768, "the table of the line lies in the CTA's scratch");
@@ -245,6 +254,7 @@ struct Line {
     int total;          // of all KV heads
     int ctas;           // that share the line, in steps of 2^shift stages
     int coarse, shift;  // steps: 2^23 at most
+    bool whole;         // no (request, KV head) pair is cut
 };
 struct Plan {
     const int* len;     // shared-memory copies of the context lengths and page-list offsets
@@ -427,6 +437,7 @@ __device__ __forceinline__ Plan make_plan(const MixedParams& p, int* unit_prefix
 }
 
 // The line of a decode-only launch.  A request whose page list ends before its context has no stages in it, and no output.
+template <int D>
 __device__ __forceinline__ Line make_line(const MixedParams& p, int* prefix, int* len_s, int* indptr_s, int* scratch) {
     const int per_thread = (p.n + kThreads - 1) / kThreads;
     const int first = min(p.n, (int)threadIdx.x * per_thread), last = min(p.n, first + per_thread);
@@ -449,22 +460,27 @@ __device__ __forceinline__ Line make_line(const MixedParams& p, int* prefix, int
     line.indptr = indptr_s;
     line.prefix = prefix;
     int before = block_exclusive_scan(here, scratch + 16, &line.stages);
-    for (int i = first; i < last; ++i) {
-        const int stages = prefix[i];
-        prefix[i] = before;
-        before += stages;
-    }
     if (line.stages < 0 || (int64_t)line.stages * p.Hkv > kLineMaxStages) {
         if (blockIdx.x == 0 && threadIdx.x == 0) report(p.ctrl, SW_ERR_WORKSPACE, kSiteScratch, line.stages);
         line.stages = 0;
     }
+    const int few = min(line_whole_max(D), kLineWhole + line.stages * p.Hkv / ((int)gridDim.x * 4));
+    bool longer = false;
+    for (int i = first; i < last; ++i) {
+        const int stages = prefix[i];
+        longer |= stages > few;
+        prefix[i] = before;
+        before += stages;
+    }
     if (threadIdx.x == 0) prefix[p.n] = line.stages;
     if (threadIdx.x == 32) scratch[kLineTable + kLineGroups * kLineWords] = 0;
     line.total = line.stages * p.Hkv;
-    line.ctas = max(1, min((int)gridDim.x, line.total / kWarps));
+    line.ctas = line.total / kWarps;
+    line.whole = __syncthreads_or(longer) == 0;
+    if (line.whole) line.ctas = max(line.ctas, p.n * p.Hkv);
+    line.ctas = max(1, min((int)gridDim.x, line.ctas));
     line.shift = max(0, 9 - __clz(line.total));
     line.coarse = ((line.total - 1) >> line.shift) + 1;
-    __syncthreads();
     return line;
 }
 
@@ -1086,7 +1102,17 @@ __device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const Mixed
     ring.buf = ring_of(warp);
     ring.bar = smem + Geo<D>::kBarOffset + warp * kStages * 8;
     ring.it = 0;
-    const int x0 = warp_begin(warp), x1 = warp_begin(warp + 1), total = x1 - x0;
+    int x0 = warp_begin(warp), x1 = warp_begin(warp + 1);
+    if (line.whole) {
+        int x = lane == 0 ? x0 : x1, kvh, i;
+        if (x < line.total) {
+            const int page = locate(x, kvh, i), pages = prefix[i + 1] - prefix[i];
+            x += 2 * page < pages ? -page : pages - page;
+        }
+        x0 = __shfl_sync(0xffffffffu, x, 0);
+        x1 = __shfl_sync(0xffffffffu, x, 1);
+    }
+    const int total = x1 - x0;
     int id = 0, head = 0, issued = 0;   // lane l: page id and KV head of stage x0 + 32 n + l
     auto issue_next = [&]() {
         if ((issued & 31) == 0) {
@@ -1441,7 +1467,7 @@ __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid
     int* lens = reinterpret_cast<int*>(smem + Geo<D>::kLenOffset);
     int* indptr = reinterpret_cast<int*>(smem + Geo<D>::kIndptrOffset);
     if constexpr (kForm == kLine) {
-        const Line line = make_line(p, unit_prefix, lens, indptr, scratch);
+        const Line line = make_line<D>(p, unit_prefix, lens, indptr, scratch);
         run_line<D>(&kvp_map, p, line, scratch, sets, base, (int)blockIdx.x);
         if (threadIdx.x == 0) atomicInc(reinterpret_cast<unsigned*>(&p.ctrl[kCtrArrived]), 2 * gridDim.x - 1);
         return;

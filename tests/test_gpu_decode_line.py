@@ -115,6 +115,19 @@ def test_expired_waits_leave_no_wrong_rows(oracle, heads, lens, fused):
     G.compare(out.reshape(-1, shape.head_dim), lse.reshape(-1), ref, ref_lse, f"{heads} afterwards")
 
 
+@pytest.mark.parametrize("fused", [True, False])
+@pytest.mark.parametrize("heads", [(32, 8, 128), (8, 2, 64), (8, 1, 64), (2, 2, 128)])
+def test_short_contexts_are_not_cut(oracle, heads, fused):
+    """Launches whose pairs all go whole to a warp, and the first ones with a pair that is too long for that."""
+    rng = np.random.default_rng(83)
+    for lens in ([1], [128], [129], [128] * 5, [129] + [16] * 4, [1] * 432, [16, 17] * 100,
+                 [int(x) for x in rng.integers(1, 129, 40)], [int(x) for x in rng.integers(1, 129, 432)],
+                 [int(x) for x in rng.integers(100, 20 * 16 + 1, 432)],                      # more stages: up to 20 and 24 are whole
+                 [24 * 16] * 432, [24 * 16] * 431 + [24 * 16 + 1], [20 * 16 + 1] * 432):
+        if fused or len(lens) * max(lens) < 30000:
+            run(oracle, heads, lens, f"{heads} {len(lens)} x {max(lens)}", fused)
+
+
 def test_long_stretches(oracle):
     """Two pairs of 100000 and 13000 pages: 64 pages a warp and more."""
     batch = W.make_batch(W.AttnShape(1, 1, 64), 113003, [16 * 100000 - 3, 16 * 13000 - 7], 0, 0, np.random.default_rng(3))
