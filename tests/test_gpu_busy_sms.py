@@ -1,5 +1,5 @@
 """Decode-only launches beside kernels that hold SMs for longer than the launch: the CTAs that find no SM start when others have ended,
-and no unit may wait for theirs.  Results against the oracle."""
+and no unit, and no stretch of the line, may wait for theirs.  Results against the oracle."""
 import numpy as np
 import pytest
 
@@ -13,11 +13,14 @@ HOLD_CYCLES = 300_000_000   # about 150 ms per SM held, thousands of times a lau
 
 @pytest.mark.parametrize("form", ["fused", "two", "static"])
 @pytest.mark.parametrize("heads,lens", [
-    ((32, 8, 128), [300, 1500, 64, 2048, 900, 700, 1700, 250]),    # every unit has a warp of its own: shared merges
-    ((16, 4, 64), [9000]),                                          # many units of one request
-    ((8, 2, 128), [60000, 30000]),                                  # more than 24 units each
-    ((32, 4, 128), [1000] * 30 + [40000, 100]),                     # groups of eight
-    ((4, 4, 64), [5000, 300]),                                      # one query head per KV head: the last ticket merges
+    ((32, 8, 128), [300, 1500, 64, 2048, 900, 700, 1700, 250]),    # the line
+    ((16, 4, 64), [9000]),
+    ((8, 2, 128), [60000, 30000]),
+    ((32, 4, 128), [1000] * 30 + [40000, 100]),                     # groups of eight: units, shared merges
+    ((4, 4, 64), [5000, 300]),                                      # the line
+    ((4, 4, 64), [20] * 432 + [5000]),                              # 433 requests: units, merged by the last ticket
+    ((8, 2, 128), [20] * 432 + [60000]),                            # more than 24 units of one request: shared merges
+    ((4, 2, 64), [20] * 432 + [900]),                               # every unit has a warp of its own: shared merges
 ])
 @pytest.mark.parametrize("held", [1, 3])
 def test_launches_end_although_sms_are_held(oracle, heads, lens, form, held):
@@ -25,6 +28,8 @@ def test_launches_end_although_sms_are_held(oracle, heads, lens, form, held):
 
     from paper_2609_07883_b200 import binding as B
 
+    if form == "static" and len(lens) > 256:
+        pytest.skip("more requests than the static variant takes")
     shape = W.AttnShape(*heads)
     rng = np.random.default_rng(31)
     batch = W.make_batch(shape, sum(-(-x // 16) for x in lens) + 5, lens, 0, 0, rng)

@@ -1,5 +1,5 @@
 """Decode-only launches whose stages are shared out in a line: stretches shorter than a CTA's warps, pairs on one warp, on several and on
-several CTAs, the largest batch of the rule and the first one beyond it, CTAs that come late, page lists that are too short."""
+several CTAs, the largest batch of the rule and the first one beyond it, page lists that are too short, waits that expire."""
 import ctypes
 
 import numpy as np
@@ -132,25 +132,6 @@ def test_long_stretches(oracle):
     """Two pairs of 100000 and 13000 pages: 64 pages a warp and more."""
     batch = W.make_batch(W.AttnShape(1, 1, 64), 113003, [16 * 100000 - 3, 16 * 13000 - 7], 0, 0, np.random.default_rng(3))
     G.run_device_case(oracle, batch, None, 72, "long stretches", fused=True)
-
-
-@pytest.mark.parametrize("heads,lens,P,C", [
-    ((32, 8, 128), [int(x) for x in np.linspace(256, 2048, 64)], 512, 512),     # half of the CTAs come late
-    ((32, 8, 128), [2500] * 40, 0, 300),                                        # fewer of them
-    ((32, 8, 128), [1, 16, 17, 300], 4000, 64),                                 # the early ones do it all
-    ((16, 4, 64), [int(x) for x in np.linspace(1, 4000, 50)], 37, 1000),
-    ((16, 8, 128), [900] * 30, 100, 260),
-])
-@pytest.mark.parametrize("fused", [True, False])
-def test_beside_a_chunk(oracle, heads, lens, P, C, fused):
-    """CTAs with chunk-prefill entries join the line late, with less of it."""
-    rng = np.random.default_rng(8)
-    shape = W.AttnShape(*heads)
-    batch = W.make_batch(shape, sum(-(-x // 16) for x in lens) + -(-(P + C) // 16) + 3, lens, P, C, rng)
-    rows = G.boundary_rows(C, heads[0] // heads[1])[::7] + list(range(C, C + len(lens)))
-    pairs = [(r, int(rng.integers(heads[0]))) for r in rows]
-    for seed in (73, 74):
-        G.run_device_case(oracle, batch, pairs, seed, f"{heads} {len(lens)} beside {P}+{C}", fused=fused)
 
 
 @pytest.mark.parametrize("heads", [(8, 8, 64), (32, 8, 128)])
