@@ -216,10 +216,13 @@ constexpr int kMinLateCtas = 24;   // fewer late CTAs than this: their delay is 
 // head and request by request, and every CTA gets an equal stretch of it, every warp an equal part of that.  So all warps stream the
 // same number of pages, and the results of a (request, KV head) pair that lies on several warps meet in shared memory: what goes
 // through global memory is one partial result per CTA that a pair reaches beyond, not one per warp.
-// Per launch of 32/8/128, units -> line: one context of 8192 tokens 18.0 -> 15.6 us (33.5 MB: 2.1 TB/s), of 32768 38.7 -> 30, 16
-// of 256-2048 22.1 -> 21.5, 64 of those 58.4 -> 55.3, 8 of 200-400 12.6 -> 11.3, four of 49152 (55 pages a warp, which were two rounds of
-// units) 140.7 -> 123.0 (6.5 TB/s), 128 log-normal ones 259 -> 252.4, 16 of 32k-131k 791 -> 774 (7.4 TB/s); 20 of 256-4096 tokens of 16/4/64
-// 18.6 -> 16.0.  What is left: 4 us to the first copies, CTAs that end up to 15 % apart (the SMs' rates differ), 2-4 us of merges.
+// Per launch of 32/8/128, units -> line: one context of 8192 tokens 18.1 -> 15.4 us (33.5 MB: 2.2 TB/s), of 32768 38.7 -> 29.7, 16
+// of 256-2048 22.1 -> 21.4, 64 of those 57.9 -> 54.4, 8 of 200-400 12.7 -> 11.0, 16 of 8192 90.5 -> 85.6, four of 49152 (55 pages a warp, which
+// were two rounds of units) 139.7 -> 123.0 (6.5 TB/s), 128 log-normal ones 256 -> 249.1 (6.8 TB/s), 16 of 32k-131k 775 -> 760
+// (7.1 TB/s); 20 of 256-4096 tokens of 16/4/64 18.7 -> 16.1.  What is left: 4 us to the first copies, CTAs that end up to 15 % apart (the
+// SMs' rates differ), 2-4 us of merges.
+// A CTA whose SM another kernel holds has its stretch for good; when it comes, the others have ended and it has their bandwidth: beside one
+// held SM the launches above take 1.13 to 1.4 times as long, with units they took 1.06 (16 of 32k-131k, four rounds) to 1.6.
 // (Beside chunk-prefill entries units stay: shares fixed by an estimate of when the late CTAs come were slower as often as faster, 16
 // contexts of 256-2048 beside 300 tokens 26.4 -> 31.8 us, 40 of 256-8192 of 16/4/64 beside 700 42.2 -> 40.1.)
 constexpr int kLineMaxStages = 0x7fffff00;   // 16 TB at head size 128
@@ -1335,9 +1338,9 @@ namespace sw {
 // ---------------------------------------------------------------------------------------------------------------
 // Forms of the kernel, chosen by the host: iterations with one prefill chunk, whose descriptors are then plain kernel parameters; with
 // several (descriptors looked up per work item); without any, where the decodes may be worked off as a line (line_form), and the others.
-// A form has only the code that it needs: with the line's code in the kernel of one chunk, the small mixed launch of 8/2/64 took 13.6 us and 64
-// contexts beside 512 tokens 63.7, with kernels of their own 12.8 and 62.3; 20 contexts
-// of 8/1/128, worked off as units, take 16.8 us in a kernel of their own and 21.6 beside the line's code (18.3 with all in one).
+// A form has only the code that it needs: with the line's code in the kernel of one chunk, the small mixed launch of 8/2/64 took 13.6 us
+// and 64 contexts beside 512 tokens 63.7, with kernels of their own 13.2 and 62.5; 20 contexts of 8/1/128, worked off as units, take
+// 16.8 us in a kernel of their own and 21.6 beside the line's code (18.3 with all in one).
 enum Form { kOneChunk, kSeveralChunks, kLine, kUnits };
 template <int D, Form kForm>
 __global__ void __launch_bounds__(kThreads, 1) sw_mixed_attn_kernel(const __grid_constant__ CUtensorMap kv_map,

@@ -676,8 +676,10 @@ __device__ __forceinline__ bool pf_mma(const MixedParams& p, const PfShared& sh,
 }
 
 // The same with kAhead: S of a tile is issued after the other tile's P V, a step earlier, PV0(j), QK1(j + 1), PV1(j), QK0(j + 2), ..., so that
-// it lies ready when the tile's softmax warps have written P.  (4111 + 1777 tokens of 16/4/64: 80.4 -> 76.8 us; entries of a few steps
-// lose 0.2: four contexts beside 256 + 128 of 8/2/64 12.9 -> 13.1.)
+// it lies ready when the tile's softmax warps have written P.  Against the kernel with the plain order: 4111 + 1777 tokens of 16/4/64 78.5 -> 76.7
+// us, 1000 + 512 of 8/2/64 21.9 -> 21.3, 256 + 128 12.3 -> 12.1; 4000 + 64, in pieces of one step, 23.4 -> 23.8.  (Entries of up to four steps
+// in the plain order, both in one kernel: 23.4, but 256 + 128 beside four contexts 13.1 -> 14.4.  One rolled loop over (step, tile)
+// with the same order: 76.7 -> 86.)
 template <int D>
 __device__ __forceinline__ bool pf_mma_ahead(const MixedParams& p, const PfShared& sh, const PfItem& it, PfMmaState& st) {
     const bool leader = elect_one();
