@@ -1065,12 +1065,14 @@ __device__ __forceinline__ void list_last_pages(const MixedParams& p, const int*
 // Position x of the line is page x % stages, in the order of the requests, of KV head x / stages.  CTA c has [c T / C, (c + 1) T / C) of the T
 // stages, its warp w the same share of those.  (Lines of 2^23 stages and more are shared out in steps of 2^shift stages, so that
 // positions times CTAs fit 32 bits.  This arithmetic stands in a chain of instructions that are executed once, and fetched for it: with
-// shares that need no product, and 64-bit divisions, one 8192-token context took 16.6 us instead of 15.1.)  Page copies run ahead of the (request, KV head) pair that is being worked on.  A pair
-// that begins and ends in the warp is finished by it.  Any other leaves a partial result in shared memory, in the warp's first page
-// buffer if it is the last thing the warp does and in the plan's unused space otherwise; when all warps are done, warps merge the
-// pairs row by row.  A pair that goes on beyond the CTA is published (slots of a pair's CTAs follow one another) and merged by the CTA
-// that publishes last, so nobody waits for another CTA.  If a wait expires, the warp ends (its own copies awaited) and the CTA merges and
-// publishes nothing: the launch is reported, and the pairs that it did not finish keep what their rows held before.
+// shares that need no product, and 64-bit divisions, one 8192-token context took 16.6 us instead of 15.1.)
+//
+// Page copies run ahead of the (request, KV head) pair that is being worked on.  A pair that begins and ends in the warp is finished
+// by it (all are where none is cut: line.whole).  Any other leaves a partial result in shared memory, in the warp's first page buffer if
+// it is the last thing the warp does and in the plan's unused space otherwise; when all warps are done, warps merge the pairs row by
+// row.  A pair that goes on beyond the CTA is published (slots of a pair's CTAs follow one another) and merged by the CTA that publishes
+// last, so nobody waits for another CTA.  If a wait expires, the warp ends (its own copies awaited) and the CTA merges and publishes
+// nothing: the launch is reported, and the pairs that it did not finish keep what their rows held before.
 template <int D>
 __device__ __forceinline__ void run_line(const CUtensorMap* kvp_map, const MixedParams& p, const Line& line, int* scratch,
                                          unsigned* sets, uint32_t smem, int cta) {

@@ -64,8 +64,9 @@ def test_long_request_beside_a_one_token_chunk(oracle, heads):
     ((8, 1, 64), [511 * 16]), ((8, 1, 64), [511 * 16 + 1]), ((8, 1, 64), [20, 512 * 16 + 5, 3]),   # 128 units of four pages and more
     ((4, 4, 64), [64]), ((4, 4, 64), [65]), ((4, 4, 64), [1, 1, 300]),
 ])
-def test_contexts_at_the_edges_of_the_small_batch_rule(oracle, heads, lens):
-    run(oracle, heads, lens, f"{heads} {len(lens)} x {max(lens)}")
+@pytest.mark.parametrize("chunk", [0, 1])
+def test_contexts_at_the_edges_of_the_small_batch_rule(oracle, heads, lens, chunk):
+    run(oracle, heads, lens, f"{heads} {len(lens)} x {max(lens)}, chunk {chunk}", chunk=chunk)
 
 
 @pytest.mark.parametrize("heads", [(8, 1, 64), (16, 2, 128), (8, 2, 64), (4, 2, 64), (8, 2, 128)])
